@@ -26,8 +26,8 @@ struct kgs_batch {
     bool own_stream = false;  // graphs cannot be captured on the legacy default stream
     int n = 0;
     std::vector<kgs_ctx *> ctx;
-    int precision = KGS_MIXED, tv = 2, bz = 32, line16 = 0, uniform = 0, nxo_max = 1;
-    int dev_src = 0;  // deviation-form FP32 source (kgs_opts.dev_source)
+    int precision = KGS_MIXED, bz = 32, nxo_max = 1;
+    SweepKind kind;   // the sweep kernel that serves every instance
     int max_iters = 1000;
     double tol = 1e-8;
     std::vector<char> active;
@@ -154,8 +154,7 @@ int enqueue_iteration(kgs_batch *b, int which)
     ba.skip_publish = b->skip_publish;
     // external records: inside a capture a plain record only orders streams
     KGS_CHECK(cudaEventRecordWithFlags(b->ev[0], st, cudaEventRecordExternal));
-    KGS_CHECK(launch_sweep_persistent(b->precision, b->tv, b->line16, b->uniform, ba, b->nxo_max, b->grid, st, 1,
-                                      b->dev_src));
+    KGS_CHECK(launch_sweep_persistent(b->kind, ba, b->nxo_max, b->grid, st));
     KGS_CHECK(cudaEventRecordWithFlags(b->ev[1], st, cudaEventRecordExternal));
     for (int i = 0; i < b->n; i++)
         if (b->active[i] &&
@@ -316,15 +315,12 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
     }
     b->n = n;
     b->precision = opts->precision;
-    b->dev_src = opts->dev_source ? 1 : 0;
     b->max_iters = opts->max_iters > 0 ? opts->max_iters : 1000;
     b->tol = opts->tol > 0.0 ? opts->tol : 1e-8;
     b->ctx.assign(n, nullptr);
     b->active.assign(n, 1);
     b->done.assign(n, 0);
     std::vector<int> flag_off(n);
-    b->line16 = 1;
-    b->uniform = 1;
     for (int i = 0; i < n; i++) {
         const kgs_problem &p = probs[i];
         kgs_opts o = *opts;
@@ -341,12 +337,13 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
         const HostTables &t = b->ctx[i]->t;
         b->tok_off.push_back(b->n_tok);
         b->n_tok += ctx_n_tokens(t);
-        b->tv = t.tv;
         b->bz = t.bz;
         b->nxo_max = std::max(b->nxo_max, t.nxo_max);
-        for (int q = 0; q < 8; q++)
-            if (t.oct_vcount[q] > 0 && t.oct_nx[q] != 16) b->line16 = 0;
-        if (!ctx_sweep_args(b->ctx[i]).uniform) b->uniform = 0;
+        const SweepKind k = t.kind();
+        if (i == 0) b->kind = k;
+        b->kind.line16 &= k.line16;
+        b->kind.uniform &= k.uniform;
+        b->kind.lines_max = std::max(b->kind.lines_max, k.lines_max);
         flag_off[i] = (int)b->n_flags;
         b->n_flags += (size_t)t.n_vg * t.nbx * t.nby * t.nbz;
     }
@@ -370,8 +367,8 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
     // persistent grid: as many CTAs as fit on the device at once
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess) return fail(KGS_ECUDA);
-    const size_t smem = sweep_smem_bytes(b->precision, b->tv, b->line16, b->nxo_max);
-    per_sm = sweep_persistent_occupancy(b->precision, b->tv, b->line16, b->uniform, smem, 1, b->dev_src);
+    const size_t smem = sweep_smem_bytes(b->kind, b->nxo_max);
+    per_sm = sweep_persistent_occupancy(b->kind, smem);
     if (per_sm < 1) return fail(KGS_ECUDA);
     b->grid = sms * per_sm;
     b->scratch_stride = sweep_scratch_bytes(b->bz);

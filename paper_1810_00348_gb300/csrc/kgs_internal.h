@@ -91,16 +91,21 @@ struct SweepArgs {
     int nx, ny, nz, bz;           // grid, block extent along z
     int nbx, nby, nbz;            // blocks per axis
     const int4 *work;             // per CTA row: octant, reflected block coords
-    const int *oct_vstart;        // [8] first sorted velocity of each octant
+    const int *oct_vstart;        // [8] first velocity slot of each octant
     const int *oct_vcount;        // [8] velocities per octant
     const int *oct_vgbase;        // [8] first global velocity-group index
-    int Nv;                       // all velocities
+    int Nv;                       // all velocity slots
     int vg_size;                  // velocities per CTA
     const void *vel;              // Real[Nv][4]: xi_x, xi_y, xi_z, w (octant-sorted)
     const void *velm;             // Real[Nv][8]: w_x, w_y w_z, the low parts of xi_x, xi_y, xi_z
                                   // (xi = hi + lo with hi = the value in vel), M_ref (FP32
                                   // path; 0 for FP64), the rounding error of M_ref (FP32
                                   // path), 1 unused
+    int pack;                     // packed velocity slots (HostTables::pack, FP32 with two velocities per thread)
+    int oct_line0[8];             // packed: first row of each octant in lines
+    const float *lines;           // packed: [lines][8] xi_y, xi_z, w_y w_z, low parts of xi_y, xi_z
+    const float *xnodes;          // packed: [8][xn_stride][4] xi_x, its low part, w_x
+    int xn_stride;
     int oct_nx[8];                // x nodes in each octant (length of its velocity x-lines)
     int nxo_max;                  // max over octants of oct_nx
     int any_solid;                // the problem has solid cells
@@ -181,18 +186,33 @@ __host__ __device__ inline double flag_value<double>(int f)
 __device__ __forceinline__ int flag_bits(float v) { return __float_as_int(v); }
 __device__ __forceinline__ int flag_bits(double v) { return (int)__double_as_longlong(v); }
 
-// order: upwind order of the sweep; order 2 exists for tv = 1 on uniform
-// grids only.  dev: the first-order FP32 sweep with the deviation-form source
-// (uniform grids).  Other combinations: 0 CTAs per SM / cudaErrorInvalidValue.
-cudaError_t launch_sweep_persistent(int precision, int tv, int line16, int uniform, const BatchSweepArgs &b, int nxo_max,
-                                    int grid, cudaStream_t s, int order = 1, int dev = 0);
+// Which sweep kernel serves a problem.
+struct SweepKind {
+    int precision = 0;            // 0 FP64, 1 FP32
+    int tv = 1;                   // velocities per thread (FP64, order 2: 1)
+    int line16 = 0;               // SweepArgs::line16
+    int uniform = 0;              // SweepArgs::uniform
+    int order = 1;                // upwind order; order 2 exists for tv = 1 on uniform grids only
+    int dev = 0;                  // first-order FP32 sweep with the deviation-form source (uniform grids)
+    int pack = 0;                 // SweepArgs::pack: the packed FP32 kernel (kgs_sweep_f2.cu)
+    int lines_max = 1;            // x-lines that a velocity group can touch, at most
+};
+// Persistent sweep.  Combinations that do not exist: 0 CTAs per SM /
+// cudaErrorInvalidValue.
+cudaError_t launch_sweep_persistent(const SweepKind &k, const BatchSweepArgs &b, int nxo_max, int grid,
+                                    cudaStream_t s);
 // Resident CTAs per SM of the persistent kernel (also sets its shared-memory limit).
-int sweep_persistent_occupancy(int precision, int tv, int line16, int uniform, size_t smem, int order = 1,
-                               int dev = 0);
+int sweep_persistent_occupancy(const SweepKind &k, size_t smem);
+size_t sweep_smem_bytes(const SweepKind &k, int nxo_max);
+// Sweep launch (one wavefront stage, order 1, no deviation-form source).
+cudaError_t launch_sweep(const SweepKind &k, const SweepArgs &a, int n_items, int max_vg, cudaStream_t s);
 
-// Sweep launch (one wavefront stage, order 1).  precision: 0 FP64, 1 FP32.
-cudaError_t launch_sweep(int precision, int tv, const SweepArgs &a, int n_items, int max_vg, cudaStream_t s);
-size_t sweep_smem_bytes(int precision, int tv, int line16, int nxo_max, int order = 1);
+// The packed FP32 kernels (k.pack), reached through the functions above.
+size_t sweep2_smem_bytes(const SweepKind &k, int nxo_max);
+int sweep2_occupancy(const SweepKind &k, size_t smem);
+cudaError_t launch_sweep2_persistent(const SweepKind &k, const BatchSweepArgs &b, int nxo_max, int grid,
+                                     cudaStream_t s);
+cudaError_t launch_sweep2_staged(const SweepKind &k, const SweepArgs &a, int n_items, int max_vg, cudaStream_t s);
 
 // Per-cell sums of the staged sweep's per-group partials (fixed group order).
 struct PartSumArgs {

@@ -62,6 +62,12 @@ struct Carve {
     }
 };
 
+constexpr int TOO_LARGE = 2;  // noalloc_iterate: the problem does not fit (no CUDA call was made)
+
+int noalloc_iterate(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid *vgrid, const kgs_gas *gas,
+                    const kgs_bc *bc, int precision, int wall_norm, int pack, double M0, const double *macros_in,
+                    const double *rho_w_in, double *macros_out, double *rho_w_out, double *residual, void *stream);
+
 }  // namespace
 
 extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid *vgrid,
@@ -73,18 +79,35 @@ extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, c
     if (macros_out == macros_in || rho_w_out == rho_w_in) return KGS_EINVAL;
     int rc = validate_problem(grid, solid, vgrid, gas, bc, precision, wall_norm, 0, 0);
     if (rc) return rc;
+    // packed velocity slots (HostTables::pack) need a little more scratch: a
+    // problem that fits only without them runs unpacked
+    rc = noalloc_iterate(grid, solid, vgrid, gas, bc, precision, wall_norm, 1, M0, macros_in, rho_w_in, macros_out,
+                         rho_w_out, residual, stream);
+    if (rc == TOO_LARGE)
+        rc = noalloc_iterate(grid, solid, vgrid, gas, bc, precision, wall_norm, 0, M0, macros_in, rho_w_in,
+                             macros_out, rho_w_out, residual, stream);
+    return rc == TOO_LARGE ? KGS_EINVAL : rc;
+}
+
+namespace {
+
+int noalloc_iterate(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid *vgrid, const kgs_gas *gas,
+                    const kgs_bc *bc, int precision, int wall_norm, int pack, double M0, const double *macros_in,
+                    const double *rho_w_in, double *macros_out, double *rho_w_out, double *residual, void *stream)
+{
+    int rc;
     HostTables t;
-    build_tables(t, grid, solid, vgrid, gas, bc, precision, wall_norm, 0, 0);
+    build_tables(t, grid, solid, vgrid, gas, bc, precision, wall_norm, 0, 0, 0, 0, 1, 0, pack);
     const size_t n = t.ncell, rsz = t.real_bytes();
     const int n_red = (int)((n + 255) / 256);
 
     Carve cv;
     const size_t o_coef = cv.take(n * NCOEF * rsz);
     const size_t o_vel = cv.take(t.vel64.size() * rsz);
-    const size_t o_velm = cv.take((size_t)t.Nv * 8 * rsz);
+    const size_t o_velm = cv.take((size_t)t.Nvs * 8 * rsz);
     const size_t o_mt = cv.take(t.mt.size() * rsz);
-    const size_t fx_bytes = (size_t)t.nz * t.ny * t.Nv * rsz, fy_bytes = (size_t)t.nz * t.nx * t.Nv * rsz,
-                 fz_bytes = (size_t)t.ny * t.nx * t.Nv * rsz;
+    const size_t fx_bytes = (size_t)t.nz * t.ny * t.Nvs * rsz, fy_bytes = (size_t)t.nz * t.nx * t.Nvs * rsz,
+                 fz_bytes = (size_t)t.ny * t.nx * t.Nvs * rsz;
     const size_t o_fx = cv.take(fx_bytes), o_fy = cv.take(fy_bytes), o_fz = cv.take(fz_bytes);
     const size_t o_part = cv.take((size_t)t.n_vg * NPART * n * 8);
     const size_t o_sums = cv.take((size_t)NSUM * n * sizeof(double));
@@ -97,11 +120,13 @@ extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, c
     const size_t o_work = cv.take(t.work.size() * sizeof(int4));
     const size_t o_oct = cv.take(3 * 8 * sizeof(int));
     const size_t o_vgoct = cv.take(t.vg_oct.size() * sizeof(int));
+    const size_t o_lines = cv.take(t.pack ? t.lines32.size() * sizeof(float) : 0),
+                 o_xnodes = cv.take(t.pack ? t.xnodes32.size() * sizeof(float) : 0);
     const size_t o_solid = cv.take(t.any_solid ? n : 0);
     const size_t o_bmass = cv.take(close_blocks(n) * sizeof(double)), o_bres = cv.take((size_t)n_red * 10 * sizeof(double)),
                  o_bbad = cv.take(n_red * sizeof(int)), o_scale = cv.take(2 * sizeof(double)),
                  o_resid = cv.take(2 * sizeof(double));
-    if (cv.used > (size_t)KGS_NOALLOC_SCRATCH_BYTES) return KGS_EINVAL;  // too large for the fixed array
+    if (cv.used > (size_t)KGS_NOALLOC_SCRATCH_BYTES) return TOO_LARGE;  // for the fixed array
 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return KGS_ECUDA;
@@ -137,6 +162,8 @@ extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, c
               put(o_norm, t.wall_norm.data(), t.wall_norm.size() * sizeof(double)) &&
               put(o_work, t.work.data(), t.work.size() * sizeof(int4)) && put(o_oct, oct, sizeof oct) &&
               put(o_vgoct, t.vg_oct.data(), t.vg_oct.size() * sizeof(int)) &&
+              (!t.pack || (put(o_lines, t.lines32.data(), t.lines32.size() * sizeof(float)) &&
+                           put(o_xnodes, t.xnodes32.data(), t.xnodes32.size() * sizeof(float)))) &&
               (!t.any_solid || put(o_solid, t.solid.data(), n));
     if (!ok) return KGS_ECUDA;
     // what the previous call left behind: face planes and coefficients start at zero
@@ -164,15 +191,19 @@ extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, c
     a.oct_vstart = d_oct;
     a.oct_vcount = d_oct + 8;
     a.oct_vgbase = d_oct + 16;
-    a.Nv = t.Nv;
+    a.Nv = t.Nvs;
     a.vg_size = t.vg_size;
     a.vel = b + o_vel;
     a.velm = b + o_velm;
     a.nxo_max = t.nxo_max;
-    a.line16 = 1;
+    a.line16 = t.lines16() ? 1 : 0;
+    a.pack = t.pack;
+    a.lines = reinterpret_cast<const float *>(b + o_lines);
+    a.xnodes = reinterpret_cast<const float *>(b + o_xnodes);
+    a.xn_stride = t.xn_stride;
     for (int o = 0; o < 8; o++) {
         a.oct_nx[o] = t.oct_nx[o] > 0 ? t.oct_nx[o] : 1;
-        if (t.oct_vcount[o] > 0 && t.oct_nx[o] != 16) a.line16 = 0;
+        a.oct_line0[o] = t.oct_line0[o];
     }
     a.any_solid = t.any_solid ? 1 : 0;
     t.set_uniformity(a);
@@ -186,9 +217,10 @@ extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, c
     a.part = b + o_part;
     a.ncell = n;
     const int4 *d_work = reinterpret_cast<const int4 *>(b + o_work);
+    const SweepKind kind = t.kind();
     for (size_t s = 0; s < t.stage_n.size(); s++) {
         a.work = d_work + t.stage_off[s];
-        if (launch_sweep(t.precision, t.tv, a, t.stage_n[s], t.max_vg, st) != cudaSuccess) return KGS_ECUDA;
+        if (launch_sweep(kind, a, t.stage_n[s], t.max_vg, st) != cudaSuccess) return KGS_ECUDA;
     }
     PartSumArgs pa;
     pa.ncell = n;
@@ -237,3 +269,5 @@ extern "C" int kgs_iterate_noalloc(const kgs_grid *grid, const uint8_t *solid, c
     if (residual) *residual = h[0];
     return h[1] != 0.0 ? KGS_EDIVERGED : KGS_OK;
 }
+
+}  // namespace

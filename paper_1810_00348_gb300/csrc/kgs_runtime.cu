@@ -152,12 +152,18 @@ SweepArgs kgs::ctx_sweep_args(const kgs_ctx *c)
     a.oct_vstart = c->d_vstart;
     a.oct_vcount = c->d_vcount;
     a.oct_vgbase = c->d_vgbase;
-    a.Nv = t.Nv;
+    a.Nv = t.Nvs;
     a.vg_size = t.vg_size;
     a.vel = c->vel;
     a.velm = c->velm;
     a.nxo_max = t.nxo_max;
-    for (int o = 0; o < 8; o++) a.oct_nx[o] = t.oct_nx[o] > 0 ? t.oct_nx[o] : 1;
+    for (int o = 0; o < 8; o++) {
+        a.oct_nx[o] = t.oct_nx[o] > 0 ? t.oct_nx[o] : 1;
+        a.oct_line0[o] = t.oct_line0[o];
+    }
+    a.lines = c->lines;
+    a.xnodes = c->xnodes;
+    a.xn_stride = t.xn_stride;
     a.any_solid = t.any_solid ? 1 : 0;
     a.blk_plain = c->blk_plain;
     a.coef = c->coef;
@@ -177,9 +183,8 @@ SweepArgs kgs::ctx_sweep_args(const kgs_ctx *c)
     a.acc_slots = t.acc_slots;
     a.tok = c->p_tok;
     a.ncell = t.ncell;
-    a.line16 = 1;
-    for (int o = 0; o < 8; o++)
-        if (t.oct_vcount[o] > 0 && t.oct_nx[o] != 16) a.line16 = 0;
+    a.line16 = t.lines16() ? 1 : 0;
+    a.pack = t.pack;
     t.set_uniformity(a);
     return a;
 }
@@ -221,8 +226,7 @@ int kgs::ctx_launch_stages(kgs_ctx *c)
         ba.skip_publish = -1;
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[0], st));
         KGS_CHECK(
-            launch_sweep_persistent(t.precision, t.tv, a.line16, a.uniform, ba, t.nxo_max, c->persist_grid, st,
-                                    t.order, t.dev && t.order == 1));
+            launch_sweep_persistent(t.kind(), ba, t.nxo_max, c->persist_grid, st));
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[1], st));
         c->kernel_launches += 1;
         c->sweep_launches += 1;
@@ -232,7 +236,7 @@ int kgs::ctx_launch_stages(kgs_ctx *c)
     for (int s = 0; s < ns; s++) {
         a.work = c->work + t.stage_off[s];
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[2 * s], st));
-        KGS_CHECK(launch_sweep(t.precision, t.tv, a, t.stage_n[s], t.max_vg, st));
+        KGS_CHECK(launch_sweep(t.kind(), a, t.stage_n[s], t.max_vg, st));
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[2 * s + 1], st));
     }
     c->kernel_launches += ns;
@@ -243,7 +247,7 @@ int kgs::ctx_launch_stages(kgs_ctx *c)
 void kgs::ctx_stage_items(const HostTables &t, int inst, int stage, std::vector<int4> &out)
 {
     for (int o = 0; o < 8; o++) {
-        const int ng = (t.oct_vcount[o] + t.vg_size - 1) / t.vg_size;
+        const int ng = t.groups(o);
         for (int vg = 0; vg < ng; vg++)
             for (int bzr = 0; bzr < t.nbz; bzr++)
                 for (int byr = 0; byr < t.nby; byr++) {
@@ -292,10 +296,8 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     const HostTables &t = c->t;
     int sms = 0;
     KGS_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
-    const SweepArgs a = ctx_sweep_args(c);
-    const int per_sm = sweep_persistent_occupancy(t.precision, t.tv, a.line16, a.uniform,
-                                                  sweep_smem_bytes(t.precision, t.tv, a.line16, t.nxo_max, t.order),
-                                                  t.order, t.dev && t.order == 1);
+    const SweepKind kind = t.kind();
+    const int per_sm = sweep_persistent_occupancy(kind, sweep_smem_bytes(kind, t.nxo_max));
     // the second-order sweep and the deviation-form source exist only in the
     // persistent kernel
     if (per_sm < 1 && (t.order == 2 || t.dev)) return KGS_EINVAL;
@@ -498,9 +500,9 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         (rc = dalloc_t(c, &c->rho_w, 6 * n)) || (rc = dalloc_t(c, &c->rho_w_new, 6 * n)) ||
         (rc = dalloc(c, &c->coef, n * NCOEF * rsz)) || (rc = upload(c, &c->vel64, t.vel64)) || (rc = upload(c, &c->axis64, t.axis64)) ||
         (rc = upload_real(c, &c->vel, t.vel64)) || (rc = upload_real(c, &c->mtab, t.mt)) ||
-        (rc = dalloc(c, &c->FX, (size_t)t.nz * t.ny * t.Nv * rsz)) ||
-        (rc = dalloc(c, &c->FY, (size_t)t.nz * t.nx * t.Nv * rsz)) ||
-        (rc = dalloc(c, &c->FZ, (size_t)t.ny * t.nx * t.Nv * rsz)) ||
+        (rc = dalloc(c, &c->FX, (size_t)t.nz * t.ny * t.Nvs * rsz)) ||
+        (rc = dalloc(c, &c->FY, (size_t)t.nz * t.nx * t.Nvs * rsz)) ||
+        (rc = dalloc(c, &c->FZ, (size_t)t.ny * t.nx * t.Nvs * rsz)) ||
         (rc = dalloc_t(c, &c->sums, (size_t)NSUM * n)) || (rc = upload(c, &c->rdx, t.rdx)) ||
         (rc = upload(c, &c->rdy, t.rdy)) || (rc = upload(c, &c->rdz, t.rdz)) || (rc = upload(c, &c->ddx, t.dx)) ||
         (rc = upload(c, &c->ddy, t.dy)) || (rc = upload(c, &c->ddz, t.dz)) ||
@@ -514,6 +516,7 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->scale, 2)) ||
         (rc = dalloc_t(c, &c->resid, 3)))
         return fail(rc);
+    if (t.pack && ((rc = upload(c, &c->lines, t.lines32)) || (rc = upload(c, &c->xnodes, t.xnodes32)))) return fail(rc);
     if (t.precision == KGS_FP64) {
         if ((rc = upload(c, reinterpret_cast<double **>(&c->velm), t.velm64))) return fail(rc);
     } else {
@@ -521,18 +524,18 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
     }
     if (t.any_solid && ((rc = upload(c, &c->solid, t.solid)) || (rc = upload(c, &c->blk_plain, t.blk_plain))))
         return fail(rc);
-    if (t.order == 2 && ((rc = dalloc(c, &c->FX2, (size_t)t.nz * t.ny * t.Nv * rsz)) ||
-                         (rc = dalloc(c, &c->FY2, (size_t)t.nz * t.nx * t.Nv * rsz)) ||
-                         (rc = dalloc(c, &c->FZ2, (size_t)t.ny * t.nx * t.Nv * rsz))))
+    if (t.order == 2 && ((rc = dalloc(c, &c->FX2, (size_t)t.nz * t.ny * t.Nvs * rsz)) ||
+                         (rc = dalloc(c, &c->FY2, (size_t)t.nz * t.nx * t.Nvs * rsz)) ||
+                         (rc = dalloc(c, &c->FZ2, (size_t)t.ny * t.nx * t.Nvs * rsz))))
         return fail(rc);
-    if (cudaMemset(c->FX, 0, (size_t)t.nz * t.ny * t.Nv * rsz) != cudaSuccess ||
-        cudaMemset(c->FY, 0, (size_t)t.nz * t.nx * t.Nv * rsz) != cudaSuccess ||
-        cudaMemset(c->FZ, 0, (size_t)t.ny * t.nx * t.Nv * rsz) != cudaSuccess ||
+    if (cudaMemset(c->FX, 0, (size_t)t.nz * t.ny * t.Nvs * rsz) != cudaSuccess ||
+        cudaMemset(c->FY, 0, (size_t)t.nz * t.nx * t.Nvs * rsz) != cudaSuccess ||
+        cudaMemset(c->FZ, 0, (size_t)t.ny * t.nx * t.Nvs * rsz) != cudaSuccess ||
         cudaMemset(c->coef, 0, n * NCOEF * rsz) != cudaSuccess)
         return fail(KGS_ECUDA);
-    if (t.order == 2 && (cudaMemset(c->FX2, 0, (size_t)t.nz * t.ny * t.Nv * rsz) != cudaSuccess ||
-                         cudaMemset(c->FY2, 0, (size_t)t.nz * t.nx * t.Nv * rsz) != cudaSuccess ||
-                         cudaMemset(c->FZ2, 0, (size_t)t.ny * t.nx * t.Nv * rsz) != cudaSuccess))
+    if (t.order == 2 && (cudaMemset(c->FX2, 0, (size_t)t.nz * t.ny * t.Nvs * rsz) != cudaSuccess ||
+                         cudaMemset(c->FY2, 0, (size_t)t.nz * t.nx * t.Nvs * rsz) != cudaSuccess ||
+                         cudaMemset(c->FZ2, 0, (size_t)t.ny * t.nx * t.Nvs * rsz) != cudaSuccess))
         return fail(KGS_ECUDA);
     if (cudaMallocHost(&c->h_resid, 3 * sizeof(double)) != cudaSuccess) return fail(KGS_ENOMEM);
     if (cudaMemset(c->resid, 0, 3 * sizeof(double)) != cudaSuccess) return fail(KGS_ECUDA);

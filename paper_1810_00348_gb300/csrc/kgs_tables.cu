@@ -17,6 +17,21 @@ double maxwellian(double rho, const double U[3], double T, const double xi[3])
 
 }  // namespace
 
+void pack_order(int v0, int count, int nxo, std::vector<int> &place)
+{
+    place.clear();
+    for (int half = 0; half < 2; half++) {
+        const int b = half * NT, n = std::min(NT, count - b);
+        if (n <= 0) break;
+        const int head = std::min(n, (nxo - (v0 + b) % nxo) % nxo), full = (n - head) / nxo, pairs = full / 2;
+        for (int q = 0; q < pairs; q++)
+            for (int ix = 0; ix < nxo; ix++)
+                for (int h = 0; h < 2; h++) place.push_back(b + head + (2 * q + h) * nxo + ix);
+        for (int v = 0; v < head; v++) place.push_back(b + v);
+        for (int v = head + 2 * pairs * nxo; v < n; v++) place.push_back(b + v);
+    }
+}
+
 bool dev_source_applies(const kgs_grid *grid, const kgs_bc *bc)
 {
     for (int s = 0; s < 6; s++)
@@ -93,7 +108,7 @@ int validate_problem(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid
 
 void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid *vg,
                   const kgs_gas *gas, const kgs_bc *bc, int precision, int wall_norm, int v_per_cta, int block_z,
-                  int vz_begin, int vz_end, int order, int dev_source)
+                  int vz_begin, int vz_end, int order, int dev_source, int pack)
 {
     t.nx = grid->nx;
     t.ny = grid->ny;
@@ -142,22 +157,56 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
     for (int i = 0; i < nz; i++) t.rdz[i] = 1.0 / t.dz[i];
 
     // ---- velocities sorted by octant (bit d set: xi_d >= 0), ix fastest ----
-    std::vector<int> vsorted;
-    vsorted.reserve(t.Nv);
     auto oct_of = [&](int ix, int iy, int iz) {
         return (vg->xi_x[ix] >= 0.0 ? 1 : 0) | (vg->xi_y[iy] >= 0.0 ? 2 : 0) | (vg->xi_z[iz] >= 0.0 ? 4 : 0);
     };
+    t.pack = pack && t.precision == KGS_MIXED && t.tv == 2;
+    std::vector<int> vsorted, natural, place;  // slot -> velocity
+    vsorted.reserve(t.Nv + 8);
+    t.lines32.clear();
     for (int o = 0; o < 8; o++) {
+        natural.clear();
         t.oct_vstart[o] = (int)vsorted.size();
+        t.oct_line0[o] = (int)(t.lines32.size() / 8);
         for (int iz = t.vz0; iz < t.vz1; iz++)
-            for (int iy = 0; iy < t.nvy; iy++)
+            for (int iy = 0; iy < t.nvy; iy++) {
+                const size_t before = natural.size();
                 for (int ix = 0; ix < t.nvx; ix++)
-                    if (oct_of(ix, iy, iz) == o) vsorted.push_back(ix + t.nvx * (iy + t.nvy * iz));
-        t.oct_vcount[o] = (int)vsorted.size() - t.oct_vstart[o];
+                    if (oct_of(ix, iy, iz) == o) natural.push_back(ix + t.nvx * (iy + t.nvy * iz));
+                if (natural.size() == before) continue;
+                const double y = vg->xi_y[iy], z = vg->xi_z[iz];
+                const float rec[8] = {(float)y, (float)z, (float)(vg->w_y[iy] * vg->w_z[iz]),
+                                      (float)(y - (double)(float)y), (float)(z - (double)(float)z), 0.f, 0.f, 0.f};
+                t.lines32.insert(t.lines32.end(), rec, rec + 8);
+            }
+        t.oct_vcount[o] = (int)natural.size();
         int cnt = 0;
         for (int ix = 0; ix < t.nvx; ix++) cnt += ((vg->xi_x[ix] >= 0.0 ? 1 : 0) == (o & 1));
         t.oct_nx[o] = cnt;
         t.nxo_max = std::max(t.nxo_max, cnt);
+        if (!t.pack) {
+            vsorted.insert(vsorted.end(), natural.begin(), natural.end());
+            continue;
+        }
+        for (int v0 = 0; v0 < t.oct_vcount[o]; v0 += t.vg_size) {
+            pack_order(v0, std::min(t.vg_size, t.oct_vcount[o] - v0), cnt, place);
+            for (int p : place) vsorted.push_back(natural[v0 + p]);
+        }
+        if (vsorted.size() % 2) vsorted.push_back(vsorted.back());  // swept, never summed
+    }
+    t.Nvs = (int)vsorted.size();
+    t.xn_stride = t.nxo_max;
+    t.xnodes32.assign((size_t)8 * t.xn_stride * 4, 0.f);
+    for (int o = 0; o < 8; o++) {
+        float *e = &t.xnodes32[(size_t)o * t.xn_stride * 4];
+        for (int ix = 0; ix < t.nvx; ix++) {
+            if ((vg->xi_x[ix] >= 0.0 ? 1 : 0) != (o & 1)) continue;
+            const double x = vg->xi_x[ix];
+            e[0] = (float)x;
+            e[1] = (float)(x - (double)(float)x);
+            e[2] = (float)vg->w_x[ix];
+            e += 4;
+        }
     }
     t.axis64.clear();
     t.axis64.insert(t.axis64.end(), vg->xi_x, vg->xi_x + t.nvx);
@@ -166,10 +215,10 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
     t.axis64.insert(t.axis64.end(), vg->w_x, vg->w_x + t.nvx);
     t.axis64.insert(t.axis64.end(), vg->w_y, vg->w_y + t.nvy);
     t.axis64.insert(t.axis64.end(), vg->w_z, vg->w_z + t.nvz);
-    t.vel64.assign((size_t)t.Nv * 4, 0.0);
-    t.velm64.assign((size_t)t.Nv * 8, 0.0);
-    t.velm32.assign((size_t)t.Nv * 8, 0.f);
-    for (int g = 0; g < t.Nv; g++) {
+    t.vel64.assign((size_t)t.Nvs * 4, 0.0);
+    t.velm64.assign((size_t)t.Nvs * 8, 0.0);
+    t.velm32.assign((size_t)t.Nvs * 8, 0.f);
+    for (int g = 0; g < t.Nvs; g++) {
         const int a = vsorted[g];
         const int ix = a % t.nvx, iy = (a / t.nvx) % t.nvy, iz = a / (t.nvx * t.nvy);
         t.vel64[g * 4 + 0] = vg->xi_x[ix];
@@ -191,7 +240,7 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
     t.max_vg = 0;
     for (int o = 0; o < 8; o++) {
         t.oct_vgbase[o] = (int)t.vg_oct.size();
-        const int ng = (t.oct_vcount[o] + t.vg_size - 1) / t.vg_size;
+        const int ng = t.groups(o);
         for (int g = 0; g < ng; g++) t.vg_oct.push_back(o);
         t.max_vg = std::max(t.max_vg, ng);
     }
@@ -201,7 +250,7 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
     // most the smallest group count of a non-empty octant
     t.nacc = NACC_MAX;
     for (int o = 0; o < 8; o++)
-        if (t.oct_vcount[o] > 0) t.nacc = std::min(t.nacc, (t.oct_vcount[o] + t.vg_size - 1) / t.vg_size);
+        if (t.oct_vcount[o] > 0) t.nacc = std::min(t.nacc, t.groups(o));
 
     // ---- wall tables: kinds 0..5 domain sides, 6 solid surfaces ----
     double wallU[7][3], wallT[7];
@@ -246,7 +295,19 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
             refT = bc->T_in;
             for (int d = 0; d < 3; d++) refU[d] = bc->U_in[d];
         }
-        for (int g = 0; g < t.Nv; g++) {
+        std::vector<int> slot(t.Nvs);  // the sums run over the velocities in sorted order
+        int n_slot = 0;
+        for (int o = 0; o < 8; o++) {
+            for (int v0 = 0; v0 < t.oct_vcount[o]; v0 += t.vg_size) {
+                const int count = std::min(t.vg_size, t.oct_vcount[o] - v0);
+                if (t.pack) pack_order(v0, count, t.oct_nx[o], place);
+                for (int p = 0; p < count; p++)
+                    slot[n_slot + (t.pack ? place[p] : p)] = t.oct_vstart[o] + v0 + p;
+                n_slot += count;
+            }
+        }
+        slot.resize(n_slot);
+        for (const int g : slot) {
             const double *v = &t.vel64[g * 4];
             const double m64 = maxwellian(refRho, refU, refT, v);
             const float m32 = (float)m64;
@@ -263,11 +324,11 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
             }
         }
     }
-    t.mt.assign((size_t)MT_ROWS * t.Nv, 0.0);
-    for (int g = 0; g < t.Nv; g++) {
+    t.mt.assign((size_t)MT_ROWS * t.Nvs, 0.0);
+    for (int g = 0; g < t.Nvs; g++) {
         const double *v = &t.vel64[g * 4];
-        for (int k = 0; k < 7; k++) t.mt[(size_t)k * t.Nv + g] = maxwellian(1.0, wallU[k], wallT[k], v);
-        t.mt[(size_t)MT_INFLOW * t.Nv + g] = t.any_inflow ? maxwellian(bc->rho_in, bc->U_in, bc->T_in, v) : 0.0;
+        for (int k = 0; k < 7; k++) t.mt[(size_t)k * t.Nvs + g] = maxwellian(1.0, wallU[k], wallT[k], v);
+        t.mt[(size_t)MT_INFLOW * t.Nvs + g] = t.any_inflow ? maxwellian(bc->rho_in, bc->U_in, bc->T_in, v) : 0.0;
     }
     // ---- per (side, cell): wall kind and flags ----
     t.wall_kind.assign(6 * n, -1);
