@@ -152,6 +152,7 @@ int enqueue_iteration(kgs_batch *b, int which)
     ba.error = b->d_error;
     ba.spin_limit = b->spin_limit;
     ba.skip_publish = b->skip_publish;
+    ba.announce_every = announce_every(b->precision, ba.n_items, b->grid);
     // external records: inside a capture a plain record only orders streams
     KGS_CHECK(cudaEventRecordWithFlags(b->ev[0], st, cudaEventRecordExternal));
     KGS_CHECK(launch_sweep_persistent(b->kind, ba, b->nxo_max, b->grid, st));

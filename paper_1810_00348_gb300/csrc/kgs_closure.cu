@@ -24,12 +24,15 @@ template <typename Real>
 __global__ void coef_kernel(const double *__restrict__ mac, const uint8_t *__restrict__ solid,
                             const uint8_t *__restrict__ side_flags, const double *__restrict__ rdx,
                             const double *__restrict__ rdy, const double *__restrict__ rdz, int nx, int ny, int nz,
-                            double mu_ref, double omega, double Pr, int dev_src, Real *__restrict__ coef)
+                            double mu_ref, double omega, double Pr, int dev_src, Real *__restrict__ coef,
+                            const double *__restrict__ rho_w, float *__restrict__ rho_w32)
 {
     const size_t ncell = (size_t)nx * ny * nz;
     const size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncell) return;
     const int i = (int)(c % nx), j = (int)((c / nx) % ny), k = (int)(c / ((size_t)nx * ny));
+    if (rho_w32)
+        for (int s = 0; s < 6; s++) rho_w32[s * ncell + c] = (float)rho_w[s * ncell + c];
     Real out[NCOEF];
     for (int q = 0; q < NCOEF; q++) out[q] = Real(0);
     const int sf = side_flags[c];  // bits 0..5 solid neighbour, 6..11 wall face (packed in 2 bytes)
@@ -642,15 +645,16 @@ inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 cudaError_t launch_coef(int precision, const double *mac, const uint8_t *solid, const uint8_t *side_flags,
                         const double *rdx, const double *rdy, const double *rdz, int nx, int ny, int nz,
-                        double mu_ref, double omega, double Pr, void *coef, cudaStream_t s, int dev_src)
+                        double mu_ref, double omega, double Pr, void *coef, cudaStream_t s, int dev_src,
+                        const double *rho_w, float *rho_w32)
 {
     const size_t n = (size_t)nx * ny * nz;
     if (precision == 0)
         coef_kernel<double><<<nblk(n, 256), 256, 0, s>>>(mac, solid, side_flags, rdx, rdy, rdz, nx, ny, nz, mu_ref,
-                                                          omega, Pr, 0, static_cast<double *>(coef));
+                                                          omega, Pr, 0, static_cast<double *>(coef), nullptr, nullptr);
     else
         coef_kernel<float><<<nblk(n, 256), 256, 0, s>>>(mac, solid, side_flags, rdx, rdy, rdz, nx, ny, nz, mu_ref,
-                                                         omega, Pr, dev_src, static_cast<float *>(coef));
+                                                         omega, Pr, dev_src, static_cast<float *>(coef), rho_w, rho_w32);
     return cudaGetLastError();
 }
 

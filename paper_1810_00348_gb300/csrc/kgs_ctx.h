@@ -27,6 +27,7 @@ struct kgs_ctx {
     void *coef = nullptr, *vel = nullptr, *velm = nullptr, *mtab = nullptr, *FX = nullptr, *FY = nullptr,
          *FZ = nullptr;
     float *lines = nullptr, *xnodes = nullptr;            // packed FP32 sweep: HostTables::lines32, xnodes32
+    float *rho_w32 = nullptr;                             // packed FP32 sweep: rho_w in FP32
     void *FX2 = nullptr, *FY2 = nullptr, *FZ2 = nullptr;  // second face planes of the order-2 sweep
     void *part = nullptr;   // staged sweep only: per-(group, cell) partials
     void *acc = nullptr;    // persistent sweep: ordered accumulators [nacc][ncell][acc_slots]

@@ -99,8 +99,8 @@ struct SweepArgs {
     const void *vel;              // Real[Nv][4]: xi_x, xi_y, xi_z, w (octant-sorted)
     const void *velm;             // Real[Nv][8]: w_x, w_y w_z, the low parts of xi_x, xi_y, xi_z
                                   // (xi = hi + lo with hi = the value in vel), M_ref (FP32
-                                  // path; 0 for FP64), the rounding error of M_ref (FP32
-                                  // path), 1 unused
+                                  // path; 0 for FP64), the rounding error of M_ref and
+                                  // |xi|^2 of the rounded node (FP32 path)
     int pack;                     // packed velocity slots (HostTables::pack, FP32 with two velocities per thread)
     int oct_line0[8];             // packed: first row of each octant in lines
     const float *lines;           // packed: [lines][8] xi_y, xi_z, w_y w_z, low parts of xi_y, xi_z
@@ -112,6 +112,7 @@ struct SweepArgs {
     const uint8_t *blk_plain;     // [nbz][nby][nbx]: 1 = no solid cell and no solid neighbour in the block (or NULL)
     const void *coef;             // Real[ncell][NCOEF]
     const double *rho_w;          // [6][ncell]
+    const float *rho_w32;         // the same in FP32 (persistent packed FP32 sweep)
     const void *mtab;             // Real[MT_ROWS][Nv]: unit wall Maxwellians, free stream
     int side_inflow[6];           // domain side s is a free-stream boundary
     void *FX, *FY, *FZ;           // face planes: [nz*ny][Nv], [nz*nx][Nv], [ny*nx][Nv]
@@ -120,7 +121,7 @@ struct SweepArgs {
     void *part;                   // staged sweep: [n_vg][ncell][NPART], double (FP64 path) or
                                   // float2 (s, c) with value s - c (FP32 path, Kahan pair)
     void *acc;                    // persistent sweep: [nacc][ncell][acc_slots] ordered accumulators
-    int nacc;                     // accumulators: velocity group g of an octant adds into g % nacc
+    int nacc;                     // accumulators: velocity group g (of all groups) adds into g % nacc
     int acc_slots;                // ACC_COMPACT or ACC_SPLIT
     int *tok;                     // persistent sweep: [nacc][nbz][nby][nbx] chain tokens
     unsigned long long ncell;
@@ -138,7 +139,7 @@ struct BatchSweepArgs {
     const int4 *items;
     int n_items;
     int *counter;                 // claim counter, zero at launch
-    int *flags;                   // completion flags, zero at launch
+    int *flags;                   // progress of each item, zero at launch
     const int *flag_off;          // [n_inst] first flag of each instance
     const int *pos;               // [n_items] place of each item in its accumulator chain
     void *scratch;                // [grid][bz * SLICE][NPART] per-CTA moment partials
@@ -146,7 +147,21 @@ struct BatchSweepArgs {
     int *error;                   // set to 1 when a bounded wait gives up
     long long spin_limit;         // polls before a wait gives up
     int skip_publish;             // fault injection: this item never sets its flag (-1: none)
+    int announce_every;           // slices between two announcements of an item's progress (announce_every())
 };
+// A block that announces its progress lets its x and y neighbours overlap
+// with it, at the price of a release (which waits for the block's stores) per
+// announcement.  FP64 slices take 20 us or more and announce each.  FP32 slices
+// take 6 to 12 us: measured times per iteration with an announcement every 1 /
+// 2 / 8 slices or only at the end are 392 / 412 / 545 / 734 us for 64 items
+// (16^3 cells x 16^3 velocities), 3.66 / 3.66 / 3.74 / 5.3 ms for 2520 items
+// (45 x 38 x 41 x 22 x 19 x 24) and 19.44 / 19.33 / 19.26 / 19.3 ms for 16384
+// (64^3 x 32^3), on 304 resident blocks.
+inline int announce_every(int precision, int n_items, int grid)
+{
+    if (precision == 0 || n_items <= grid) return 1;
+    return n_items <= 16 * grid ? 2 : 8;
+}
 // Bytes of one CTA's scratch partials for blocks bz cells deep (both precisions
 // store 8 bytes per slot).
 inline size_t sweep_scratch_bytes(int bz) { return (size_t)bz * SLICE * NPART * 8; }
@@ -245,10 +260,12 @@ struct ClosureArgs {
 };
 
 // dev_src (FP32 only): the C_RDX / C_RDY slots carry the exponent terms of
-// the second-order sweep's deviation source instead of 1/dx, 1/dy.
+// the second-order sweep's deviation source instead of 1/dx, 1/dy.  rho_w32
+// (may be NULL) receives rho_w [6][ncell] rounded to FP32.
 cudaError_t launch_coef(int precision, const double *mac, const uint8_t *solid, const uint8_t *cell_flags_side,
                         const double *rdx, const double *rdy, const double *rdz, int nx, int ny, int nz,
-                        double mu_ref, double omega, double Pr, void *coef, cudaStream_t s, int dev_src = 0);
+                        double mu_ref, double omega, double Pr, void *coef, cudaStream_t s, int dev_src = 0,
+                        const double *rho_w = nullptr, float *rho_w32 = nullptr);
 // Cells per block of the closure kernel; blk_mass holds close_blocks(ncell)
 // values.
 constexpr int CLOSE_CELLS = 32;

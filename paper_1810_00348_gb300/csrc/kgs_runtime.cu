@@ -168,6 +168,7 @@ SweepArgs kgs::ctx_sweep_args(const kgs_ctx *c)
     a.blk_plain = c->blk_plain;
     a.coef = c->coef;
     a.rho_w = c->rho_w;
+    a.rho_w32 = c->rho_w32;
     a.mtab = c->mtab;
     for (int s = 0; s < 6; s++) a.side_inflow[s] = t.side_inflow[s];
     a.FX = c->FX;
@@ -193,7 +194,7 @@ int kgs::ctx_launch_coef(kgs_ctx *c)
 {
     const HostTables &t = c->t;
     KGS_CHECK(launch_coef(t.precision, c->mac, c->solid, c->side_flags, c->rdx, c->rdy, c->rdz, t.nx, t.ny, t.nz,
-                          t.mu_ref, t.omega, t.Pr, c->coef, c->stream, t.dev ? 1 : 0));
+                          t.mu_ref, t.omega, t.Pr, c->coef, c->stream, t.dev ? 1 : 0, c->rho_w, c->rho_w32));
     c->kernel_launches += 1;
     return KGS_OK;
 }
@@ -224,6 +225,7 @@ int kgs::ctx_launch_stages(kgs_ctx *c)
         ba.error = reinterpret_cast<int *>(c->resid + 2);
         ba.spin_limit = c->spin_limit;
         ba.skip_publish = -1;
+        ba.announce_every = announce_every(t.precision, ba.n_items, c->persist_grid);
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[0], st));
         KGS_CHECK(
             launch_sweep_persistent(t.kind(), ba, t.nxo_max, c->persist_grid, st));
@@ -267,12 +269,12 @@ void kgs::chain_positions(const std::vector<int4> &items, const std::vector<cons
     for (size_t it = 0; it < items.size(); it++) {
         const int4 w = items[it];
         const HostTables &t = *tabs[w.x];
-        const int o = w.y >> 24, vg = w.y & 0xffffff;
+        const int o = w.y >> 24;
         const int bxr = w.z & 1023, byr = (w.z >> 10) & 1023, bzr = (w.z >> 20) & 1023;
         const int bx = (o & 1) ? bxr : t.nbx - 1 - bxr;
         const int by = (o & 2) ? byr : t.nby - 1 - byr;
         const int bz = (o & 4) ? bzr : t.nbz - 1 - bzr;
-        const size_t key = (((size_t)(vg % t.nacc) * t.nbz + bz) * t.nby + by) * t.nbx + bx;
+        const size_t key = (((size_t)(w.w % t.nacc) * t.nbz + bz) * t.nby + by) * t.nbx + bx;
         pos[it] = count[w.x][key]++;
     }
 }
@@ -516,7 +518,8 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->scale, 2)) ||
         (rc = dalloc_t(c, &c->resid, 3)))
         return fail(rc);
-    if (t.pack && ((rc = upload(c, &c->lines, t.lines32)) || (rc = upload(c, &c->xnodes, t.xnodes32)))) return fail(rc);
+    if (t.pack && ((rc = upload(c, &c->lines, t.lines32)) || (rc = upload(c, &c->xnodes, t.xnodes32)) || (rc = dalloc_t(c, &c->rho_w32, 6 * n))))
+        return fail(rc);
     if (t.precision == KGS_FP64) {
         if ((rc = upload(c, reinterpret_cast<double **>(&c->velm), t.velm64))) return fail(rc);
     } else {

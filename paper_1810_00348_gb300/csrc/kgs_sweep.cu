@@ -123,7 +123,7 @@ struct SmemLayout {
 // and FX2/FY2/FZ2 carry the block outflow one cell further upwind.
 template <typename Real, int TV, int LINE, bool COHERENT, bool UNIF, int ORDER = 1, bool DEV = false>
 __device__ __forceinline__ void sweep_item(const SweepArgs &a, const int4 w, const int vgy, unsigned char *smem,
-                                           void *scratch)
+                                           void *scratch, Pipe *pipe)
 {
     // the deviation-form FP32 source (uniform grids: it uses the width slots)
     constexpr bool DEVF = sizeof(Real) == 4 && (ORDER == 2 || DEV);
@@ -444,6 +444,7 @@ __device__ __forceinline__ void sweep_item(const SweepArgs &a, const int4 w, con
                 }
             }
         }
+        if (COHERENT && t == 0) pipe->wait(min(lk + 2, ez));
         __syncthreads();
         // c_x = xi_x - U_x of each cell of the slice as a float pair, per x node
         // (lines of LINE nodes keep theirs in registers instead)
@@ -740,6 +741,7 @@ __device__ __forceinline__ void sweep_item(const SweepArgs &a, const int4 w, con
             }
         }
         __syncthreads();
+        if (COHERENT && t == 0) pipe->announce(lk + 1, ez);
 
         // ---- moments of the slice over the group's velocities ----
         {
@@ -981,19 +983,20 @@ __device__ __forceinline__ void sweep_item(const SweepArgs &a, const int4 w, con
         }
     }
 }
+
 // One wavefront stage: CTA (x, y) = (work item x of the stage, velocity group y).
 template <typename Real, int TV, int LINE, bool UNIF>
 __global__ void __launch_bounds__(NT, 2) sweep_kernel(const SweepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    sweep_item<Real, TV, LINE, false, UNIF>(a, a.work[blockIdx.x], blockIdx.y, smem, nullptr);
+    sweep_item<Real, TV, LINE, false, UNIF>(a, a.work[blockIdx.x], blockIdx.y, smem, nullptr, nullptr);
 }
 template <typename Real, int TV, int LINE, bool UNIF, int ORDER, bool DEV>
 __global__ void __launch_bounds__(NT, 2) sweep_persistent_kernel(const BatchSweepArgs b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    persistent_loop<Real>(b, [&](const SweepArgs &a, const int4 w, const int vg, void *scratch) {
-        sweep_item<Real, TV, LINE, true, UNIF, ORDER, DEV>(a, w, vg, smem, scratch);
+    persistent_loop<Real>(b, [&](const SweepArgs &a, const int4 w, const int vg, void *scratch, Pipe &pipe) {
+        sweep_item<Real, TV, LINE, true, UNIF, ORDER, DEV>(a, w, vg, smem, scratch, &pipe);
     });
 }
 

@@ -163,29 +163,65 @@ __device__ __forceinline__ void st_release(int *p, int v)
     asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Bounded wait for a completion flag: true once it is set, false after
-// `limit` polls (the caller then records an error and returns).
-__device__ inline bool wait_flag(const int *p, long long limit)
+// Bounded wait for a counter that only grows to reach `v`: its value then, or
+// -1 after `limit` polls (the caller then records an error and returns).
+__device__ inline int wait_count(const int *p, int v, long long limit)
 {
     for (long long i = 0; i < limit; i++) {
-        if (ld_acquire(p) != 0) return true;
+        const int have = ld_acquire(p);
+        if (have >= v) return have;
         __nanosleep(100);
     }
-    return false;
+    return -1;
 }
 
-// Bounded wait for a chain token to reach `v` (tokens only grow).
-__device__ inline bool wait_token(const int *p, int v, long long limit)
-{
-    for (long long i = 0; i < limit; i++) {
-        if (ld_acquire(p) >= v) return true;
-        __nanosleep(100);
+// Progress of a work item: the flag of (group, block) counts the slices whose
+// x and y outflow is written, and becomes ITEM_DONE once the z outflow is
+// too.  The block downwind in x or y sweeps its slice k as soon as slice k
+// upwind is there, so neighbours overlap instead of running one after the
+// other: with few items the time of an iteration is the longest chain of
+// slices, (blocks along x + blocks along y - 2) * every + nz, instead of
+// (stages) * bz.
+constexpr int ITEM_DONE = 1 << 30;
+// Lives in shared memory, used by thread 0 alone: in registers of every thread
+// it would cost the sweep loop its last free ones.
+struct Pipe {
+    const int *up_x, *up_y;  // flags of the upwind blocks (null: none)
+    int *own;                // this item's flag (null: never announced)
+    int have;                // slices known to be there upwind
+    int every;               // slices between announcements
+    int go;                  // no wait of this item has expired
+    long long limit;
+    int *error;
+    // Thread 0: wait until `need` slices are there upwind.  After an expired
+    // wait the error word is set and the item runs on without waiting or
+    // announcing (its results are discarded): an exit inside the slice loop
+    // costs the loop's code about 10%.
+    __device__ __forceinline__ void wait(int need)
+    {
+        if (have >= need) return;
+        int n = ITEM_DONE;
+        if (up_x) n = min(n, wait_count(up_x, need, limit));
+        if (n > 0 && up_y) n = min(n, wait_count(up_y, need, limit));
+        if (n < 0) {
+            atomicExch(error, 1);
+            go = 0;
+            own = nullptr;
+            n = ITEM_DONE;
+        }
+        have = n;
     }
-    return false;
-}
+    // Thread 0, after a barrier that follows the outflow stores of slice
+    // done - 1 (the last slice is announced with the z outflow).  The barrier
+    // and the release order every thread's stores before the flag.
+    __device__ __forceinline__ void announce(int done, int of) const
+    {
+        if (own && done < of && done % every == 0) st_release(own, done);
+    }
+};
 
-// Ordered accumulation of one item's moment partials.  Velocity group g of
-// an octant adds into accumulator k = g % nacc; the items of one (k, block)
+// Ordered accumulation of one item's moment partials.  Velocity group g (of
+// all groups) adds into accumulator k = g % nacc; the items of one (k, block)
 // form a chain in the order they were claimed, and the item at place `pos`
 // adds after the one at pos - 1 (the first one stores).  The order is fixed
 // by the work list, so the sums are bit-reproducible, and no item waits for
@@ -246,10 +282,10 @@ struct BlockSpan {
 
 // Before the chain wait: pull the block's accumulator records into L2.
 template <typename Real>
-__device__ void chain_prefetch(const SweepArgs &a, const BlockSpan &b, int vg)
+__device__ void chain_prefetch(const SweepArgs &a, const BlockSpan &b, int vgg)
 {
     const unsigned char *acc = static_cast<const unsigned char *>(a.acc) +
-                               (size_t)(vg % a.nacc) * a.ncell * a.acc_slots * 8;
+                               (size_t)(vgg % a.nacc) * a.ncell * a.acc_slots * 8;
     const int rec = a.acc_slots * 8;
     for (int r = threadIdx.x; r < b.ez * BY; r += NT) {  // one row of ex cells
         const int lj = r % BY, lk = r / BY;
@@ -263,7 +299,7 @@ __device__ void chain_prefetch(const SweepArgs &a, const BlockSpan &b, int vg)
 }
 
 template <typename Real>
-__device__ void chain_add(const SweepArgs &a, int o, int bxr, int byr, int bzr, int vg, int pos,
+__device__ void chain_add(const SweepArgs &a, int o, int bxr, int byr, int bzr, int vgg, int pos,
                           const void *scratch)
 {
     using Out = typename PartOut<Real>::T;
@@ -278,7 +314,7 @@ __device__ void chain_add(const SweepArgs &a, int o, int bxr, int byr, int bzr, 
         constexpr int VPC = NPART * 8 / 16;  // vectors per cell record
         constexpr int CH = 4;
         const V *sc = static_cast<const V *>(scratch);
-        V *acc = reinterpret_cast<V *>(static_cast<Out *>(a.acc) + (size_t)(vg % a.nacc) * ncell * ACC_COMPACT);
+        V *acc = reinterpret_cast<V *>(static_cast<Out *>(a.acc) + (size_t)(vgg % a.nacc) * ncell * ACC_COMPACT);
         const int n = b.ez * SLICE * VPC;
         for (int base = threadIdx.x; base < n; base += NT * CH) {
             V sv[CH], av[CH];
@@ -306,7 +342,7 @@ __device__ void chain_add(const SweepArgs &a, int o, int bxr, int byr, int bzr, 
     // ACC_SPLIT: the item's flux slots go to the slots of the sides ahead of
     // its octant; the first item of the chain stores zero on the other sides
     const Out *sc = static_cast<const Out *>(scratch);
-    Out *acc = static_cast<Out *>(a.acc) + (size_t)(vg % a.nacc) * ncell * ACC_SPLIT;
+    Out *acc = static_cast<Out *>(a.acc) + (size_t)(vgg % a.nacc) * ncell * ACC_SPLIT;
     const int n = b.ez * SLICE * NPART;
 #pragma unroll 4
     for (int e = threadIdx.x; e < n; e += NT) {
@@ -347,6 +383,7 @@ template <typename Real, typename Item>
 __device__ __forceinline__ void persistent_loop(const BatchSweepArgs &b, Item item_sweep)
 {
     __shared__ SweepArgs sa;
+    __shared__ Pipe pipe;
     __shared__ int s_item, s_go;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(b.counter, 1);
@@ -362,49 +399,50 @@ __device__ __forceinline__ void persistent_loop(const BatchSweepArgs &b, Item it
             int *dst = reinterpret_cast<int *>(&sa);
             for (int q = threadIdx.x; q < (int)(sizeof(SweepArgs) / sizeof(int)); q += NT) dst[q] = src[q];
         }
-        int *fl = b.flags + b.flag_off[inst];
         if (threadIdx.x == 0) {
             const SweepArgs &a = b.inst[inst];
             const int vgg = item.w;  // global velocity-group index within the instance
-            auto fidx = [&](int x, int y, int z) { return ((vgg * a.nbz + z) * a.nby + y) * a.nbx + x; };
+            int *own = b.flags + b.flag_off[inst] + ((vgg * a.nbz + bzr) * a.nby + byr) * a.nbx + bxr;
+            pipe.up_x = bxr > 0 ? own - 1 : nullptr;
+            pipe.up_y = byr > 0 ? own - a.nbx : nullptr;
+            pipe.own = it != b.skip_publish ? own : nullptr;
+            pipe.have = 0;
+            pipe.every = b.announce_every;
+            pipe.limit = b.spin_limit;
+            pipe.error = b.error;
             bool ok = *b.error == 0;
-            if (ok && bxr > 0) ok = wait_flag(fl + fidx(bxr - 1, byr, bzr), b.spin_limit);
-            if (ok && byr > 0) ok = wait_flag(fl + fidx(bxr, byr - 1, bzr), b.spin_limit);
-            if (ok && bzr > 0) ok = wait_flag(fl + fidx(bxr, byr, bzr - 1), b.spin_limit);
-            if (!ok) atomicExch(b.error, 1);
-            s_go = ok ? 1 : 0;
+            if (ok && bzr > 0) {
+                ok = wait_count(own - a.nbx * a.nby, ITEM_DONE, b.spin_limit) >= 0;
+                if (!ok) atomicExch(b.error, 1);
+            }
+            pipe.go = ok;
+            if (ok) pipe.wait(1);
         }
         __syncthreads();
-        if (!s_go) break;
+        if (!pipe.go) break;
         void *scratch = static_cast<unsigned char *>(b.scratch) + (size_t)blockIdx.x * b.scratch_stride;
-        item_sweep(sa, make_int4(o, bxr, byr, bzr), vg, scratch);
+        item_sweep(sa, make_int4(o, bxr, byr, bzr), vg, scratch, pipe);
         __syncthreads();
-        // the downwind blocks may start: the face planes are written
-        if (threadIdx.x == 0 && it != b.skip_publish) {
-            __threadfence();
-            const int vgg = item.w;
-            st_release(fl + ((vgg * sa.nbz + bzr) * sa.nby + byr) * sa.nbx + bxr, 1);
-        }
+        if (!pipe.go) break;
+        // the downwind blocks may finish: the face planes are written
+        if (threadIdx.x == 0 && pipe.own) st_release(pipe.own, ITEM_DONE);
         // then the item's turn in its accumulator chain
-        const int pos = b.pos[it];
+        const int pos = b.pos[it], vgg = item.w;
         const int bxi = (o & 1) ? bxr : sa.nbx - 1 - bxr;
         const int byi = (o & 2) ? byr : sa.nby - 1 - byr;
         const int bzi = (o & 4) ? bzr : sa.nbz - 1 - bzr;
-        int *tk = sa.tok + (((size_t)(vg % sa.nacc) * sa.nbz + bzi) * sa.nby + byi) * sa.nbx + bxi;
-        if (pos > 0) chain_prefetch<Real>(sa, BlockSpan(sa, o, bxr, byr, bzr), vg);
+        int *tk = sa.tok + (((size_t)(vgg % sa.nacc) * sa.nbz + bzi) * sa.nby + byi) * sa.nbx + bxi;
+        if (pos > 0) chain_prefetch<Real>(sa, BlockSpan(sa, o, bxr, byr, bzr), vgg);
         if (threadIdx.x == 0) {
-            bool ok = pos == 0 || wait_token(tk, pos, b.spin_limit);
+            bool ok = pos == 0 || wait_count(tk, pos, b.spin_limit) >= 0;
             if (!ok) atomicExch(b.error, 1);
             s_go = ok ? 1 : 0;
         }
         __syncthreads();
         if (!s_go) break;
-        chain_add<Real>(sa, o, bxr, byr, bzr, vg, pos, scratch);
+        chain_add<Real>(sa, o, bxr, byr, bzr, vgg, pos, scratch);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            st_release(tk, pos + 1);
-        }
+        if (threadIdx.x == 0) st_release(tk, pos + 1);
     }
 }
 

@@ -81,7 +81,7 @@ struct LineSums {
 
 struct Layout2 {
     static constexpr size_t off_coef = align16(sizeof(float2) * NPOS * CSP);
-    static constexpr size_t off_x = off_coef + align16(sizeof(float) * SLICE * NCOEF);
+    static constexpr size_t off_x = off_coef + sizeof(float) * SLICE * NCOEF;
     // x nodes of the octant (xi_x, its low part, w_x, -)
     __host__ __device__ static size_t off_cx(int nxm) { return off_x + sizeof(float4) * nxm; }
     // c_x tables of lines that do not have 16 nodes: [2][SLICE][cxs], an odd stride
@@ -96,6 +96,12 @@ struct Layout2 {
     }
 };
 
+// Barrier of the two warps that sum the two halves of the same 32 cells.
+__device__ __forceinline__ void pair_barrier()
+{
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x / 32) % 2) : "memory");
+}
+
 // One work item (see sweep_item of kgs_sweep.cu for the meaning of the
 // arguments and of the partials that it writes).
 //   LINE   16: every x-line has 16 slots, whose c_x stay in registers
@@ -103,7 +109,7 @@ struct Layout2 {
 //   DEV    the deviation-form source (uniform grids)
 template <int LINE, bool COHERENT, bool UNIF, bool DEV>
 __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, const int vgy, unsigned char *smem,
-                                            void *scratch)
+                                            void *scratch, Pipe *pipe)
 {
     static_assert(!DEV || UNIF, "the deviation-form source needs a uniform grid");
     const int nxm = a.nxo_max;
@@ -175,8 +181,7 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
         xi[0] = make_float2(p.x, q.x);
         xi[1] = make_float2(p.y, q.y);
         xi[2] = make_float2(p.z, q.z);
-        const double p0 = p.x, p1 = p.y, p2 = p.z, q0 = q.x, q1 = q.y, q2 = q.z;
-        xsq = make_float2((float)(p0 * p0 + p1 * p1 + p2 * p2), (float)(q0 * q0 + q1 * q1 + q2 * q2));
+        xsq = make_float2(velm[gv * 8 + 7], velm[gv * 8 + 15]);
         mref = make_float2(velm[gv * 8 + 5], velm[gv * 8 + 13]);
         if constexpr (DEV) dmref = make_float2(velm[gv * 8 + 6], velm[gv * 8 + 14]);
     }
@@ -208,8 +213,13 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
     const int tail = mn > 0 ? mn - head - full * nxo : 0;
     const int mline = mn > 0 ? (v0 + mb) / nxo - line0 : 0;  // line of its first velocity
 
+    // the persistent sweep reads the wall densities in FP32: converting them
+    // here would take a 64-cycle FP64-pipe instruction per value and warp
+    auto rho_wall = [&](int side, size_t cell) -> float {
+        return COHERENT ? a.rho_w32[side * ncell + cell] : (float)a.rho_w[side * ncell + cell];
+    };
     auto wall_rho = [&](int side, size_t cell) -> float {
-        return a.side_inflow[side] ? 1.f : (float)a.rho_w[side * ncell + cell];
+        return a.side_inflow[side] ? 1.f : rho_wall(side, cell);
     };
     auto ld2 = [](const float *p) { return ld_face<COHERENT>(reinterpret_cast<const float2 *>(p)); };
 
@@ -301,6 +311,7 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
 #pragma unroll
             for (int li = 0; li < BX; li++) slice[(HROW + li) * CSP + t] = phy[li];
         }
+        if (COHERENT && t == 0) pipe->wait(min(lk + 2, ez));
         __syncthreads();
         // c_x = xi_x - U_x of each cell of the slice as a float pair, per x slot
         if constexpr (LINE == 0) {
@@ -371,7 +382,10 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
             // The 15 diagonals unrolled: the upwind x and y values of a cell
             // were computed on the previous diagonal by this thread and stay
             // in registers (prev[row]); the z value (the cell itself in slice
-            // k - 1) and the halo come from shared memory.
+            // k - 1) and the halo come from shared memory.  A diagonal is
+            // stored once all its cells are computed: a store between them
+            // would keep the compiler from moving the next cell's shared
+            // loads above it (64^3 x 32^3: 19.7 -> 19.3 ms, cube 116 -> 113).
             float2 prev[BY];
 #pragma unroll
             for (int d = 0; d < BX + BY - 1; d++) {
@@ -380,13 +394,18 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
                     const int lj = (d < BY - 1 ? d : BY - 1) - k;
                     const int li = d - lj;
                     if (lj >= 0 && li < BX) {
-                        float2 *at = slice + (lj * BX + li) * CSP + t;
-                        const float2 fz = *at;
+                        const float2 fz = slice[(lj * BX + li) * CSP + t];
                         const float2 fx = li == 0 ? slice[(HCOL + lj) * CSP + t] : prev[lj];
                         const float2 fy = lj == 0 ? slice[(HROW + li) * CSP + t] : prev[lj > 0 ? lj - 1 : 0];
                         const float2 f = cell_update(cs + (lj * BX + li) * NCOEF, fx, fy, fz);
                         prev[lj] = f;
-                        if (ok) *at = f;
+                    }
+                }
+                if (ok) {
+#pragma unroll
+                    for (int k = 0; k < BY; k++) {
+                        const int lj = (d < BY - 1 ? d : BY - 1) - k, li = d - lj;
+                        if (lj >= 0 && li < BX) slice[(lj * BX + li) * CSP + t] = prev[lj];
                     }
                 }
             }
@@ -412,11 +431,11 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
                                 const size_t cell = CELL(GX(li), GY(lj), z);
                                 const float2 msol = row2(MT_SOLID);
                                 if (flags & (F_SOLID_SIDE << sidex))
-                                    fx = ghost((float)a.rho_w[sidex * ncell + cell], msol);
+                                    fx = ghost(rho_wall(sidex, cell), msol);
                                 if (flags & (F_SOLID_SIDE << sidey))
-                                    fy = ghost((float)a.rho_w[sidey * ncell + cell], msol);
+                                    fy = ghost(rho_wall(sidey, cell), msol);
                                 if (flags & (F_SOLID_SIDE << sidez))
-                                    fz = ghost((float)a.rho_w[sidez * ncell + cell], msol);
+                                    fz = ghost(rho_wall(sidez, cell), msol);
                             }
                             const float2 f = cell_update(c, fx, fy, fz);
                             if (ok) *at = f;
@@ -445,21 +464,24 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
                 *reinterpret_cast<float2 *>(fo + li * step) = slice[((ey - 1) * BX + li) * CSP + t];
             }
         }
+        // the moment phase's cell: read before the barrier that frees the staged record
+        const float *mc = cs + mcl * NCOEF;
+        const int mflags = flag_bits(mc[C_FLAGS]);
+        const float ux = -0.5f * mc[C_M2UX];
+        const float2 uyz = make_float2(-0.5f * mc[C_M2UY], -0.5f * mc[C_M2UZ]);
         __syncthreads();
+        if (COHERENT && t == 0) pipe->announce(lk + 1, ez);
 
         // ---- moments of the slice over the group's velocities ----
         {
             const int cl = mcl, vp = mvp;
             const int li = cl % BX, lj = cl / BX;
             const bool valid = li < ex && lj < ey;
-            const float *c = cs + cl * NCOEF;
-            const int flags = flag_bits(c[C_FLAGS]);
+            const int flags = mflags;
             // running sums in pairs of slots: (S0, S1x) (S1y, S1z) (S2yy, S2zz)
             // (S2xy, S2xz) (S2xx, S2yz) (S3y, S3z) (S3x, Fx) (Fy, Fz)
             KahanPair S[8];
             if (valid && !(flags & F_SOLID)) {
-                const float ux = -0.5f * c[C_M2UX];
-                const float2 uyz = make_float2(-0.5f * c[C_M2UY], -0.5f * c[C_M2UZ]);
                 const bool wx = flags & (F_WALL_SIDE << headx);
                 const bool wy = flags & (F_WALL_SIDE << heady);
                 const bool wz = flags & (F_WALL_SIDE << headz);
@@ -573,7 +595,7 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
 #pragma unroll
                 for (int q = 0; q < NPART; q++) red[q * SLICE + cl] = out[q];
             }
-            __syncthreads();
+            pair_barrier();
             if (vp == 0 && valid) {
                 float2 *pp = COHERENT ? static_cast<float2 *>(scratch) + ((size_t)lk * SLICE + cl) * NPART
                                       : static_cast<float2 *>(a.part) +
@@ -605,15 +627,15 @@ template <int LINE, bool UNIF>
 __global__ void __launch_bounds__(NT, 2) sweep2_staged_kernel(const SweepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    sweep_item2<LINE, false, UNIF, false>(a, a.work[blockIdx.x], blockIdx.y, smem, nullptr);
+    sweep_item2<LINE, false, UNIF, false>(a, a.work[blockIdx.x], blockIdx.y, smem, nullptr, nullptr);
 }
 
 template <int LINE, bool UNIF, bool DEV>
 __global__ void __launch_bounds__(NT, 2) sweep2_persistent_kernel(const BatchSweepArgs b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    persistent_loop<float>(b, [&](const SweepArgs &a, const int4 w, const int vg, void *scratch) {
-        sweep_item2<LINE, true, UNIF, DEV>(a, w, vg, smem, scratch);
+    persistent_loop<float>(b, [&](const SweepArgs &a, const int4 w, const int vg, void *scratch, Pipe &pipe) {
+        sweep_item2<LINE, true, UNIF, DEV>(a, w, vg, smem, scratch, &pipe);
     });
 }
 

@@ -231,6 +231,8 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
         t.velm64[g * 8 + 1] = vg->w_y[iy] * vg->w_z[iz];
         t.velm32[g * 8 + 0] = (float)vg->w_x[ix];
         t.velm32[g * 8 + 1] = (float)(vg->w_y[iy] * vg->w_z[iz]);
+        const double r0 = (float)t.vel64[g * 4], r1 = (float)t.vel64[g * 4 + 1], r2 = (float)t.vel64[g * 4 + 2];
+        t.velm32[g * 8 + 7] = (float)std::fma(r2, r2, std::fma(r1, r1, r0 * r0));
         for (int d = 0; d < 3; d++) {
             const double x = t.vel64[g * 4 + d];
             t.velm32[g * 8 + 2 + d] = (float)(x - (double)(float)x);
@@ -245,12 +247,11 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
         t.max_vg = std::max(t.max_vg, ng);
     }
     t.n_vg = (int)t.vg_oct.size();
-    // accumulators: velocity group g of an octant adds into g % nacc, and
-    // every accumulator must receive a group of every block, so nacc is at
-    // most the smallest group count of a non-empty octant
-    t.nacc = NACC_MAX;
-    for (int o = 0; o < 8; o++)
-        if (t.oct_vcount[o] > 0) t.nacc = std::min(t.nacc, t.groups(o));
+    // accumulators: velocity group g adds into g % nacc, so that each of them
+    // receives a group of every block.  Counting over all octants keeps the
+    // chains of small velocity grids short: with one or two groups per octant
+    // all eight octants would otherwise add one after the other.
+    t.nacc = std::max(1, std::min(NACC_MAX, t.n_vg));
 
     // ---- wall tables: kinds 0..5 domain sides, 6 solid surfaces ----
     double wallU[7][3], wallT[7];
