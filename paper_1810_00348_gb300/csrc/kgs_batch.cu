@@ -368,6 +368,20 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
     // persistent grid: as many CTAs as fit on the device at once
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess) return fail(KGS_ECUDA);
+    if (b->precision == KGS_FP64) {
+        // one kernel serves every instance: the separated sweep if all of
+        // them have their axis factors
+        SweepKind k = b->kind;
+        k.sep = 1;
+        bool all = sweep_persistent_occupancy(k, sweep_smem_bytes(k, b->nxo_max)) >= 1;
+        for (int i = 0; i < n && all; i++) {
+            const int rc = ctx_alloc_axis(b->ctx[i]);
+            if (rc) return fail(rc);
+            all = b->ctx[i]->ax_tab != nullptr;
+        }
+        for (int i = 0; i < n && !all; i++) ctx_free_axis(b->ctx[i]);
+        b->kind.sep = all;
+    }
     const size_t smem = sweep_smem_bytes(b->kind, b->nxo_max);
     per_sm = sweep_persistent_occupancy(b->kind, smem);
     if (per_sm < 1) return fail(KGS_ECUDA);

@@ -313,6 +313,31 @@ __global__ void __launch_bounds__(CLOSE_CELLS * NPART) part_sums_kernel(const Pa
     }
 }
 
+// The 13 sums about 0 -> the sums about U: c = xi - U expanded in each.
+__device__ __forceinline__ void shift_sums(double (&s)[SUM_F0], const double U[3])
+{
+    const double S0 = s[P_S0], S1[3] = {s[P_S1X], s[P_S1Y], s[P_S1Z]};
+    const double S2[3][3] = {{s[P_S2XX], s[P_S2XY], s[P_S2XZ]},
+                             {s[P_S2XY], s[P_S2YY], s[P_S2YZ]},
+                             {s[P_S2XZ], s[P_S2YZ], s[P_S2ZZ]}};
+    const double tr = S2[0][0] + S2[1][1] + S2[2][2];
+    const double U2 = U[0] * U[0] + U[1] * U[1] + U[2] * U[2];
+    const double US1 = U[0] * S1[0] + U[1] * S1[1] + U[2] * S1[2];
+    for (int i = 0; i < 3; i++) {
+        // (x_i - U_i) |x - U|^2 = x_i |x|^2 - 2 x_i U.x + x_i U^2 - U_i |x|^2 + 2 U_i U.x - U_i U^2
+        const double US2 = U[0] * S2[i][0] + U[1] * S2[i][1] + U[2] * S2[i][2];
+        s[P_S3X + i] = s[P_S3X + i] - 2.0 * US2 + U2 * S1[i] - U[i] * tr + 2.0 * U[i] * US1 - U[i] * U2 * S0;
+        s[P_S1X + i] = S1[i] - U[i] * S0;
+    }
+    auto c2 = [&](int i, int j) { return S2[i][j] - U[i] * S1[j] - U[j] * S1[i] + U[i] * U[j] * S0; };
+    s[P_S2XX] = c2(0, 0);
+    s[P_S2YY] = c2(1, 1);
+    s[P_S2ZZ] = c2(2, 2);
+    s[P_S2XY] = c2(0, 1);
+    s[P_S2XZ] = c2(0, 2);
+    s[P_S2YZ] = c2(1, 2);
+}
+
 // Per-cell sums of the persistent sweep's ordered accumulators, ACC_CELLS
 // cells per block.  First the block's (cell, slot) pairs in address order
 // (coalesced): each adds its slot's nacc accumulators in accumulator order
@@ -373,7 +398,15 @@ __global__ void __launch_bounds__(ACC_CELLS) acc_sums_kernel(const AccSumArgs a)
 #pragma unroll
         for (int q = 0; q < SUM_F0; q++) a.sums[(size_t)q * ncell + c] = tc[q] + ref[q];
     } else {
-        for (int q = 0; q < SUM_F0; q++) a.sums[(size_t)q * ncell + c] = tc[q];
+        double s[SUM_F0];
+        for (int q = 0; q < SUM_F0; q++) s[q] = tc[q];
+        if (a.raw) {
+            double U[3];
+            const double *cf = static_cast<const double *>(a.coef) + c * NCOEF;
+            for (int d = 0; d < 3; d++) U[d] = -0.5 * cf[C_M2UX + d];
+            shift_sums(s, U);
+        }
+        for (int q = 0; q < SUM_F0; q++) a.sums[(size_t)q * ncell + c] = s[q];
     }
 #pragma unroll
     for (int side = 0; side < 6; side++) {

@@ -26,6 +26,8 @@ struct kgs_ctx {
     double *mac = nullptr, *mac_new = nullptr, *rho_w = nullptr, *rho_w_new = nullptr;
     void *coef = nullptr, *vel = nullptr, *velm = nullptr, *mtab = nullptr, *FX = nullptr, *FY = nullptr,
          *FZ = nullptr;
+    void *ax_tab = nullptr;                               // separated FP64 sweep: axis factors (null: not used)
+    double *ax_nodes = nullptr;                           // HostTables::ax_nodes
     float *lines = nullptr, *xnodes = nullptr;            // packed FP32 sweep: HostTables::lines32, xnodes32
     float *rho_w32 = nullptr;                             // packed FP32 sweep: rho_w in FP32
     void *FX2 = nullptr, *FY2 = nullptr, *FZ2 = nullptr;  // second face planes of the order-2 sweep
@@ -84,6 +86,12 @@ void ctx_stage_items(const HostTables &t, int inst, int stage, std::vector<int4>
 // tokens, scratch, grid), or the staged sweep's partials if the persistent
 // kernel cannot be resident.
 int ctx_persist_init(kgs_ctx *c);
+// Kernel of a standalone context's sweep.
+SweepKind ctx_kind(const kgs_ctx *c);
+// Axis factors of the separated FP64 sweep; without the memory for them the
+// context keeps the sweep that needs none (ax_tab stays null).
+int ctx_alloc_axis(kgs_ctx *c);
+void ctx_free_axis(kgs_ctx *c);
 // Ordered accumulators of a context whose sweep runs persistent.
 int ctx_alloc_acc(kgs_ctx *c);
 // Chain tokens per (accumulator, block) of one instance.

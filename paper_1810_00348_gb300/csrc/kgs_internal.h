@@ -107,6 +107,10 @@ struct SweepArgs {
     const float *xnodes;          // packed: [8][xn_stride][4] xi_x, its low part, w_x
     int xn_stride;
     int oct_nx[8];                // x nodes in each octant (length of its velocity x-lines)
+    int oct_ny[8];                // y nodes in each octant (x-lines per velocity plane)
+    const void *ax_tab;           // separated FP64 sweep: double4[ncell][ax_n] axis factors (kgs_sweep_d.cu)
+    int ax_n, ax_nx, ax_ny;       // nodes of the three axes, of x and of y, in HostTables::ax_nodes order
+    int ax_neg[3];                // negative nodes of each axis (they come first)
     int nxo_max;                  // max over octants of oct_nx
     int any_solid;                // the problem has solid cells
     const uint8_t *blk_plain;     // [nbz][nby][nbx]: 1 = no solid cell and no solid neighbour in the block (or NULL)
@@ -211,6 +215,7 @@ struct SweepKind {
     int dev = 0;                  // first-order FP32 sweep with the deviation-form source (uniform grids)
     int pack = 0;                 // SweepArgs::pack: the packed FP32 kernel (kgs_sweep_f2.cu)
     int lines_max = 1;            // x-lines that a velocity group can touch, at most
+    int sep = 0;                  // first-order FP64 sweep with separated equilibria (kgs_sweep_d.cu)
 };
 // Persistent sweep.  Combinations that do not exist: 0 CTAs per SM /
 // cudaErrorInvalidValue.
@@ -221,6 +226,14 @@ int sweep_persistent_occupancy(const SweepKind &k, size_t smem);
 size_t sweep_smem_bytes(const SweepKind &k, int nxo_max);
 // Sweep launch (one wavefront stage, order 1, no deviation-form source).
 cudaError_t launch_sweep(const SweepKind &k, const SweepArgs &a, int n_items, int max_vg, cudaStream_t s);
+
+// The separated FP64 kernel (k.sep), reached through the functions above, and
+// the axis factors that it reads, from the FP64 cell coefficients.
+size_t sweep_d_smem_bytes(const SweepKind &k, int nxo_max);
+int sweep_d_occupancy(const SweepKind &k, size_t smem);
+cudaError_t launch_sweep_d(const SweepKind &k, const BatchSweepArgs &b, int nxo_max, int grid, cudaStream_t s);
+cudaError_t launch_axis_tables(const void *coef, const double *nodes, unsigned long long ncell, int nvx, int nvy,
+                               int na, void *tab, cudaStream_t s);
 
 // The packed FP32 kernels (k.pack), reached through the functions above.
 size_t sweep2_smem_bytes(const SweepKind &k, int nxo_max);
@@ -277,6 +290,7 @@ struct AccSumArgs {
     const void *acc;
     int nacc;
     int acc_slots;
+    int raw;                      // FP64: the accumulated sums are about 0, not about U^n
     unsigned long long ncell;
     const uint8_t *solid;         // [ncell] or NULL
     double *sums;                 // [NSUM][ncell]

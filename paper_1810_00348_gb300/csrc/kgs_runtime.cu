@@ -160,10 +160,16 @@ SweepArgs kgs::ctx_sweep_args(const kgs_ctx *c)
     for (int o = 0; o < 8; o++) {
         a.oct_nx[o] = t.oct_nx[o] > 0 ? t.oct_nx[o] : 1;
         a.oct_line0[o] = t.oct_line0[o];
+        a.oct_ny[o] = t.oct_ny[o];
     }
     a.lines = c->lines;
     a.xnodes = c->xnodes;
     a.xn_stride = t.xn_stride;
+    a.ax_tab = c->ax_tab;
+    a.ax_n = (int)t.ax_nodes.size();
+    a.ax_nx = t.ax_nx;
+    a.ax_ny = t.ax_ny;
+    for (int d = 0; d < 3; d++) a.ax_neg[d] = t.ax_neg[d];
     a.any_solid = t.any_solid ? 1 : 0;
     a.blk_plain = c->blk_plain;
     a.coef = c->coef;
@@ -196,7 +202,46 @@ int kgs::ctx_launch_coef(kgs_ctx *c)
     KGS_CHECK(launch_coef(t.precision, c->mac, c->solid, c->side_flags, c->rdx, c->rdy, c->rdz, t.nx, t.ny, t.nz,
                           t.mu_ref, t.omega, t.Pr, c->coef, c->stream, t.dev ? 1 : 0, c->rho_w, c->rho_w32));
     c->kernel_launches += 1;
+    if (c->ax_tab) {
+        KGS_CHECK(launch_axis_tables(c->coef, c->ax_nodes, t.ncell, t.ax_nx, t.ax_ny, (int)t.ax_nodes.size(),
+                                     c->ax_tab, c->stream));
+        c->kernel_launches += 1;
+    }
     return KGS_OK;
+}
+
+SweepKind kgs::ctx_kind(const kgs_ctx *c)
+{
+    SweepKind k = c->t.kind();
+    k.sep = c->ax_tab != nullptr;
+    return k;
+}
+
+int kgs::ctx_alloc_axis(kgs_ctx *c)
+{
+    const HostTables &t = c->t;
+    int rc = upload(c, &c->ax_nodes, t.ax_nodes);
+    if (!rc) rc = dalloc(c, &c->ax_tab, t.ncell * t.ax_nodes.size() * 4 * sizeof(double));
+    if (rc == KGS_ENOMEM) {
+        // the sweep that needs no axis factors serves a problem whose factors do not fit
+        (void)cudaGetLastError();
+        ctx_free_axis(c);
+        rc = KGS_OK;
+    }
+    return rc;
+}
+
+void kgs::ctx_free_axis(kgs_ctx *c)
+{
+    for (void *p : {static_cast<void *>(c->ax_nodes), c->ax_tab}) {
+        if (!p) continue;
+        c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
+        cudaFree(p);
+    }
+    if (c->ax_tab) c->device_bytes -= c->t.ncell * c->t.ax_nodes.size() * 4 * sizeof(double);
+    if (c->ax_nodes) c->device_bytes -= c->t.ax_nodes.size() * sizeof(double);
+    c->ax_tab = nullptr;
+    c->ax_nodes = nullptr;
 }
 
 int kgs::ctx_launch_stages(kgs_ctx *c)
@@ -228,7 +273,7 @@ int kgs::ctx_launch_stages(kgs_ctx *c)
         ba.announce_every = announce_every(t.precision, ba.n_items, c->persist_grid);
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[0], st));
         KGS_CHECK(
-            launch_sweep_persistent(t.kind(), ba, t.nxo_max, c->persist_grid, st));
+            launch_sweep_persistent(ctx_kind(c), ba, t.nxo_max, c->persist_grid, st));
         if (c->profiling) KGS_CHECK(cudaEventRecord(c->ev[1], st));
         c->kernel_launches += 1;
         c->sweep_launches += 1;
@@ -298,7 +343,13 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     const HostTables &t = c->t;
     int sms = 0;
     KGS_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
-    const SweepKind kind = t.kind();
+    if (t.precision == KGS_FP64 && t.order == 1) {
+        SweepKind k = t.kind();
+        k.sep = 1;
+        int rc;
+        if (sweep_persistent_occupancy(k, sweep_smem_bytes(k, t.nxo_max)) >= 1 && (rc = ctx_alloc_axis(c))) return rc;
+    }
+    const SweepKind kind = ctx_kind(c);
     const int per_sm = sweep_persistent_occupancy(kind, sweep_smem_bytes(kind, t.nxo_max));
     // the second-order sweep and the deviation-form source exist only in the
     // persistent kernel
@@ -336,6 +387,7 @@ int kgs::ctx_launch_sums(kgs_ctx *c)
         aa.acc = c->acc;
         aa.nacc = t.nacc;
         aa.acc_slots = t.acc_slots;
+        aa.raw = c->ax_tab != nullptr;
         aa.ncell = t.ncell;
         aa.solid = c->solid;
         aa.sums = c->sums;

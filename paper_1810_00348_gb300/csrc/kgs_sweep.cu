@@ -1051,9 +1051,10 @@ int occupancy_t(size_t smem)
     return n;
 }
 
-// Instantiation chosen at run time.  Two velocities per thread come here only
-// when the packed kernel does not apply (HostTables::pack = 0), with the
-// general moment loop.
+// Instantiation chosen at run time.  The first-order FP64 sweep comes here
+// only without the memory for its axis factors (k.sep = 0), two velocities per
+// thread only without packed slots (HostTables::pack = 0): both with the
+// general moment loop alone.
 template <template <typename, int, int, bool, int, bool> class F, typename... Args>
 auto dispatch(const SweepKind &k, Args &&...args)
 {
@@ -1068,9 +1069,6 @@ auto dispatch(const SweepKind &k, Args &&...args)
         return k.line16 ? F<float, 1, 16, true, 1, true>::run(args...) : F<float, 1, 0, true, 1, true>::run(args...);
     }
     if (k.precision == 0) {
-        if (k.line16)
-            return k.uniform ? F<double, 1, 16, true, 1, false>::run(args...)
-                             : F<double, 1, 16, false, 1, false>::run(args...);
         return k.uniform ? F<double, 1, 0, true, 1, false>::run(args...)
                          : F<double, 1, 0, false, 1, false>::run(args...);
     }
@@ -1107,6 +1105,7 @@ bool exists(const SweepKind &k)
 int sweep_persistent_occupancy(const SweepKind &k, size_t smem)
 {
     if (!exists(k)) return 0;
+    if (k.sep) return sweep_d_occupancy(k, smem);
     return k.pack ? sweep2_occupancy(k, smem) : dispatch<Occupancy>(k, smem);
 }
 
@@ -1114,17 +1113,19 @@ cudaError_t launch_sweep_persistent(const SweepKind &k, const BatchSweepArgs &b,
 {
     if (b.n_items == 0) return cudaSuccess;
     if (!exists(k)) return cudaErrorInvalidValue;
+    if (k.sep) return launch_sweep_d(k, b, nxo_max, grid, s);
     return k.pack ? launch_sweep2_persistent(k, b, nxo_max, grid, s) : dispatch<PersistentLaunch>(k, b, nxo_max, grid, s);
 }
 
 size_t sweep_smem_bytes(const SweepKind &k, int nxo_max)
 {
+    if (k.sep) return sweep_d_smem_bytes(k, nxo_max);
     if (k.pack) return sweep2_smem_bytes(k, nxo_max);
     const bool line = k.line16 != 0;
     if (k.order == 2)
         return k.precision == 0 ? SmemLayout<double, 1, 2>::total(nxo_max, line)
                                 : SmemLayout<float, 1, 2>::total(nxo_max, line);
-    if (k.precision == 0) return SmemLayout<double, 1>::total(nxo_max, line);
+    if (k.precision == 0) return SmemLayout<double, 1>::total(nxo_max, false);
     return k.tv == 2 ? SmemLayout<float, 2>::total(nxo_max, false) : SmemLayout<float, 1>::total(nxo_max, line);
 }
 

@@ -208,6 +208,21 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
             e += 4;
         }
     }
+    t.ax_nodes.clear();
+    t.ax_nx = t.nvx;
+    t.ax_ny = t.nvy;
+    const double *axis[3] = {vg->xi_x, vg->xi_y, vg->xi_z};
+    const int first[3] = {0, 0, t.vz0}, end[3] = {t.nvx, t.nvy, t.vz1};
+    for (int d = 0; d < 3; d++) {
+        t.ax_neg[d] = 0;
+        for (int sign = 0; sign < 2; sign++)
+            for (int i = first[d]; i < end[d]; i++)
+                if ((axis[d][i] >= 0.0) == (sign == 1)) {
+                    t.ax_nodes.push_back(axis[d][i]);
+                    t.ax_neg[d] += sign == 0;
+                }
+    }
+    for (int o = 0; o < 8; o++) t.oct_ny[o] = std::max(1, (o & 2) ? t.nvy - t.ax_neg[1] : t.ax_neg[1]);
     t.axis64.clear();
     t.axis64.insert(t.axis64.end(), vg->xi_x, vg->xi_x + t.nvx);
     t.axis64.insert(t.axis64.end(), vg->xi_y, vg->xi_y + t.nvy);

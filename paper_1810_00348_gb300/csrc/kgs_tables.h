@@ -44,6 +44,8 @@ struct HostTables {
     int acc_slots = ACC_COMPACT;             // ACC_SPLIT if a cell has walls on both sides along an axis
     std::vector<int> vg_oct;                 // octant of each velocity group
     std::vector<double> vel64;               // [Nvs][4] xi_x, xi_y, xi_z, w
+    std::vector<double> ax_nodes;            // nodes of the x, y and swept z axis, the negative ones of each first
+    int ax_nx = 0, ax_ny = 0, ax_neg[3] = {0, 0, 0}, oct_ny[8] = {0};
     std::vector<double> axis64;              // 1D nodes and weights: xi_x, xi_y, xi_z, w_x, w_y, w_z
     std::vector<double> velm64;              // [Nvs][8] w_x, w_y w_z, 0 ...
     std::vector<float> velm32;               // [Nvs][8] w_x, w_y w_z, low parts of xi
