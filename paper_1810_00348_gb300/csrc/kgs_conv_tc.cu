@@ -2,30 +2,32 @@
 // generation tensor cores (tcgen05.mma, accumulator in tensor memory).
 //
 // GEMM view: out[v][co] = sum over taps t and input channels ci of
-// in[v + off(t)][ci] W[t][co][ci].  A CTA owns an 8 (x) by 16 (y) patch of two
-// consecutive z-planes: two accumulators of M = 128 rows (voxels) each, all
-// output channels (N = cout_p <= 112), so every weight tile that reaches
-// shared memory feeds the MMAs of both planes.  The input planes z0 - 1 ..
-// z0 + 2 (10 x 18 voxels, all channels each) go through a ring of three
-// slots in the K-major no-swizzle layout the MMA reads: 16-byte rows (8
-// channels of one voxel), x fastest within a channel octet, so that for every
-// tap the 8 x positions of an output row segment are 8 consecutive 16-byte
-// rows (one 8 x 16 B core matrix) and the 16 y rows and the channel octets
-// are fixed strides.  Each tap is then C/16 MMAs of 128 x N x 16 per plane
-// reading shifted windows of the staged planes; no im2col copy is made.  The
-// planes move with cp.async: the first two before the pipeline starts, the
-// third and fourth by two loader warps while the tensor core works (the
-// fourth reuses the first's slot once the taps kz = 0 are done).  The
-// weights, packed beforehand so that a tap is one contiguous block in the
-// layout the MMA reads, move with one bulk copy per tap into a ring of four
-// buffers.  Two threads drive the pipeline without CTA-wide barriers: a
-// producer issues the copy of tap t once the MMAs of tap t-4 have released
-// its buffer (commit barrier), and an issuer starts the MMAs of tap t once
-// its copy has landed (transaction barrier); the remaining threads wait at a
-// CTA barrier, not polling, until the issuer has seen the last MMA complete.
-// The epilogue reads the accumulators with tcgen05.ld (warp w owns TMEM lanes
-// 32w..32w+31 = output rows) and applies bias + ReLU, bias only, or the ReLU
-// mask of the backward pass.
+// in[v + off(t)][ci] W[t][co][ci].  The unit of work is an 8 (x) by 16 (y)
+// patch of two consecutive z-planes: two accumulators of M = 128 rows (voxels)
+// each, all output channels (N = cout_p <= 112), so every weight tile that
+// reaches shared memory feeds the MMAs of both planes.  One CTA per SM takes a
+// contiguous range of units, z fastest, so that it marches up the columns of
+// the volume: of a unit's four input planes (10 x 18 voxels, all channels
+// each) the first two are the last two of the unit before.  The planes go
+// through a ring of three slots in the K-major no-swizzle layout the MMA
+// reads: 16-byte rows (8 channels of one voxel), x fastest within a channel
+// octet, so that for every tap the 8 x positions of an output row segment are
+// 8 consecutive 16-byte rows (one 8 x 16 B core matrix) and the 16 y rows and
+// the channel octets are fixed strides.  Each tap is then C/16 MMAs of 128 x N
+// x 16 per plane reading shifted windows of the staged planes; no im2col copy
+// is made.  The weights, packed beforehand so that a tap is one contiguous
+// block in the layout the MMA reads, move with one bulk copy per tap into a
+// ring of four buffers.
+//
+// The warps have one role each, joined by barriers per slot and no CTA-wide
+// ones: a producer issues the weight copies, an issuer the MMAs, five warps
+// copy planes (cp.async, a slot ahead), and four warps read the accumulators
+// of the previous unit with tcgen05.ld (two sets take turns in tensor memory)
+// and apply bias + ReLU, bias only, or the ReLU mask of the backward pass.
+// What bounds it: the tensor core's reads of the shifted windows (their core
+// matrices straddle two 128-byte lines) at about 90 cycles per MMA instead of
+// 56.  With a CTA per unit, which loaded its first planes before and read its
+// accumulators after its MMAs, a unit took 65000 cycles for 378 MMAs.
 //
 // The weight gradient (wgrad_tc_kernel) is the per-tap GEMM dW[t][co][ci] =
 // sum over voxels v of dy[v][co] in[v + off(t)][ci], with the output
@@ -38,10 +40,8 @@
 // that share (kz, ky): three accumulators in tensor memory, and per 8 x 16
 // voxel tile one staged dy tile plus one 16 x 10 voxel block of input plane
 // z + kz - 1 whose x windows at offsets 0, 1, 2 are the three B operands.
-// Three tile buffers rotate (the copies of tile i + 2 in flight while the
-// MMAs of tile i run), each released by its commit barrier.  A CTA covers a
-// chunk of tiles of one sample and writes its partial; the caller sums the
-// partials in a fixed order.
+// A CTA covers a chunk of tiles of one sample and writes its partial; the
+// caller sums the partials in a fixed order.
 //
 // Every wait on a barrier is bounded; on expiry the CTA records the error,
 // waits (bounded) for its own MMAs, frees its tensor memory and returns.
@@ -56,11 +56,12 @@ namespace {
 
 constexpr int TX = 8, TY = 16;                 // output patch: 128 voxels = 128 GEMM rows
 constexpr int HX = TX + 2, HY = TY + 2, HZ = 3;  // input plane of the patch; ring of HZ plane slots
-constexpr int THREADS = 128;
-constexpr int OZ = 2;                          // output planes per CTA (two accumulators)
+constexpr int OZ = 2;                          // output planes per step (two accumulators)
 constexpr int TMEM_HALF = 128;                 // columns of one accumulator (>= N)
-constexpr int TMEM_COLS = OZ * TMEM_HALF;      // a power of two
-constexpr int LOADERS = 64;                    // threads that stream the later input planes
+constexpr int TMEM_COLS = 2 * OZ * TMEM_HALF;  // two pairs in turn; a power of two
+constexpr int FIRST_LOADER = 6;                // warps: producer, issuer, four of the epilogue, then the loaders
+constexpr int LOADERS = 160;                   // threads that load input planes: a row of 10 x 14 pieces at least
+constexpr int THREADS = FIRST_LOADER * 32 + LOADERS;
 constexpr int NBUF = 4;                        // weight buffers: up to four taps in flight
 constexpr long long WAIT_POLLS = 1ll << 20;    // try_wait polls before giving up
 
@@ -179,66 +180,60 @@ __global__ void pack_w_kernel(const uint4 *__restrict__ w, int cout_p, int c8n, 
     wpk[t * per + (size_t)c8 * cout_p + co] = w[i];
 }
 
-template <int MODE>
+// RES: the weights of all 27 taps fit beside the planes and are copied once
+// per CTA; otherwise they stream through the ring, once per unit.
+template <int MODE, bool RES>
 __global__ void __launch_bounds__(THREADS, 1)
     conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__restrict__ wpk,
                    const float *__restrict__ bias, void *out, const __nv_bfloat16 *__restrict__ gate, ConvDims dm,
                    int *err)
 {
     extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ __align__(8) uint64_t full_bar[NBUF], empty_bar[NBUF], done_bar, plane_full[2], plane_empty;
+    __shared__ __align__(8) uint64_t full_bar[NBUF], empty_bar[NBUF], plane_full[HZ], plane_empty[HZ], acc_full[2],
+        acc_empty[2], done_bar;
     __shared__ uint32_t tmem_base;
-    __shared__ int s_fail, s_last;  // a wait gave up; last tap whose MMAs were committed
+    __shared__ int s_fail, s_last;  // a wait gave up; last weight copy whose MMAs were committed
 
     const int C8 = dm.cin_p / 8, cout_p = dm.cout_p;
     const uint32_t plane_bytes = (uint32_t)HY * C8 * HX * 16;
     const uint32_t w_bytes = (uint32_t)C8 * cout_p * 16;
-    unsigned char *wbuf = sm + HZ * plane_bytes;
-    const int tiles_x = (dm.W + TX - 1) / TX;
-    const int x0 = (blockIdx.x % tiles_x) * TX, y0 = (blockIdx.x / tiles_x) * TY;
-    const int z0 = blockIdx.y * OZ, b = blockIdx.z;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    auto full = [&](int t) { return smem_u32(&full_bar[t % NBUF]); };    // weights of tap t landed
-    auto empty = [&](int t) { return smem_u32(&empty_bar[t % NBUF]); };  // MMAs of tap t done
-    auto use = [](int t) { return (uint32_t)((t / NBUF) & 1); };         // phase parity of tap t's use
-    const uint32_t halo_a = smem_u32(sm), w_a = smem_u32(wbuf);
-    volatile int *fail = &s_fail;  // written by the pipeline threads
-    auto issue_w = [&](int t) {  // bulk copy of tap t into buffer t % NBUF
-        mbar_expect_tx(full(t), w_bytes);
-        bulk_copy(w_a + (uint32_t)(t % NBUF) * w_bytes, wpk + (size_t)t * cout_p * dm.cin_p, w_bytes, full(t));
-    };
-    // input plane p (z = z0 - 1 + p, p = 0..3) in slot p % 3: element (hx, hy,
-    // channel octet c8) at ((hy * C8 + c8) * HX + hx) * 16
+    const int tiles_x = (dm.W + TX - 1) / TX, tiles = tiles_x * ((dm.H + TY - 1) / TY);
+    const int pairs = (dm.D + OZ - 1) / OZ;  // plane pairs of a column (one patch of one sample)
+    const long long units = (long long)dm.B * tiles * pairs;
+    const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+    const int n_pairs = (int)(u1 - u0);
     const size_t vol = (size_t)dm.D * dm.H * dm.W;
-    auto load_plane = [&](int p, int first, int stride) {
-        const int gz = z0 - 1 + p;
-        const uint32_t dst = halo_a + (uint32_t)(p % HZ) * plane_bytes;
-        for (int i = first; i < HY * HX * C8; i += stride) {
-            const int c8 = i % C8, r = i / C8;
-            const int hx = r % HX, hy = r / HX;
-            const int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
-            const bool valid = gx >= 0 && gy >= 0 && gz >= 0 && gx < dm.W && gy < dm.H && gz < dm.D;
-            const __nv_bfloat16 *src =
-                valid ? in + ((size_t)b * vol + ((size_t)gz * dm.H + gy) * dm.W + gx) * dm.cin_p + c8 * 8 : in;
-            cp_async16(dst + (uint32_t)((hy * C8 + c8) * HX + hx) * 16, src, valid);
-        }
-        cp_async_commit();
-    };
+    const int t = threadIdx.x, warp = t / 32, lane = t % 32;
+    const uint32_t halo_a = smem_u32(sm), w_a = halo_a + HZ * plane_bytes;
+    volatile int *fail = &s_fail;  // written by the pipeline threads
+    // weight copy T (pair T / 27 of this CTA, tap T % 27) goes through ring slot T % NBUF
+    auto full = [&](int T) { return smem_u32(&full_bar[T % NBUF]); };    // weights landed
+    auto empty = [&](int T) { return smem_u32(&empty_bar[T % NBUF]); };  // MMAs done
+    auto use = [](int T) { return (uint32_t)((T / NBUF) & 1); };         // phase parity
+    // plane n of this CTA's sequence goes through slot n % HZ
+    auto pfull = [&](int n) { return smem_u32(&plane_full[n % HZ]); };
+    auto pempty = [&](int n) { return smem_u32(&plane_empty[n % HZ]); };
+    auto puse = [](int n) { return (uint32_t)((n / HZ) & 1); };
+    // the pair starts a column: its four planes are new (else the last two of the pair before come first)
+    auto fresh = [&](long long u) { return u == u0 || u % pairs == 0; };
 
-    if (threadIdx.x == 0) {
+    if (t == 0) {
         for (int q = 0; q < NBUF; q++) {
             mbar_init(smem_u32(&full_bar[q]), 1);
             mbar_init(smem_u32(&empty_bar[q]), 1);
         }
+        for (int q = 0; q < HZ; q++) {
+            mbar_init(smem_u32(&plane_full[q]), LOADERS);
+            mbar_init(smem_u32(&plane_empty[q]), 1);
+        }
+        for (int q = 0; q < 2; q++) {
+            mbar_init(smem_u32(&acc_full[q]), 1);
+            mbar_init(smem_u32(&acc_empty[q]), 128);
+        }
         mbar_init(smem_u32(&done_bar), 1);
-        mbar_init(smem_u32(&plane_full[0]), LOADERS);
-        mbar_init(smem_u32(&plane_full[1]), LOADERS);
-        mbar_init(smem_u32(&plane_empty), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_fail = 0;
         s_last = -1;
-        // the first NBUF taps need no free buffer: start them now
-        for (int t = 0; t < NBUF; t++) issue_w(t);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -246,132 +241,217 @@ __global__ void __launch_bounds__(THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // the first two input planes, by every thread
-    load_plane(0, threadIdx.x, THREADS);
-    load_plane(1, threadIdx.x, THREADS);
-    cp_async_wait<0>();
-    fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    int issued = -1;  // last weight copy issued (thread 0)
 
-    int issued = NBUF - 1;  // last tap whose weight copy was issued (thread 0)
-    if (threadIdx.x == 0) {
-        // producer: tap t reuses the buffer of tap t - NBUF once its MMAs are done
-        for (int t = NBUF; t < 27; t++) {
-            if (*fail || !mbar_wait(empty(t - NBUF), use(t - NBUF))) {
+    if (t == 0 && RES) {
+        mbar_expect_tx(smem_u32(&full_bar[0]), 27 * w_bytes);
+        for (int tap = 0; tap < 27; tap++)
+            bulk_copy(w_a + (uint32_t)tap * w_bytes, wpk + (size_t)tap * cout_p * dm.cin_p, w_bytes,
+                      smem_u32(&full_bar[0]));
+        issued = 0;
+    } else if (t == 0) {
+        // weight producer: copy T reuses the slot of copy T - NBUF once its MMAs are done
+        for (int T = 0; T < 27 * n_pairs; T++) {
+            if (*fail || (T >= NBUF && !mbar_wait(empty(T - NBUF), use(T - NBUF)))) {
                 *fail = 1;
                 break;
             }
-            issue_w(t);
-            issued = t;
+            mbar_expect_tx(full(T), w_bytes);
+            bulk_copy(w_a + (uint32_t)(T % NBUF) * w_bytes, wpk + (size_t)(T % 27) * cout_p * dm.cin_p, w_bytes, full(T));
+            issued = T;
         }
-    } else if (threadIdx.x == 32) {
+    } else if (t == 32) {
         // MMA issuer: per tap and channel pair, one MMA of 128 x N x 16 for
-        // each output plane, both reading the same weights
-        const uint32_t tmem = tmem_base;
+        // each output plane, both reading the same weights.  The thread's own
+        // instruction latency sets the pace of small layers, so descriptors
+        // advance by additions (their address field counts 16-byte units) and
+        // ring slots by counters: with both formed anew for every MMA a step
+        // of two MMAs took 300 cycles whatever its size.
         const uint32_t idesc = instr_desc(128, cout_p);
-        const uint32_t a_lbo = HX * 16, a_sbo = (uint32_t)C8 * HX * 16;
-        const uint32_t b_lbo = (uint32_t)cout_p * 16, b_sbo = 8 * 16;
-        for (int t = 0; t < 27; t++) {
-            const int kx = t % 3, ky = (t / 3) % 3, kz = t / 9;
-            // plane kz + 1 (for the second output plane) first used by the taps kz
-            bool ok = !*fail;
-            if (ok && t == 9) ok = mbar_wait(smem_u32(&plane_full[0]), 0);
-            if (ok && t == 18) ok = mbar_wait(smem_u32(&plane_full[1]), 0);
-            if (!ok || !mbar_wait(full(t), use(t))) {
+        const uint64_t a_desc = smem_desc(0, HX * 16, (uint32_t)C8 * HX * 16), a_kc = 2 * HX;
+        const uint64_t b_desc = smem_desc(0, (uint32_t)cout_p * 16, 8 * 16), b_kc = 2 * (uint32_t)cout_p;
+        const uint32_t halo16 = halo_a >> 4, plane16 = plane_bytes >> 4, row16 = (uint32_t)C8 * HX;
+        const int KC = C8 / 2;
+        int n0 = 0;                   // first plane of the pair: planes n0 .. n0 + 3
+        int T = 0, slot = 0;          // weight copy (RES: tap), its ring slot
+        uint32_t phase = 0;
+        bool ok = true;
+        if (RES) {
+            ok = mbar_wait(smem_u32(&full_bar[0]), 0);
+            if (ok) s_last = 0;
+        }
+        for (int j = 0; j < n_pairs && ok; j++) {
+            if (j > 0) n0 += fresh(u0 + j) ? 4 : 2;
+            const bool end = j + 1 == n_pairs || fresh(u0 + j + 1);  // the column ends here
+            const uint32_t acc = tmem + (uint32_t)((j & 1) * OZ * TMEM_HALF);
+            // the accumulators of pair j - 2 have been read
+            if (j >= 2) ok = mbar_wait(smem_u32(&acc_empty[j & 1]), (uint32_t)((j - 2) / 2 & 1));
+            ok = ok && mbar_wait(pfull(n0), puse(n0));
+            uint32_t first = 0;  // the pair's first MMA overwrites its accumulator
+            for (int kz = 0; kz < 3 && ok; kz++) {
+                ok = !*fail && mbar_wait(pfull(n0 + kz + 1), puse(n0 + kz + 1));
+                tc_fence_after();
+                const uint64_t pa0 = a_desc + halo16 + (uint32_t)((n0 + kz) % HZ) * plane16;      // output z0
+                const uint64_t pa1 = a_desc + halo16 + (uint32_t)((n0 + kz + 1) % HZ) * plane16;  // output z0 + 1
+                for (int ky = 0; ky < 3 && ok; ky++)
+                    for (int kx = 0; kx < 3; kx++) {
+                        if (!RES) {
+                            if (!ok || *fail || !mbar_wait(smem_u32(&full_bar[slot]), phase)) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                        }
+                        uint64_t d0 = pa0 + (uint32_t)ky * row16 + kx, d1 = pa1 + (uint32_t)ky * row16 + kx;
+                        uint64_t bd = b_desc + ((w_a + (uint32_t)(RES ? 9 * kz + 3 * ky + kx : slot) * w_bytes) >> 4);
+                        for (int kc = 0; kc < KC; kc++) {
+                            tc_mma(acc, d0, bd, idesc, first);
+                            tc_mma(acc + TMEM_HALF, d1, bd, idesc, first);
+                            first = 1;
+                            d0 += a_kc;
+                            d1 += a_kc;
+                            bd += b_kc;
+                        }
+                        if (!RES) {
+                            tc_commit(smem_u32(&empty_bar[slot]));
+                            s_last = T++;
+                            if (++slot == NBUF) slot = 0, phase ^= 1;
+                        }
+                    }
+                if (!ok) break;
+                // planes that no later MMA reads
+                if (kz < 2) {
+                    tc_commit(pempty(n0 + kz));
+                } else if (end) {
+                    tc_commit(pempty(n0 + 2));
+                    tc_commit(pempty(n0 + 3));
+                }
+            }
+            if (ok) tc_commit(smem_u32(&acc_full[j & 1]));
+        }
+        if (!ok) *fail = 1;
+        // all MMAs of the CTA are complete once the done barrier has fired
+        tc_commit(smem_u32(&done_bar));
+        if (!mbar_wait(smem_u32(&done_bar), 0)) *fail = 1;
+    } else if (warp >= FIRST_LOADER) {
+        // loaders: a thread keeps its (x, channel octet) and walks down the
+        // rows of a plane; whole rows per pass
+        const int lt = t - FIRST_LOADER * 32, per = HX * C8, rows = LOADERS / per;
+        const int r0 = lt / per, c8 = lt % per / HX, px = lt % HX;  // x fastest: conflict-free stores
+        const bool idle = r0 >= rows;
+        int n = 0;
+        bool ok = true;
+        auto load = [&](long long u, int p) {  // plane z0 - 1 + p of unit u as plane n
+            const long long col = u / pairs;
+            const int patch = (int)(col % tiles), b = (int)(col / tiles);
+            const int z = (int)(u % pairs) * OZ - 1 + p;
+            const int x = patch % tiles_x * TX - 1 + px, y = patch / tiles_x * TY - 1 + r0;
+            if (idle) return;
+            const bool plane = x >= 0 && x < dm.W && z >= 0 && z < dm.D;
+            const __nv_bfloat16 *src =
+                in + ((long long)b * (long long)vol + ((long long)z * dm.H + y) * dm.W + x) * dm.cin_p + c8 * 8;
+            uint32_t dst = halo_a + (uint32_t)(n % HZ) * plane_bytes + (uint32_t)((r0 * C8 + c8) * HX + px) * 16;
+            for (int r = r0, yy = y; r < HY; r += rows, yy += rows) {
+                const bool in_y = plane && yy >= 0 && yy < dm.H;
+                cp_async16(dst, in_y ? src : in, in_y);
+                src += (long long)rows * dm.W * dm.cin_p;
+                dst += (uint32_t)(rows * C8 * HX) * 16;
+            }
+        };
+        for (long long u = u0; u < u1 && ok; u++) {
+            for (int p = fresh(u) ? 0 : 2; p < 4; p++, n++) {
+                // plane n reuses the slot of plane n - HZ once no MMA reads it
+                if (n >= HZ && (*fail || !mbar_wait(pempty(n - HZ), puse(n - HZ)))) {
+                    *fail = 1;  // the issuer's wait on this plane then gives up too
+                    ok = false;
+                    break;
+                }
+                load(u, p);
+                cp_async_commit();
+                // the first HZ planes are issued together, the later ones one per nine taps
+                if (n < HZ - 1) continue;
+                if (n == HZ - 1) {
+                    static_assert(HZ == 3, "two planes are outstanding before this one");
+                    cp_async_wait<2>();
+                    fence_async_smem();
+                    mbar_arrive(pfull(0));
+                    cp_async_wait<1>();
+                    fence_async_smem();
+                    mbar_arrive(pfull(1));
+                }
+                cp_async_wait<0>();
+                fence_async_smem();
+                mbar_arrive(pfull(n));
+            }
+        }
+        cp_async_wait<0>();
+    } else if (warp >= 2) {
+        // epilogue warps 2 .. 5: warp w reads the TMEM lanes 32 (w % 4) ..
+        // (output rows) while the MMAs of the next pair run
+        const int quad = warp % 4, row = quad * 32 + lane;
+        for (int j = 0; j < n_pairs; j++) {
+            if (*fail || !mbar_wait(smem_u32(&acc_full[j & 1]), (uint32_t)(j / 2 & 1))) {
                 *fail = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t pa0 = halo_a + (uint32_t)(kz % HZ) * plane_bytes;        // plane kz: output z0
-            const uint32_t pa1 = halo_a + (uint32_t)((kz + 1) % HZ) * plane_bytes;  // plane kz + 1: output z0 + 1
-            for (int kc = 0; kc < C8 / 2; kc++) {
-                const uint32_t off = (uint32_t)(((ky * C8 + 2 * kc) * HX + kx) * 16);
-                const uint64_t bd =
-                    smem_desc(w_a + (uint32_t)(t % NBUF) * w_bytes + (uint32_t)(2 * kc * cout_p * 16), b_lbo, b_sbo);
-                tc_mma(tmem, smem_desc(pa0 + off, a_lbo, a_sbo), bd, idesc, (t | kc) != 0);
-                tc_mma(tmem + TMEM_HALF, smem_desc(pa1 + off, a_lbo, a_sbo), bd, idesc, (t | kc) != 0);
-            }
-            tc_commit(empty(t));
-            if (t == 8) tc_commit(smem_u32(&plane_empty));  // plane 0 (slot 0) no longer read
-            s_last = t;
-        }
-        tc_commit(smem_u32(&done_bar));  // all MMAs issued by this thread
-        // all MMAs of the CTA are complete once the done barrier has fired.
-        // Only this thread waits for it; the others are parked at the CTA
-        // barrier below instead of polling beside the pipeline threads.
-        if (!mbar_wait(smem_u32(&done_bar), 0)) *fail = 1;
-    } else if (threadIdx.x >= THREADS - LOADERS) {
-        // loaders: plane 2 into slot 2 now, plane 3 into slot 0 once the MMAs
-        // of the taps kz = 0 have released plane 0
-        const int lt = threadIdx.x - (THREADS - LOADERS);
-        load_plane(2, lt, LOADERS);
-        cp_async_wait<0>();
-        fence_async_smem();
-        mbar_arrive(smem_u32(&plane_full[0]));
-        if (mbar_wait(smem_u32(&plane_empty), 0)) {
-            load_plane(3, lt, LOADERS);
-            cp_async_wait<0>();
-            fence_async_smem();
-        } else {
-            *fail = 1;  // the issuer's wait on plane_full[1] then gives up too
-        }
-        mbar_arrive(smem_u32(&plane_full[1]));
-    }
-    __syncthreads();  // the outcome in s_fail / s_last is uniform after it
-    const int last = s_last;
-    const uint32_t tmem = tmem_base;
-    tc_fence_after();
-    if (s_fail || last != 26) {
-        if (threadIdx.x == 0) {
-            atomicExch(err, 1);
-            // weight copies issued but never consumed land before the CTA
-            // leaves (bounded; at most NBUF are outstanding, on distinct barriers)
-            for (int t = last + 1; t <= issued; t++) (void)mbar_wait(full(t), use(t));
-        }
-    } else {
-        const int row = warp * 32 + lane;
-        const int vx = x0 + row % TX, vy = y0 + row / TX;
-        const bool inside = vx < dm.W && vy < dm.H;
-        for (int oz = 0; oz < OZ; oz++) {
-            const int z = z0 + oz;
-            if (z >= dm.D) break;  // uniform over the CTA
-            const size_t vo = (size_t)b * vol + ((size_t)z * dm.H + vy) * dm.W + vx;
-            for (int c0 = 0; c0 < cout_p; c0 += 16) {
-                float v[16];
-                tc_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(oz * TMEM_HALF + c0), v);  // all lanes
-                if (!inside) continue;
-                if (MODE == 1) {
-                    float *o = static_cast<float *>(out) + vo * cout_p + c0;
+            const long long u = u0 + j, col = u / pairs;
+            const int patch = (int)(col % tiles), b = (int)(col / tiles), z0 = (int)(u % pairs) * OZ;
+            const int vx = patch % tiles_x * TX + row % TX, vy = patch / tiles_x * TY + row / TX;
+            const bool inside = vx < dm.W && vy < dm.H;
+            const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((j & 1) * OZ * TMEM_HALF);
+            for (int oz = 0; oz < OZ; oz++) {
+                const int z = z0 + oz;
+                if (z >= dm.D) break;  // uniform over the CTA
+                const size_t vo = (size_t)b * vol + ((size_t)z * dm.H + vy) * dm.W + vx;
+                for (int c0 = 0; c0 < cout_p; c0 += 16) {
+                    float v[16];
+                    tc_ld16(acc + (uint32_t)(oz * TMEM_HALF + c0), v);  // all lanes
+                    if (!inside) continue;
+                    if (MODE == 1) {
+                        float *o = static_cast<float *>(out) + vo * cout_p + c0;
 #pragma unroll
-                    for (int i = 0; i < 16; i += 4)
-                        *reinterpret_cast<float4 *>(o + i) =
-                            make_float4(v[i] + bias[c0 + i], v[i + 1] + bias[c0 + i + 1], v[i + 2] + bias[c0 + i + 2],
-                                        v[i + 3] + bias[c0 + i + 3]);
-                } else {
-                    __align__(16) __nv_bfloat162 h[8];
-                    if (MODE == 0) {
-#pragma unroll
-                        for (int i = 0; i < 8; i++)
-                            h[i] = __floats2bfloat162_rn(fmaxf(v[2 * i] + bias[c0 + 2 * i], 0.f),
-                                                         fmaxf(v[2 * i + 1] + bias[c0 + 2 * i + 1], 0.f));
+                        for (int i = 0; i < 16; i += 4)
+                            *reinterpret_cast<float4 *>(o + i) =
+                                make_float4(v[i] + bias[c0 + i], v[i + 1] + bias[c0 + i + 1],
+                                            v[i + 2] + bias[c0 + i + 2], v[i + 3] + bias[c0 + i + 3]);
                     } else {
-                        __align__(16) __nv_bfloat162 g[8];
-                        const uint4 *gp = reinterpret_cast<const uint4 *>(gate + vo * cout_p + c0);
-                        reinterpret_cast<uint4 *>(g)[0] = gp[0];
-                        reinterpret_cast<uint4 *>(g)[1] = gp[1];
+                        __align__(16) __nv_bfloat162 h[8];
+                        if (MODE == 0) {
 #pragma unroll
-                        for (int i = 0; i < 8; i++)
-                            h[i] = __floats2bfloat162_rn(__bfloat162float(g[i].x) > 0.f ? v[2 * i] : 0.f,
-                                                         __bfloat162float(g[i].y) > 0.f ? v[2 * i + 1] : 0.f);
+                            for (int i = 0; i < 8; i++)
+                                h[i] = __floats2bfloat162_rn(fmaxf(v[2 * i] + bias[c0 + 2 * i], 0.f),
+                                                             fmaxf(v[2 * i + 1] + bias[c0 + 2 * i + 1], 0.f));
+                        } else {
+                            __align__(16) __nv_bfloat162 g[8];
+                            const uint4 *gp = reinterpret_cast<const uint4 *>(gate + vo * cout_p + c0);
+                            reinterpret_cast<uint4 *>(g)[0] = gp[0];
+                            reinterpret_cast<uint4 *>(g)[1] = gp[1];
+#pragma unroll
+                            for (int i = 0; i < 8; i++)
+                                h[i] = __floats2bfloat162_rn(__bfloat162float(g[i].x) > 0.f ? v[2 * i] : 0.f,
+                                                             __bfloat162float(g[i].y) > 0.f ? v[2 * i + 1] : 0.f);
+                        }
+                        uint4 *o = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(out) + vo * cout_p + c0);
+                        o[0] = reinterpret_cast<uint4 *>(h)[0];
+                        o[1] = reinterpret_cast<uint4 *>(h)[1];
                     }
-                    uint4 *o = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(out) + vo * cout_p + c0);
-                    o[0] = reinterpret_cast<uint4 *>(h)[0];
-                    o[1] = reinterpret_cast<uint4 *>(h)[1];
                 }
             }
+            tc_fence_before();
+            mbar_arrive(smem_u32(&acc_empty[j & 1]));
         }
+    }
+    __syncthreads();  // the pipeline has ended; the outcome in s_fail is uniform after it
+    if (t == 0 && s_fail) {
+        atomicExch(err, 1);
+        // weight copies issued but never consumed land before the CTA
+        // leaves (bounded; at most NBUF are outstanding, on distinct barriers)
+        for (int T = s_last + 1; T <= issued; T++) (void)mbar_wait(full(T), use(T));
     }
     tc_fence_before();
     __syncthreads();
@@ -393,11 +473,32 @@ __global__ void __launch_bounds__(THREADS, 1)
 // tile it stages dy of the tile, [y][co/8][x][16 B], and rows y0 + ky - 1 ..
 // y0 + ky + 14, columns x0 - 1 .. x0 + 8 of input plane z + kz - 1,
 // [y][ci/8][x][16 B]; the windows of that block at x offsets 0, 1, 2 are the
-// B operands of the three taps.  Three tile buffers rotate: the copies of
-// tile i + 2 are in flight while the tensor core works on tile i.
-constexpr int WG_TILES = 32;  // voxel tiles of 128 per CTA
-constexpr int WG_BUF = 3;     // tile buffers
-constexpr int WG_TMEM = 512;  // three accumulators of 128 columns
+// B operands of the three taps.
+//
+// What bounds it: per tile the tensor core needs about 2000 cycles (24 MMAs of
+// 128 x 112 x 16, whose x-shifted windows read two 128-byte lines per core
+// matrix) and the copies bring 64 KB.  Eight warps only copy and one thread
+// only issues MMAs, through barriers per tile buffer, so neither waits for
+// the other beyond the three buffers.  A copying thread keeps its (x, channel
+// octet) from tile to tile and walks down the rows by adding one stride: with
+// the place of every 16-byte piece recomputed by divisions, and CTA barriers
+// between copies and MMAs, a tile took 4800 cycles even in the smallest layer
+// (8 x 32^3 training step: 2.69 ms of weight gradients).
+constexpr int WG_BUF = 3;           // tile buffers
+constexpr int WG_TMEM = 512;        // three accumulators of 128 columns
+constexpr int WG_COPY = 256;        // copying threads: warps 0 .. 7
+constexpr int WG_THREADS = WG_COPY + 32;  // and the warp of the MMA thread
+
+// Voxel tiles of 128 per CTA: chunks as long as 32 tiles, shorter ones where
+// the device would otherwise have fewer than one CTA per SM (8 x 16^3: 72
+// CTAs of 32 tiles against 144 of 16).
+int wg_tiles_per_cta(const ConvDims &dm)
+{
+    const int tiles = ((dm.W + TX - 1) / TX) * ((dm.H + TY - 1) / TY) * dm.D;
+    int n = 32;
+    while (n > 4 && 9ll * dm.B * ((tiles + n - 1) / n) < 140) n /= 2;
+    return n;
+}
 
 // kind::f16 instruction descriptor with both operands MN-major (bits 15, 16).
 __host__ __device__ constexpr uint32_t instr_desc_mn(int M, int N)
@@ -427,12 +528,12 @@ __host__ __device__ inline WgLayout wg_layout(int cin_p, int cout_p)
     return L;
 }
 
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(WG_THREADS, 1)
     wgrad_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__restrict__ dy,
-                    float *__restrict__ part, ConvDims dm, int n_chunks, int *err)
+                    float *__restrict__ part, ConvDims dm, int n_chunks, int tiles_per_cta, int *err)
 {
     extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ __align__(8) uint64_t bar[WG_BUF], done_bar;
+    __shared__ __align__(8) uint64_t full_bar[WG_BUF], empty_bar[WG_BUF], done_bar;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
     const int cout_p = dm.cout_p, cin_p = dm.cin_p, C8o = cout_p / 8, C8i = cin_p / 8;
@@ -442,14 +543,19 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int kz = g / 3, ky = g % 3;  // taps 9 kz + 3 ky + kx, kx = 0, 1, 2
     const int tiles_x = (dm.W + TX - 1) / TX, tiles_y = (dm.H + TY - 1) / TY;
     const int n_tiles = tiles_x * tiles_y * dm.D;
-    const int tile0 = chunk * WG_TILES, nt = min(n_tiles, tile0 + WG_TILES) - tile0;
+    const int tile0 = chunk * tiles_per_cta, nt = min(n_tiles, tile0 + tiles_per_cta) - tile0;
     const size_t vol = (size_t)dm.D * dm.H * dm.W;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int t = threadIdx.x, warp = t / 32, lane = t % 32;
+    volatile int *fail = &s_fail;
 
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < WG_BUF; q++) mbar_init(smem_u32(&bar[q]), 1);
+    if (t == 0) {
+        for (int q = 0; q < WG_BUF; q++) {
+            mbar_init(smem_u32(&full_bar[q]), WG_COPY);
+            mbar_init(smem_u32(&empty_bar[q]), 1);
+        }
         mbar_init(smem_u32(&done_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_fail = 0;
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -461,97 +567,99 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base;
-    const uint32_t idesc = instr_desc_mn(128, cin_p);
 
-    // asynchronous copies of tile tile0 + i into buffer i % WG_BUF (one group)
-    auto load_tile = [&](int i) {
-        const int tile = tile0 + i;
-        const int tz = tile / (tiles_x * tiles_y), txy = tile % (tiles_x * tiles_y);
-        const int x0 = (txy % tiles_x) * TX, y0 = (txy / tiles_x) * TY;
-        const uint32_t abuf = base + (uint32_t)(i % WG_BUF) * L.buf_bytes, hbuf = abuf + L.a_bytes;
-        for (int k = threadIdx.x; k < TX * TY * C8o; k += THREADS) {
-            const int c8 = k % C8o, v = k / C8o, vx = v % TX, vy = v / TX;
-            const int gx = x0 + vx, gy = y0 + vy;
-            const bool ok = gx < dm.W && gy < dm.H;
-            const __nv_bfloat16 *src =
-                ok ? dy + ((size_t)b * vol + ((size_t)tz * dm.H + gy) * dm.W + gx) * cout_p + c8 * 8 : dy;
-            cp_async16(abuf + (uint32_t)((vy * C8o + c8) * TX + vx) * 16, src, ok);
-        }
-        const int sz = tz + kz - 1;
-        for (int k = threadIdx.x; k < TY * HX * C8i; k += THREADS) {
-            const int c8 = k % C8i, h = k / C8i, hx = h % HX, hy = h / HX;
-            const int sx = x0 + hx - 1, sy = y0 + hy + ky - 1;
-            const bool ok = sz >= 0 && sz < dm.D && sx >= 0 && sx < dm.W && sy >= 0 && sy < dm.H;
-            const __nv_bfloat16 *src =
-                ok ? in + ((size_t)b * vol + ((size_t)sz * dm.H + sy) * dm.W + sx) * cin_p + c8 * 8 : in;
-            cp_async16(hbuf + (uint32_t)((hy * C8i + c8) * HX + hx) * 16, src, ok);
-        }
-        cp_async_commit();
-    };
-
-    // Thread 0 issues the MMAs and makes every wait on their completion; the
-    // other threads wait for it at CTA barriers rather than polling beside it
-    // in its warp.  s_fail records a wait that gave up (uniform after a barrier).
-    if (threadIdx.x == 0) s_fail = 0;
-    for (int i = 0; i < WG_BUF - 1 && i < nt; i++) load_tile(i);
-    for (int i = 0; i < nt; i++) {
-        const int j = i + WG_BUF - 1;
-        if (j < nt) {
-            // tile j reuses the buffer of tile i - 1: its MMAs must have completed
-            if (i >= 1) {
-                if (threadIdx.x == 0 && !s_fail && !mbar_wait(smem_u32(&bar[(i - 1) % WG_BUF]), ((i - 1) / WG_BUF) & 1))
-                    s_fail = 1;
-                __syncthreads();
+    if (t < WG_COPY) {
+        // The copying threads split in two parts, one per tensor, in the ratio
+        // of their pieces; a part covers whole voxel rows of its block at a
+        // time, a thread one (x, octet) of them.
+        const int na = TX * C8o, nh = HX * C8i;  // 16-byte pieces per row
+        const int ra = WG_COPY / (na + nh);             // rows of the dy tile per pass (na + nh <= 252)
+        const int rh = (WG_COPY - ra * na) / nh;        // rows of the input block per pass
+        const bool is_a = t < ra * na;
+        const int u = is_a ? t : t - ra * na;
+        const int per = is_a ? na : nh, rows = is_a ? ra : rh, C8 = is_a ? C8o : C8i;
+        const bool idle = u >= rows * per;
+        const int X = is_a ? TX : HX, r0 = u / per, c8 = u % per / X, px = u % X;  // x fastest: conflict-free stores
+        const uint32_t s_off = (is_a ? 0u : L.a_bytes) + (uint32_t)((r0 * C8 + c8) * X + px) * 16;
+        const uint32_t s_step = (uint32_t)(rows * C8 * X) * 16;
+        const int cp = is_a ? cout_p : cin_p;
+        const __nv_bfloat16 *tensor = (is_a ? dy : in) + (size_t)b * vol * cp + c8 * 8;
+        const long long g_step = (long long)rows * dm.W * cp;
+        for (int i = 0; i < nt; i++) {
+            // tile i reuses the buffer of tile i - WG_BUF: its MMAs must have completed
+            if (i >= WG_BUF &&
+                (*fail || !mbar_wait(smem_u32(&empty_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF - 1) & 1))) {
+                *fail = 1;
+                break;
             }
-            load_tile(j);
-            cp_async_wait<WG_BUF - 1>();  // tile i has landed
-        } else if (i + 1 < nt) {
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        fence_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (threadIdx.x == 0 && !s_fail) {
-            const uint32_t abuf = base + (uint32_t)(i % WG_BUF) * L.buf_bytes, hbuf = abuf + L.a_bytes;
-#pragma unroll 1
-            for (int ks = 0; ks < TY / 2; ks++) {  // K = 16 voxels: tile rows 2ks, 2ks + 1
-                const uint64_t a = smem_desc(abuf + (uint32_t)(2 * ks * C8o * TX) * 16, (uint32_t)(C8o * TX * 16), TX * 16);
-#pragma unroll
-                for (int kx = 0; kx < 3; kx++) {
-                    const uint64_t bd =
-                        smem_desc(hbuf + (uint32_t)(2 * ks * C8i * HX + kx) * 16, (uint32_t)(C8i * HX * 16), HX * 16);
-                    tc_mma(tmem + (uint32_t)(kx * 128), a, bd, idesc, (i | ks) != 0);
+            const int tile = tile0 + i;
+            const int tz = tile / (tiles_x * tiles_y), txy = tile % (tiles_x * tiles_y);
+            const int x = (txy % tiles_x) * TX + px - (is_a ? 0 : 1);
+            const int y = (txy / tiles_x) * TY + r0 + (is_a ? 0 : ky - 1), z = tz + (is_a ? 0 : kz - 1);
+            if (!idle) {
+                const bool plane = x >= 0 && x < dm.W && z >= 0 && z < dm.D;
+                const __nv_bfloat16 *src = tensor + (((long long)z * dm.H + y) * dm.W + x) * cp;
+                uint32_t dst = base + (uint32_t)(i % WG_BUF) * L.buf_bytes + s_off;
+                for (int r = r0, yy = y; r < TY; r += rows, yy += rows, src += g_step, dst += s_step) {
+                    const bool ok = plane && yy >= 0 && yy < dm.H;
+                    cp_async16(dst, ok ? src : tensor, ok);
                 }
             }
-            tc_commit(smem_u32(&bar[i % WG_BUF]));
-        }
-    }
-    if (threadIdx.x == 0) {
-        tc_commit(smem_u32(&done_bar));
-        if (!mbar_wait(smem_u32(&done_bar), 0)) s_fail = 1;
-    }
-    __syncthreads();
-    tc_fence_after();
-    if (s_fail) {  // uniform: the loads below are warp-collective
-        if (threadIdx.x == 0) atomicExch(err, 1);
-    } else {
-        // row co = TMEM lane; columns kx * 128 + ci
-        const int co = warp * 32 + lane;
-        for (int kx = 0; kx < 3; kx++) {
-            const int t = (kz * 3 + ky) * 3 + kx;
-            float *dst = part + (((size_t)b * n_chunks + chunk) * 27 + t) * cout_p * cin_p;
-            for (int c0 = 0; c0 < cin_p; c0 += 16) {
-                float v[16];
-                tc_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(kx * 128 + c0), v);
-                if (co >= cout_p) continue;
-#pragma unroll
-                for (int k = 0; k < 16; k += 4)
-                    *reinterpret_cast<float4 *>(dst + (size_t)co * cin_p + c0 + k) =
-                        make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+            cp_async_commit();
+            if (i >= 1) {  // tile i - 1 has landed, while tile i is on its way
+                cp_async_wait<1>();
+                fence_async_smem();
+                mbar_arrive(smem_u32(&full_bar[(i - 1) % WG_BUF]));
             }
+        }
+        cp_async_wait<0>();
+        fence_async_smem();
+        if (nt > 0 && !*fail) mbar_arrive(smem_u32(&full_bar[(nt - 1) % WG_BUF]));
+    } else if (t == WG_COPY) {
+        // descriptors advance by additions (16-byte units), as in conv_tc_kernel
+        const uint32_t idesc = instr_desc_mn(128, cin_p);
+        const uint64_t a_desc = smem_desc(0, (uint32_t)(C8o * TX * 16), TX * 16), a_ks = 2 * C8o * TX;
+        const uint64_t b_desc = smem_desc(0, (uint32_t)(C8i * HX * 16), HX * 16), b_ks = 2 * C8i * HX;
+        uint32_t first = 0;
+        for (int i = 0; i < nt; i++) {
+            if (*fail || !mbar_wait(smem_u32(&full_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF) & 1)) {
+                *fail = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t abuf = base + (uint32_t)(i % WG_BUF) * L.buf_bytes;
+            uint64_t ad = a_desc + (abuf >> 4), bd = b_desc + ((abuf + L.a_bytes) >> 4);
+            for (int ks = 0; ks < TY / 2; ks++) {  // K = 16 voxels: tile rows 2ks, 2ks + 1
+                tc_mma(tmem, ad, bd, idesc, first);
+                tc_mma(tmem + 128, ad, bd + 1, idesc, first);
+                tc_mma(tmem + 256, ad, bd + 2, idesc, first);
+                first = 1;
+                ad += a_ks;
+                bd += b_ks;
+            }
+            tc_commit(smem_u32(&empty_bar[i % WG_BUF]));
+        }
+        // every MMA issued has completed once the done barrier fires
+        tc_commit(smem_u32(&done_bar));
+        if (!mbar_wait(smem_u32(&done_bar), 0)) *fail = 1;
+    }
+    __syncthreads();  // the other threads wait here, not polling; s_fail is uniform after it
+    tc_fence_after();
+    if (s_fail) {
+        if (t == 0) atomicExch(err, 1);
+    } else if (warp < 8) {
+        // row co = TMEM lane (warps w and w + 4 share the lanes 32 (w % 4) ..
+        // and take every other block of 16 columns); columns kx * 128 + ci
+        const int co = (warp % 4) * 32 + lane, nb = cin_p / 16;
+        for (int q = warp / 4; q < 3 * nb; q += 2) {
+            const int kx = q / nb, c0 = q % nb * 16;
+            float v[16];
+            tc_ld16(tmem + ((uint32_t)((warp % 4) * 32) << 16) + (uint32_t)(kx * 128 + c0), v);
+            if (co >= cout_p) continue;
+            float *dst = part + ((((size_t)b * n_chunks + chunk) * 27 + (kz * 3 + ky) * 3 + kx) * cout_p + co) * cin_p + c0;
+#pragma unroll
+            for (int k = 0; k < 16; k += 4)
+                *reinterpret_cast<float4 *>(dst + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
         }
     }
     tc_fence_before();
@@ -562,17 +670,36 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
 }
 
+template <int MODE, bool RES>
+cudaError_t launch(size_t smem, const __nv_bfloat16 *in, const __nv_bfloat16 *wpk, const float *bias, void *out,
+                   const __nv_bfloat16 *gate, ConvDims dm, int *err, cudaStream_t s)
+{
+    // at least 120 KB: one CTA per SM, so no CTA waits for tensor memory held by another
+    smem = std::max<size_t>(smem, 120 * 1024);
+    int dev = 0, sms = 0;
+    cudaError_t e =
+        cudaFuncSetAttribute(conv_tc_kernel<MODE, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess || (e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return e;
+    const long long units =
+        (long long)((dm.W + TX - 1) / TX) * ((dm.H + TY - 1) / TY) * ((dm.D + OZ - 1) / OZ) * dm.B;
+    conv_tc_kernel<MODE, RES><<<(unsigned)std::min<long long>(sms, units), THREADS, smem, s>>>(in, wpk, bias, out, gate,
+                                                                                            dm, err);
+    return cudaGetLastError();
+}
+
+// All taps' weights stay in shared memory where they fit (16 -> 48 and 48 -> 16
+// channels): streamed again for every unit, their small copies are bound by
+// latency (64^3 voxels: 16 -> 48 channels 73 us, 48 -> 16 97 us streamed).
 template <int MODE>
 cudaError_t launch(const __nv_bfloat16 *in, const __nv_bfloat16 *wpk, const float *bias, void *out,
                    const __nv_bfloat16 *gate, ConvDims dm, int *err, cudaStream_t s)
 {
-    const size_t smem = (size_t)HZ * HY * (dm.cin_p / 8) * HX * 16 + NBUF * (size_t)(dm.cin_p / 8) * dm.cout_p * 16;
-    cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int tiles = ((dm.W + TX - 1) / TX) * ((dm.H + TY - 1) / TY);
-    conv_tc_kernel<MODE><<<dim3(tiles, (dm.D + OZ - 1) / OZ, dm.B), THREADS, smem, s>>>(in, wpk, bias, out, gate, dm,
-                                                                                     err);
-    return cudaGetLastError();
+    const size_t planes = (size_t)HZ * HY * (dm.cin_p / 8) * HX * 16, tap = (size_t)(dm.cin_p / 8) * dm.cout_p * 16;
+    if (planes + 27 * tap <= 220 * 1024)
+        return launch<MODE, true>(planes + 27 * tap, in, wpk, bias, out, gate, dm, err, s);
+    return launch<MODE, false>(planes + NBUF * tap, in, wpk, bias, out, gate, dm, err, s);
 }
 
 }  // namespace
@@ -597,7 +724,8 @@ cudaError_t conv_tc(int mode, const __nv_bfloat16 *in, const __nv_bfloat16 *w, _
 int wgrad_chunks(const ConvDims &dm)
 {
     const int tiles = ((dm.W + TX - 1) / TX) * ((dm.H + TY - 1) / TY) * dm.D;
-    return (tiles + WG_TILES - 1) / WG_TILES;
+    const int per = wg_tiles_per_cta(dm);
+    return (tiles + per - 1) / per;
 }
 
 cudaError_t wgrad_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *dy, float *part, ConvDims dm, int *err,
@@ -610,7 +738,8 @@ cudaError_t wgrad_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *dy, float *pa
     cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int n_chunks = wgrad_chunks(dm);
-    wgrad_tc_kernel<<<dim3(9, n_chunks, dm.B), THREADS, smem, s>>>(in, dy, part, dm, n_chunks, err);
+    wgrad_tc_kernel<<<dim3(9, n_chunks, dm.B), WG_THREADS, smem, s>>>(in, dy, part, dm, n_chunks,
+                                                                      wg_tiles_per_cta(dm), err);
     return cudaGetLastError();
 }
 

@@ -19,6 +19,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -44,22 +45,57 @@ __global__ void wgrad_reduce_kernel(const float *__restrict__ part, int n_parts,
     gw[i] = s;
 }
 
-// Bias gradient gb[co] = sum over voxels of dy[v][co]: one block per channel,
-// strided per-thread sums then a tree (fixed order).
-template <typename T>
-__global__ void bias_grad_kernel(const T *__restrict__ dy, size_t nvox, int cp, float *__restrict__ gb)
+// Bias gradient gb[co] = sum over voxels of dy[v][co], in two fixed-order
+// steps: a block sums a range of voxels, a thread eight channels of every few
+// voxels with 16-byte loads (whole rows of dy, coalesced), then a block per
+// channel adds the blocks' sums.  One block per channel, each reading 2 of
+// every 2 cp bytes, took 0.67 ms of an 8 x 32^3 training step, bound by the
+// latency of 112 blocks' strided loads.
+constexpr int BIAS_BLOCKS = 1216;
+__global__ void __launch_bounds__(256) bias_part_kernel(const uint4 *__restrict__ dy, size_t nvox, int cp,
+                                                         float *__restrict__ part)
 {
-    __shared__ float sh[256];
-    const int co = blockIdx.x;
+    __shared__ float sh[8][256];
+    const int octets = cp / 8, rows = 256 / octets, t = threadIdx.x;
+    const int c = t % octets, r = t / octets;
+    const size_t per = (nvox + gridDim.x - 1) / gridDim.x, v0 = blockIdx.x * per, v1 = min(nvox, v0 + per);
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (r < rows)
+#pragma unroll 4
+        for (size_t v = v0 + r; v < v1; v += rows) {
+            const uint4 q = dy[v * octets + c];
+            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&q);
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const float2 d = __bfloat1622float2(h[k]);
+                s[2 * k] += d.x;
+                s[2 * k + 1] += d.y;
+            }
+        }
+#pragma unroll
+    for (int k = 0; k < 8; k++) sh[k][t] = s[k];
+    __syncthreads();
+    if (t < cp) {
+        float sum = 0.f;
+        for (int k = 0; k < rows; k++) sum += sh[t % 8][k * octets + t / 8];
+        part[(size_t)blockIdx.x * cp + t] = sum;
+    }
+}
+
+__global__ void __launch_bounds__(128) bias_sum_kernel(const float *__restrict__ part, int n, int cp,
+                                                        float *__restrict__ gb)
+{
+    __shared__ float sh[128];
     float s = 0.f;
-    for (size_t v = threadIdx.x; v < nvox; v += 256) s += (float)dy[v * cp + co];
+#pragma unroll 4
+    for (int k = threadIdx.x; k < n; k += 128) s += part[(size_t)k * cp + blockIdx.x];
     sh[threadIdx.x] = s;
     __syncthreads();
-    for (int k = 128; k > 0; k >>= 1) {
+    for (int k = 64; k > 0; k >>= 1) {
         if ((int)threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) gb[co] = sh[0];
+    if (threadIdx.x == 0) gb[blockIdx.x] = sh[0];
 }
 
 // Wt[26-t][ci][co] = W[t][co][ci]: weights of the data-gradient convolution.
@@ -258,6 +294,7 @@ struct kgs_net {
     __nv_bfloat16 *ga = nullptr, *gb2 = nullptr;  // gradient ping-pong (bf16)
     float *wpart = nullptr;
     size_t wpart_cap = 0;
+    float *bpart = nullptr;             // [BIAS_BLOCKS][112] partial bias gradients
     float *loss_part = nullptr;
     size_t loss_part_cap = 0;
     float *h_loss = nullptr;
@@ -366,7 +403,9 @@ int backward(kgs_net *n)
         NN_CHECK(kgs::nn::wgrad_tc(n->act[l], gcur, n->wpart, dm, n->d_err, s));
         wgrad_reduce_kernel<<<nblk(per, 256), 256, 0, s>>>(n->wpart, n->B * n_chunks, per, n->g + n->w_off[l]);
         NN_CHECK(cudaGetLastError());
-        bias_grad_kernel<__nv_bfloat16><<<dm.cout_p, 256, 0, s>>>(gcur, nvox, dm.cout_p, n->g + n->b_off[l]);
+        const int nbb = (int)std::min<size_t>(BIAS_BLOCKS, (nvox + 63) / 64);
+        bias_part_kernel<<<nbb, 256, 0, s>>>(reinterpret_cast<const uint4 *>(gcur), nvox, dm.cout_p, n->bpart);
+        bias_sum_kernel<<<dm.cout_p, 128, 0, s>>>(n->bpart, nbb, dm.cout_p, n->g + n->b_off[l]);
         NN_CHECK(cudaGetLastError());
         if (l == 0) break;
         // data gradient into layer l's input, masked by that layer's ReLU
@@ -435,7 +474,8 @@ int kgs_net_create(kgs_net **out, int n_layers, const int *channels, unsigned lo
     };
     if (cudaMalloc(&n->p, off * 4) != cudaSuccess || cudaMalloc(&n->g, off * 4) != cudaSuccess ||
         cudaMalloc(&n->m1, off * 4) != cudaSuccess || cudaMalloc(&n->m2, off * 4) != cudaSuccess ||
-        cudaMalloc(&n->pb, off * 2) != cudaSuccess || cudaMalloc(&n->wt, wmax * 2) != cudaSuccess || cudaMalloc(&n->wpk, wmax * 2) != cudaSuccess ||
+        cudaMalloc(&n->pb, off * 2) != cudaSuccess || cudaMalloc(&n->wt, wmax * 2) != cudaSuccess ||
+        cudaMalloc(&n->bpart, BIAS_BLOCKS * 112 * sizeof(float)) != cudaSuccess || cudaMalloc(&n->wpk, wmax * 2) != cudaSuccess ||
         cudaMallocHost(&n->h_loss, sizeof(float)) != cudaSuccess || cudaMalloc(&n->d_err, sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&n->h_err, sizeof(int)) != cudaSuccess)
         return fail(KGS_ENOMEM);
@@ -623,7 +663,7 @@ void kgs_net_destroy(kgs_net *n)
     if (!n) return;
     cudaStreamSynchronize(n->stream);
     free_acts(n);
-    float *bufs[] = {n->p, n->g, n->m1, n->m2, n->wpart, n->loss_part};
+    float *bufs[] = {n->p, n->g, n->m1, n->m2, n->wpart, n->bpart, n->loss_part};
     for (float *b : bufs)
         if (b) cudaFree(b);
     if (n->pb) cudaFree(n->pb);
