@@ -159,7 +159,7 @@ int enqueue_iteration(kgs_batch *b, int which)
     KGS_CHECK(cudaEventRecordWithFlags(b->ev[1], st, cudaEventRecordExternal));
     for (int i = 0; i < b->n; i++)
         if (b->active[i] &&
-            ((rc = ctx_launch_sums(b->ctx[i])) || (rc = ctx_launch_closure(b->ctx[i], b->d_resid + 2 * i, nullptr))))
+            (rc = ctx_launch_close(b->ctx[i], b->d_resid + 2 * i)))
             return rc;
     KGS_CHECK(cudaMemcpyAsync(b->h_resid, b->d_resid, (2 * b->n + 1) * sizeof(double), cudaMemcpyDeviceToHost, st));
     return KGS_OK;
@@ -253,7 +253,7 @@ bool batch_step(kgs_batch *b, bool retire, std::vector<int> &count, std::vector<
         const double r = b->h_resid[2 * i];
         bad |= b->h_resid[2 * i + 1] != 0.0;
         ctx_finish(b->ctx[i], r);
-        b->kernel_launches += 6;  // coefficients, sums, four closure kernels
+        b->kernel_launches += b->ctx[i]->ax_tab ? 4 : 3;  // coefficients, axis factors (FP64), closure, residual
         count[i]++;
         b->done[i]++;
         last[i] = r;

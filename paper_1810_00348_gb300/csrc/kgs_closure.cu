@@ -4,9 +4,9 @@
 //   acc_sums         fixed-order sum of the persistent sweep's accumulators
 //   closure          the macroscopic update of Eq. (5) and the wall densities
 //                    of Eq. (9) from the per-cell sums
-//   finalize_mass    global mass and the Section 3.4 rescale factor
-//   scale_residual   rescale, divergence check and the Section 4.1 residual
-//   finalize_residual
+//   acc_close        the two in one, for an iteration that needs no sums
+//   residual         the Section 3.4 rescale, divergence check and the
+//                    Section 4.1 residual
 //   wall_flux_init   wall densities from the flux of the initial equilibrium
 // All arithmetic in FP64.  Every reduction is a fixed-shape tree per block
 // followed by an in-order sum over blocks, so results do not depend on
@@ -87,22 +87,6 @@ __global__ void coef_kernel(const double *__restrict__ mac, const uint8_t *__res
     }
     out[C_FLAGS] = flag_value<Real>(flags);
     for (int q = 0; q < NCOEF; q++) coef[c * NCOEF + q] = out[q];
-}
-
-// Block tree sum of NV doubles per thread into blk[blockIdx.x * NV + v].
-template <int NV>
-__device__ void block_sum(double (&v)[NV], double *blk)
-{
-    __shared__ double sh[NV][RED_THREADS];
-    for (int q = 0; q < NV; q++) sh[q][threadIdx.x] = v[q];
-    __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-            for (int q = 0; q < NV; q++) sh[q][threadIdx.x] += sh[q][threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int q = 0; q < NV; q++) blk[(size_t)blockIdx.x * NV + q] = sh[q][0];
 }
 
 // Float-float accumulator: the running sum is hi + lo with |lo| <= ulp(hi)/2
@@ -342,18 +326,14 @@ __device__ __forceinline__ void shift_sums(double (&s)[SUM_F0], const double U[3
 // cells per block.  First the block's (cell, slot) pairs in address order
 // (coalesced): each adds its slot's nacc accumulators in accumulator order
 // (float-float for the FP32 path) into shared memory.  Then one thread per
-// cell maps the accumulator slots to the NSUM sum slots, adds the reference
-// Maxwellian's part (FP32 path) and writes the FP64 sums.
+// cell maps the accumulator slots to the NSUM sum slots and adds the reference
+// Maxwellian's part (FP32 path).
 constexpr int ACC_CELLS = 128;
 template <typename Real>
-__global__ void __launch_bounds__(ACC_CELLS) acc_sums_kernel(const AccSumArgs a)
+__device__ __forceinline__ void acc_totals(const AccSumArgs &a, size_t c0, int nc, double *tot)
 {
-    __shared__ double tot[ACC_CELLS * ACC_SPLIT];
-    const size_t ncell = a.ncell;
-    const size_t c0 = (size_t)blockIdx.x * ACC_CELLS;
-    const int nc = (int)min((size_t)ACC_CELLS, ncell - c0);
     const int ns = a.acc_slots, nacc = a.nacc;
-    const size_t ks = ncell * ns;
+    const size_t ks = a.ncell * ns;
     for (int j = threadIdx.x; j < nc * ns; j += ACC_CELLS) {
         const size_t at = c0 * ns + j;
         if (sizeof(Real) == 8) {
@@ -381,62 +361,71 @@ __global__ void __launch_bounds__(ACC_CELLS) acc_sums_kernel(const AccSumArgs a)
             tot[j] = t.value();
         }
     }
-    __syncthreads();
-    const int cl = threadIdx.x;
-    if (cl >= nc) return;
-    const size_t c = c0 + cl;
-    const double *tc = tot + (size_t)cl * ns;
-    if (a.solid && a.solid[c]) {
-        for (int q = 0; q < NSUM; q++) a.sums[(size_t)q * ncell + c] = 0.0;
-        return;
-    }
+}
+
+// The NSUM sums of fluid cell c from its accumulator totals tc.
+template <typename Real>
+__device__ __forceinline__ void cell_sums(const AccSumArgs &a, size_t c, const double *tc, double (&S)[NSUM])
+{
+    double s[SUM_F0];
+#pragma unroll
+    for (int q = 0; q < SUM_F0; q++) s[q] = tc[q];
     if constexpr (sizeof(Real) == 4) {
         // the FP32 sweep summed g = f - M_ref: add the reference's part
         double U[3], ref[SUM_F0];
         centre32(a.coef, c, U);
         ref_slots(a.ref, U, ref);
 #pragma unroll
-        for (int q = 0; q < SUM_F0; q++) a.sums[(size_t)q * ncell + c] = tc[q] + ref[q];
-    } else {
-        double s[SUM_F0];
-        for (int q = 0; q < SUM_F0; q++) s[q] = tc[q];
-        if (a.raw) {
-            double U[3];
-            const double *cf = static_cast<const double *>(a.coef) + c * NCOEF;
-            for (int d = 0; d < 3; d++) U[d] = -0.5 * cf[C_M2UX + d];
-            shift_sums(s, U);
-        }
-        for (int q = 0; q < SUM_F0; q++) a.sums[(size_t)q * ncell + c] = s[q];
+        for (int q = 0; q < SUM_F0; q++) s[q] += ref[q];
+    } else if (a.raw) {
+        double U[3];
+        const double *cf = static_cast<const double *>(a.coef) + c * NCOEF;
+        for (int d = 0; d < 3; d++) U[d] = -0.5 * cf[C_M2UX + d];
+        shift_sums(s, U);
     }
+#pragma unroll
+    for (int q = 0; q < SUM_F0; q++) S[q] = s[q];
 #pragma unroll
     for (int side = 0; side < 6; side++) {
         // compact layout: the flux of an axis belongs to the side that has a
         // wall, zero on the other side
-        const bool wall = a.wall_kind[(size_t)side * ncell + c] >= 0;
+        const bool wall = a.wall_kind[(size_t)side * a.ncell + c] >= 0;
         double v;
-        if (ns == ACC_COMPACT)
+        if (a.acc_slots == ACC_COMPACT)
             v = wall ? tc[SUM_F0 + side / 2] : 0.0;
         else
             v = tc[SUM_F0 + side];
         if constexpr (sizeof(Real) == 4)
             if (wall) v += a.ref.flux[side];
-        a.sums[(size_t)(SUM_F0 + side) * ncell + c] = v;
+        S[SUM_F0 + side] = v;
     }
 }
 
-// Closure of one outer iteration, one thread per cell (CLOSE_CELLS cells per
-// block): the sums about U^n become the macroscopic fields of step n+1 and
-// the wall densities (Eq. (5), Eq. (9)); the block's cell masses are summed
-// in a fixed order for the Section 3.4 rescale.
-__global__ void __launch_bounds__(CLOSE_CELLS) closure_kernel(const ClosureArgs a)
+// The sums written out, for a velocity partition (kgs_sweep_sums).
+template <typename Real>
+__global__ void __launch_bounds__(ACC_CELLS) acc_sums_kernel(const AccSumArgs a)
+{
+    __shared__ double tot[ACC_CELLS * ACC_SPLIT];
+    const size_t ncell = a.ncell, c0 = (size_t)blockIdx.x * ACC_CELLS;
+    const int nc = (int)min((size_t)ACC_CELLS, ncell - c0);
+    acc_totals<Real>(a, c0, nc, tot);
+    __syncthreads();
+    if ((int)threadIdx.x >= nc) return;
+    const size_t c = c0 + threadIdx.x;
+    double S[NSUM];
+#pragma unroll
+    for (int q = 0; q < NSUM; q++) S[q] = 0.0;
+    if (!(a.solid && a.solid[c])) cell_sums<Real>(a, c, tot + (size_t)threadIdx.x * a.acc_slots, S);
+#pragma unroll
+    for (int q = 0; q < NSUM; q++) a.sums[(size_t)q * ncell + c] = S[q];
+}
+
+// Closure of one fluid cell: the sums about U^n become the macroscopic fields
+// of step n+1 and the wall densities (Eq. (5), Eq. (9)).  Returns the cell's mass.
+__device__ __forceinline__ double close_cell(const ClosureArgs &a, size_t c, const double (&S)[NSUM])
 {
     const size_t ncell = a.ncell;
-    const size_t c = (size_t)blockIdx.x * CLOSE_CELLS + threadIdx.x;
-    const bool live = c < ncell && !(a.solid && a.solid[c]);
-    double mass = 0.0;
-    if (live) {
-        double S[NSUM];
-        for (int q = 0; q < NSUM; q++) S[q] = a.sums[(size_t)q * ncell + c];
+    {
         // The sums were taken about the lagged velocity U^n as stored in the
         // sweep precision; shift exactly to U^{n+1} = U^n + delta.
         double m2u[3];
@@ -488,10 +477,30 @@ __global__ void __launch_bounds__(CLOSE_CELLS) closure_kernel(const ClosureArgs 
             a.rho_w_new[s * ncell + c] = kind >= 0 ? S[SUM_F0 + s] * a.wall_norm[kind * 6 + s] : 0.0;
         }
         const int i = (int)(c % a.nx), j = (int)((c / a.nx) % a.ny), k = (int)(c / ((size_t)a.nx * a.ny));
-        mass = rho * a.dx[i] * a.dy[j] * a.dz[k];
+        return rho * a.dx[i] * a.dy[j] * a.dz[k];
+    }
+}
+
+__device__ __forceinline__ void close_solid(const ClosureArgs &a, size_t c)
+{
+    for (int v = 0; v < 8; v++) a.mac_new[v * a.ncell + c] = 0.0;
+    for (int s = 0; s < 6; s++) a.rho_w_new[s * a.ncell + c] = 0.0;
+}
+
+// Closure from sums in memory, one thread per cell (CLOSE_CELLS cells per
+// block); the block's cell masses are summed in a fixed order for the Section
+// 3.4 rescale.
+__global__ void __launch_bounds__(CLOSE_CELLS) closure_kernel(const ClosureArgs a)
+{
+    const size_t ncell = a.ncell;
+    const size_t c = (size_t)blockIdx.x * CLOSE_CELLS + threadIdx.x;
+    double mass = 0.0;
+    if (c < ncell && !(a.solid && a.solid[c])) {
+        double S[NSUM];
+        for (int q = 0; q < NSUM; q++) S[q] = a.sums[(size_t)q * ncell + c];
+        mass = close_cell(a, c, S);
     } else if (c < ncell) {
-        for (int v = 0; v < 8; v++) a.mac_new[v * ncell + c] = 0.0;
-        for (int s = 0; s < 6; s++) a.rho_w_new[s * ncell + c] = 0.0;
+        close_solid(a, c);
     }
     // fixed-order sum of the block's cell masses (lanes 0 .. CLOSE_CELLS-1)
     static_assert(CLOSE_CELLS == 32, "one warp per block's cells");
@@ -499,111 +508,141 @@ __global__ void __launch_bounds__(CLOSE_CELLS) closure_kernel(const ClosureArgs 
     if (threadIdx.x == 0) a.blk_mass[blockIdx.x] = mass;
 }
 
-// Total mass (fixed order: strided per-thread sums, then a tree) and the
-// Section 3.4 rescale factor.
-__global__ void __launch_bounds__(RED_THREADS)
-    finalize_mass_kernel(const double *blk_mass, int n_blocks, double M0, int rescale, double *scale)
+// Closure straight from the accumulators: the sums of a cell stay in the
+// registers of its thread (64^3 cells: 117 + 53 us with the sums written and
+// read back).
+template <typename Real>
+__global__ void __launch_bounds__(ACC_CELLS) acc_close_kernel(const AccSumArgs a, const ClosureArgs k)
 {
-    __shared__ double sh[RED_THREADS];
-    double M = 0.0;
-    for (int b = threadIdx.x; b < n_blocks; b += RED_THREADS) M += blk_mass[b];
-    sh[threadIdx.x] = M;
+    __shared__ double tot[ACC_CELLS * ACC_SPLIT];
+    __shared__ double wm[ACC_CELLS / 32];
+    const size_t ncell = a.ncell, c0 = (size_t)blockIdx.x * ACC_CELLS;
+    const int nc = (int)min((size_t)ACC_CELLS, ncell - c0);
+    acc_totals<Real>(a, c0, nc, tot);
     __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    double mass = 0.0;
+    if ((int)threadIdx.x < nc) {
+        const size_t c = c0 + threadIdx.x;
+        if (!(a.solid && a.solid[c])) {
+            double S[NSUM];
+            cell_sums<Real>(a, c, tot + (size_t)threadIdx.x * a.acc_slots, S);
+            mass = close_cell(k, c, S);
+        } else {
+            close_solid(k, c);
+        }
     }
-    if (threadIdx.x == 0) {
-        scale[0] = rescale ? M0 / sh[0] : 1.0;
-        scale[1] = sh[0];
-    }
+    for (int off = 16; off > 0; off >>= 1) mass += __shfl_down_sync(0xffffffffu, mass, off);
+    if (threadIdx.x % 32 == 0) wm[threadIdx.x / 32] = mass;
+    __syncthreads();
+    if (threadIdx.x == 0) k.blk_mass[blockIdx.x] = (wm[0] + wm[1]) + (wm[2] + wm[3]);
 }
 
-__global__ void __launch_bounds__(RED_THREADS)
-    scale_residual_kernel(double *mac_new, double *rho_w_new, const double *mac, const uint8_t *solid, size_t ncell,
-                          const double *scale, double *blk_res, int *blk_bad)
+// Total mass and the Section 3.4 rescale factor, the rescale, the divergence
+// check and the Section 4.1 residual in one launch.  Every block sums the
+// masses of all blocks of the closure itself (the same fixed order in each:
+// strided per-thread sums, then a tree); the last block to finish adds the
+// blocks' residual sums, again in a fixed order, and resets the counter.
+__global__ void __launch_bounds__(RED_THREADS) residual_kernel(const ResidualArgs a)
 {
-    const size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const double s = scale[0];
+    __shared__ double sh[10][RED_THREADS];
+    __shared__ int any_bad, last;
+    const size_t ncell = a.ncell;
+    const int t = threadIdx.x;
+    double s = 1.0;
+    if (a.rescale) {
+        double M = 0.0;
+        for (int b = t; b < a.n_mass; b += RED_THREADS) M += a.blk_mass[b];
+        sh[0][t] = M;
+        __syncthreads();
+        for (int k = RED_THREADS / 2; k > 0; k >>= 1) {
+            if (t < k) sh[0][t] += sh[0][t + k];
+            __syncthreads();
+        }
+        s = a.M0 / sh[0][0];
+        __syncthreads();
+    }
+    if (t == 0) any_bad = 0;
+    const size_t c = (size_t)blockIdx.x * RED_THREADS + t;
     double v[10];
     for (int q = 0; q < 10; q++) v[q] = 0.0;
     int bad = 0;
-    if (c < ncell && !(solid && solid[c])) {
-        mac_new[c] *= s;
-        for (int d = 0; d < 3; d++) mac_new[(5 + d) * ncell + c] *= s;
-        for (int f = 0; f < 6; f++) rho_w_new[f * ncell + c] *= s;
+    if (c < ncell && !(a.solid && a.solid[c])) {
+        double m[8];
+        for (int q = 0; q < 8; q++) m[q] = a.mac_new[q * ncell + c];
+        m[0] *= s;
+        a.mac_new[c] = m[0];
+        for (int d = 0; d < 3; d++) {
+            m[5 + d] *= s;
+            a.mac_new[(5 + d) * ncell + c] = m[5 + d];
+        }
+        for (int f = 0; f < 6; f++) a.rho_w_new[f * ncell + c] *= s;
         double pn[5], po[5];
-        for (int t = 0; t < 2; t++) {
-            const double *m = t ? mac : mac_new;
-            double *phi = t ? po : pn;
-            const double r = m[c], ux = m[ncell + c], uy = m[2 * ncell + c], uz = m[3 * ncell + c],
-                         T = m[4 * ncell + c];
+        for (int q = 0; q < 2; q++) {
+            double *phi = q ? po : pn;
+            const double r = q ? a.mac[c] : m[0], ux = q ? a.mac[ncell + c] : m[1],
+                         uy = q ? a.mac[2 * ncell + c] : m[2], uz = q ? a.mac[3 * ncell + c] : m[3],
+                         T = q ? a.mac[4 * ncell + c] : m[4];
             phi[0] = r;
             phi[1] = r * ux;
             phi[2] = r * uy;
             phi[3] = r * uz;
             phi[4] = 0.5 * r * (ux * ux + uy * uy + uz * uz) + 1.5 * r * R_GAS * T;
         }
-        for (int t = 0; t < 5; t++) {
-            const double dd = pn[t] - po[t];
-            v[t] = dd * dd;
-            v[5 + t] = pn[t] * pn[t];
+        for (int q = 0; q < 5; q++) {
+            const double dd = pn[q] - po[q];
+            v[q] = dd * dd;
+            v[5 + q] = pn[q] * pn[q];
         }
-        const double r = mac_new[c], T = mac_new[4 * ncell + c];
-        bool finite = isfinite(r) && isfinite(T);
-        for (int q = 1; q < 8; q++) finite = finite && isfinite(mac_new[q * ncell + c]);
-        if (!(r > 0.0) || !(T > 0.0) || !finite) bad = 1;
+        bool finite = true;
+        for (int q = 0; q < 8; q++) finite = finite && isfinite(m[q]);
+        if (!(m[0] > 0.0) || !(m[4] > 0.0) || !finite) bad = 1;
     }
-    block_sum<10>(v, blk_res);
-    __shared__ int any_bad;
-    if (threadIdx.x == 0) any_bad = 0;
-    __syncthreads();
-    if (bad) any_bad = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) blk_bad[blockIdx.x] = any_bad;
-}
-
-__global__ void __launch_bounds__(RED_THREADS)
-    finalize_residual_kernel(const double *blk_res, const int *blk_bad, int n_blocks, double *out)
-{
-    // fixed order: strided per-thread sums over the blocks, then a tree
-    double v[10];
-    for (int t = 0; t < 10; t++) v[t] = 0.0;
-    int bad = 0;
-    for (int b = threadIdx.x; b < n_blocks; b += RED_THREADS) {
-        for (int t = 0; t < 10; t++) v[t] += blk_res[(size_t)b * 10 + t];
-        bad |= blk_bad[b];
-    }
-    __shared__ double sh[10][RED_THREADS];
-    __shared__ int any_bad;
-    if (threadIdx.x == 0) any_bad = 0;
-    for (int t = 0; t < 10; t++) sh[t][threadIdx.x] = v[t];
-    __syncthreads();
-    if (bad) any_bad = 1;
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-            for (int t = 0; t < 10; t++) sh[t][threadIdx.x] += sh[t][threadIdx.x + s];
+    auto tree = [&]() {  // sums of v[q] over the block into sh[q][0]
+        for (int q = 0; q < 10; q++) sh[q][t] = v[q];
         __syncthreads();
+        if (bad) any_bad = 1;
+        for (int k = RED_THREADS / 2; k > 0; k >>= 1) {
+            if (t < k)
+                for (int q = 0; q < 10; q++) sh[q][t] += sh[q][t + k];
+            __syncthreads();
+        }
+    };
+    tree();
+    if (t < 10) a.blk_res[(size_t)blockIdx.x * 10 + t] = sh[t][0];
+    if (t == 0) {
+        a.blk_bad[blockIdx.x] = any_bad;
     }
-    if (threadIdx.x != 0) return;
-    double dn[5], nn[5];
-    for (int t = 0; t < 5; t++) {
-        dn[t] = sh[t][0];
-        nn[t] = sh[5 + t][0];
+    __syncthreads();
+    if (t == 0) {
+        __threadfence();
+        last = atomicAdd(a.count, 1u) == gridDim.x - 1;
+        __threadfence();
     }
-    bad = any_bad;
+    __syncthreads();
+    if (!last) return;
+    for (int q = 0; q < 10; q++) v[q] = 0.0;
+    bad = 0;
+    for (int b = t; b < (int)gridDim.x; b += RED_THREADS) {
+        for (int q = 0; q < 10; q++) v[q] += __ldcg(&a.blk_res[(size_t)b * 10 + q]);
+        bad |= __ldcg(&a.blk_bad[b]);
+    }
+    if (t == 0) any_bad = 0;
+    __syncthreads();
+    tree();
+    if (t != 0) return;
     // Section 4.1 reading: largest relative L2 change over rho, rho U, rho E;
     // denominators floored at 1e-8 ||rho||_2.
     double res = 0.0;
-    const double fl = 1e-8 * sqrt(nn[0]);
-    for (int t = 0; t < 5; t++) {
-        double den = sqrt(nn[t]);
+    const double fl = 1e-8 * sqrt(sh[5][0]);
+    for (int q = 0; q < 5; q++) {
+        double den = sqrt(sh[5 + q][0]);
         if (den < fl) den = fl;
-        const double r = sqrt(dn[t]) / den;
+        const double r = sqrt(sh[q][0]) / den;
         if (r > res) res = r;
     }
-    out[0] = res;
-    out[1] = bad ? 1.0 : 0.0;
+    a.out[0] = res;
+    a.out[1] = any_bad ? 1.0 : 0.0;
+    *a.count = 0;
 }
 
 // rho_w^0 from the flux of f^{S,0} through each wall face (Eq. (9) with the
@@ -683,10 +722,10 @@ cudaError_t launch_coef(int precision, const double *mac, const uint8_t *solid, 
 {
     const size_t n = (size_t)nx * ny * nz;
     if (precision == 0)
-        coef_kernel<double><<<nblk(n, 256), 256, 0, s>>>(mac, solid, side_flags, rdx, rdy, rdz, nx, ny, nz, mu_ref,
+        coef_kernel<double><<<nblk(n, 64), 64, 0, s>>>(mac, solid, side_flags, rdx, rdy, rdz, nx, ny, nz, mu_ref,
                                                           omega, Pr, 0, static_cast<double *>(coef), nullptr, nullptr);
     else
-        coef_kernel<float><<<nblk(n, 256), 256, 0, s>>>(mac, solid, side_flags, rdx, rdy, rdz, nx, ny, nz, mu_ref,
+        coef_kernel<float><<<nblk(n, 64), 64, 0, s>>>(mac, solid, side_flags, rdx, rdy, rdz, nx, ny, nz, mu_ref,
                                                          omega, Pr, dev_src, static_cast<float *>(coef), rho_w, rho_w32);
     return cudaGetLastError();
 }
@@ -717,26 +756,21 @@ cudaError_t launch_closure(const ClosureArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize_mass(const double *blk_mass, int n_blocks, double M0, int rescale, double *scale,
-                                 cudaStream_t s)
+cudaError_t launch_acc_close(const AccSumArgs &a, const ClosureArgs &k, cudaStream_t s)
 {
-    finalize_mass_kernel<<<1, RED_THREADS, 0, s>>>(blk_mass, n_blocks, M0, rescale, scale);
+    const unsigned nb = (unsigned)acc_close_blocks(a.ncell);
+    if (a.precision == 0)
+        acc_close_kernel<double><<<nb, ACC_CELLS, 0, s>>>(a, k);
+    else
+        acc_close_kernel<float><<<nb, ACC_CELLS, 0, s>>>(a, k);
     return cudaGetLastError();
 }
 
-cudaError_t launch_scale_residual(double *mac_new, double *rho_w_new, const double *mac, const uint8_t *solid,
-                                  unsigned long long ncell, const double *scale, double *blk_res, int *blk_bad,
-                                  int n_blocks, cudaStream_t s)
-{
-    scale_residual_kernel<<<n_blocks, RED_THREADS, 0, s>>>(mac_new, rho_w_new, mac, solid, ncell, scale, blk_res,
-                                                           blk_bad);
-    return cudaGetLastError();
-}
+unsigned long long acc_close_blocks(unsigned long long ncell) { return (ncell + ACC_CELLS - 1) / ACC_CELLS; }
 
-cudaError_t launch_finalize_residual(const double *blk_res, const int *blk_bad, int n_blocks, double *out2,
-                                     cudaStream_t s)
+cudaError_t launch_residual(const ResidualArgs &a, cudaStream_t s)
 {
-    finalize_residual_kernel<<<1, RED_THREADS, 0, s>>>(blk_res, blk_bad, n_blocks, out2);
+    residual_kernel<<<nblk((size_t)a.ncell, RED_THREADS), RED_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 

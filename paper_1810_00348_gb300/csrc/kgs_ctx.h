@@ -42,8 +42,9 @@ struct kgs_ctx {
     double *wall_norm = nullptr;
     int4 *work = nullptr;
     int *d_vstart = nullptr, *d_vcount = nullptr, *d_vgbase = nullptr, *d_vg_oct = nullptr;
-    double *blk_mass = nullptr, *blk_res = nullptr, *scale = nullptr, *resid = nullptr;
+    double *blk_mass = nullptr, *blk_res = nullptr, *resid = nullptr;
     int *blk_bad = nullptr;
+    unsigned *red_count = nullptr;   // blocks of the residual kernel that have finished (zero between launches)
     double *h_resid = nullptr;  // pinned: residual, divergence flag, wait-error word
     // persistent sweep of a standalone context: one launch per iteration over
     // the work items in stage order; a CTA waits (bounded) for the three
@@ -51,13 +52,15 @@ struct kgs_ctx {
     int persist = 0;
     int persist_grid = 0, persist_items = 0;
     int4 *p_items = nullptr;
-    int *p_counter = nullptr, *p_flags = nullptr, *p_flag_off = nullptr;
+    int *p_counter = nullptr;         // claim counter, then the flags and the chain tokens (one buffer)
+    int *p_flags = nullptr, *p_flag_off = nullptr;
     size_t p_n_flags = 0;
     int *p_pos = nullptr;             // place of each item in its accumulator chain
     int *p_tok = nullptr;             // chain tokens [nacc][nbz][nby][nbx]
     void *p_scratch = nullptr;        // per-CTA moment partials
     size_t scratch_stride = 0;
-    kgs::SweepArgs *p_args = nullptr, *h_args = nullptr;  // device copy, pinned host staging
+    kgs::SweepArgs *p_args = nullptr;        // [2] device: with rho_w = rho_w_first, and with the other buffer
+    const double *rho_w_first = nullptr;
     long long spin_limit = 20000000;  // polls of ~100 ns before a wait gives up
     size_t device_bytes = 0;
     std::vector<void *> allocs;
@@ -105,9 +108,12 @@ int ctx_launch_coef(kgs_ctx *c);
 int ctx_launch_stages(kgs_ctx *c);
 // Per-cell sums of the swept velocities into c->sums.
 int ctx_launch_sums(kgs_ctx *c);
-// Closure from the per-cell sums (sums = NULL: c->sums) into the new buffers;
-// the residual and divergence flag go to resid_dev[0..1] (device).
-int ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums);
+// Closure into the new buffers, from the accumulators (from_acc) or from
+// per-cell sums (sums = NULL: c->sums); the residual and divergence flag go to
+// resid_dev[0..1] (device).
+int ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums, bool from_acc);
+// The part of an outer iteration after the sweep.
+int ctx_launch_close(kgs_ctx *c, double *resid_dev);
 // After the iteration's work has completed: swap the state buffers.
 void ctx_finish(kgs_ctx *c, double residual);
 

@@ -300,13 +300,26 @@ struct AccSumArgs {
 };
 cudaError_t launch_acc_sums(const AccSumArgs &a, cudaStream_t s);
 cudaError_t launch_closure(const ClosureArgs &a, cudaStream_t s);
-cudaError_t launch_finalize_mass(const double *blk_mass, int n_blocks, double M0, int rescale, double *scale,
-                                 cudaStream_t s);
-cudaError_t launch_scale_residual(double *mac_new, double *rho_w_new, const double *mac, const uint8_t *solid,
-                                  unsigned long long ncell, const double *scale, double *blk_res, int *blk_bad,
-                                  int n_blocks, cudaStream_t s);
-cudaError_t launch_finalize_residual(const double *blk_res, const int *blk_bad, int n_blocks, double *out2,
-                                     cudaStream_t s);
+// launch_acc_sums and launch_closure in one, the sums kept in registers;
+// blk_mass receives acc_close_blocks(ncell) values.
+cudaError_t launch_acc_close(const AccSumArgs &a, const ClosureArgs &k, cudaStream_t s);
+unsigned long long acc_close_blocks(unsigned long long ncell);
+// Rescale, divergence check and residual after a closure.
+struct ResidualArgs {
+    double *mac_new, *rho_w_new;  // step n+1, rescaled in place
+    const double *mac;            // step n
+    const uint8_t *solid;         // [ncell] or NULL
+    unsigned long long ncell;
+    const double *blk_mass;       // [n_mass] of the closure
+    int n_mass;
+    double M0;
+    int rescale;                  // 1: scale the total mass to M0
+    double *blk_res;              // [blocks of 256 cells][10]
+    int *blk_bad;                 // [blocks of 256 cells]
+    unsigned *count;              // zero before the first launch; left zero
+    double *out;                  // residual, divergence flag
+};
+cudaError_t launch_residual(const ResidualArgs &a, cudaStream_t s);
 cudaError_t launch_wall_flux_init(const double *mac, const int8_t *wall_kind, const double *wall_norm,
                                   const double *axis64, int nvx, int nvy, int nvz, unsigned long long ncell, double R,
                                   double Pr,

@@ -7,9 +7,9 @@
 // block faces between sweep stages, the ordered per-cell moment accumulators
 // with the work list, chain places and per-CTA scratch of the persistent
 // sweep, and the per-cell sums.  kgs_iterate launches, per outer iteration,
-// the coefficient kernel, one persistent sweep launch, the sums kernel and
-// four small FP64 closure kernels, then reads back 24 bytes (residual,
-// divergence flag and the wait-error word).
+// the coefficient kernel, one persistent sweep launch, the closure and the
+// residual kernel, then reads back 24 bytes (residual, divergence flag and the
+// wait-error word).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -89,8 +89,6 @@ void free_all(kgs_ctx *c)
     c->ev.clear();
     if (c->h_resid) cudaFreeHost(c->h_resid);
     c->h_resid = nullptr;
-    if (c->h_args) cudaFreeHost(c->h_args);
-    c->h_args = nullptr;
 }
 
 // Upload macros (or the uniform state), set M0 and the wall densities from
@@ -250,15 +248,10 @@ int kgs::ctx_launch_stages(kgs_ctx *c)
     cudaStream_t st = c->stream;
     SweepArgs a = ctx_sweep_args(c);
     if (c->persist) {
-        // the previous iteration has completed (run_iteration synchronises),
-        // so the pinned staging copy is free to be rewritten
-        *c->h_args = a;
-        KGS_CHECK(cudaMemcpyAsync(c->p_args, c->h_args, sizeof(SweepArgs), cudaMemcpyHostToDevice, st));
-        KGS_CHECK(cudaMemsetAsync(c->p_counter, 0, sizeof(int), st));
-        KGS_CHECK(cudaMemsetAsync(c->p_flags, 0, c->p_n_flags * sizeof(int), st));
-        KGS_CHECK(cudaMemsetAsync(c->p_tok, 0, ctx_n_tokens(t) * sizeof(int), st));
+        // claim counter, progress flags and chain tokens lie in one buffer
+        KGS_CHECK(cudaMemsetAsync(c->p_counter, 0, (1 + c->p_n_flags + ctx_n_tokens(t)) * sizeof(int), st));
         BatchSweepArgs ba;
-        ba.inst = c->p_args;
+        ba.inst = c->p_args + (c->rho_w == c->rho_w_first ? 0 : 1);
         ba.items = c->p_items;
         ba.n_items = c->persist_items;
         ba.counter = c->p_counter;
@@ -367,34 +360,49 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     c->persist_grid = sms * per_sm;
     c->scratch_stride = sweep_scratch_bytes(t.bz);
     if ((rc = upload(c, &c->p_items, items)) || (rc = upload(c, &c->p_pos, pos)) ||
-        (rc = dalloc_t(c, &c->p_counter, 1)) || (rc = dalloc_t(c, &c->p_flags, c->p_n_flags)) ||
-        (rc = dalloc_t(c, &c->p_tok, ctx_n_tokens(t))) ||
-        (rc = upload(c, &c->p_flag_off, std::vector<int>(1, 0))) || (rc = dalloc_t(c, &c->p_args, 1)) ||
+        (rc = dalloc_t(c, &c->p_counter, 1 + c->p_n_flags + ctx_n_tokens(t))) ||
+        (rc = upload(c, &c->p_flag_off, std::vector<int>(1, 0))) || (rc = dalloc_t(c, &c->p_args, 2)) ||
         (rc = dalloc(c, &c->p_scratch, (size_t)c->persist_grid * c->scratch_stride)) || (rc = ctx_alloc_acc(c)))
         return rc;
-    KGS_CHECK(cudaMallocHost(&c->h_args, sizeof(SweepArgs)));
+    c->p_flags = c->p_counter + 1;
+    c->p_tok = c->p_flags + c->p_n_flags;
+    // the sweep's arguments, once for each of the two state buffers that the
+    // iterations alternate between
+    c->rho_w_first = c->rho_w;
+    SweepArgs args[2];
+    for (SweepArgs &x : args) {
+        x = ctx_sweep_args(c);
+        std::swap(c->rho_w, c->rho_w_new);
+    }
+    KGS_CHECK(cudaMemcpy(c->p_args, args, sizeof args, cudaMemcpyHostToDevice));
     c->persist_items = (int)items.size();
     c->persist = 1;
     return KGS_OK;
+}
+
+static AccSumArgs acc_args(const kgs_ctx *c)
+{
+    const HostTables &t = c->t;
+    AccSumArgs aa;
+    aa.precision = t.precision;
+    aa.acc = c->acc;
+    aa.nacc = t.nacc;
+    aa.acc_slots = t.acc_slots;
+    aa.raw = c->ax_tab != nullptr;
+    aa.ncell = t.ncell;
+    aa.solid = c->solid;
+    aa.sums = c->sums;
+    aa.coef = c->coef;
+    aa.wall_kind = c->wall_kind;
+    aa.ref = t.ref;
+    return aa;
 }
 
 int kgs::ctx_launch_sums(kgs_ctx *c)
 {
     const HostTables &t = c->t;
     if (c->use_acc) {
-        AccSumArgs aa;
-        aa.precision = t.precision;
-        aa.acc = c->acc;
-        aa.nacc = t.nacc;
-        aa.acc_slots = t.acc_slots;
-        aa.raw = c->ax_tab != nullptr;
-        aa.ncell = t.ncell;
-        aa.solid = c->solid;
-        aa.sums = c->sums;
-        aa.coef = c->coef;
-        aa.wall_kind = c->wall_kind;
-        aa.ref = t.ref;
-        KGS_CHECK(launch_acc_sums(aa, c->stream));
+        KGS_CHECK(launch_acc_sums(acc_args(c), c->stream));
     } else {
         PartSumArgs pa;
         pa.ncell = t.ncell;
@@ -413,7 +421,7 @@ int kgs::ctx_launch_sums(kgs_ctx *c)
     return KGS_OK;
 }
 
-int kgs::ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums)
+int kgs::ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums, bool from_acc)
 {
     const HostTables &t = c->t;
     cudaStream_t st = c->stream;
@@ -435,13 +443,34 @@ int kgs::ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums)
     ca.dz = c->ddz;
     ca.solid = c->solid;
     ca.blk_mass = c->blk_mass;
-    KGS_CHECK(launch_closure(ca, st));
-    KGS_CHECK(launch_finalize_mass(c->blk_mass, (int)close_blocks(t.ncell), c->M0, c->mass_rescale, c->scale, st));
-    KGS_CHECK(launch_scale_residual(c->mac_new, c->rho_w_new, c->mac, c->solid, t.ncell, c->scale, c->blk_res,
-                                    c->blk_bad, c->n_red_blocks, st));
-    KGS_CHECK(launch_finalize_residual(c->blk_res, c->blk_bad, c->n_red_blocks, resid_dev, st));
-    c->kernel_launches += 4;
+    if (from_acc)
+        KGS_CHECK(launch_acc_close(acc_args(c), ca, st));
+    else
+        KGS_CHECK(launch_closure(ca, st));
+    ResidualArgs ra;
+    ra.mac_new = c->mac_new;
+    ra.rho_w_new = c->rho_w_new;
+    ra.mac = c->mac;
+    ra.solid = c->solid;
+    ra.ncell = t.ncell;
+    ra.blk_mass = c->blk_mass;
+    ra.n_mass = from_acc ? (int)acc_close_blocks(t.ncell) : (int)close_blocks(t.ncell);
+    ra.M0 = c->M0;
+    ra.rescale = c->mass_rescale;
+    ra.blk_res = c->blk_res;
+    ra.blk_bad = c->blk_bad;
+    ra.count = c->red_count;
+    ra.out = resid_dev;
+    KGS_CHECK(launch_residual(ra, st));
+    c->kernel_launches += 2;
     return KGS_OK;
+}
+
+int kgs::ctx_launch_close(kgs_ctx *c, double *resid_dev)
+{
+    if (c->use_acc) return ctx_launch_closure(c, resid_dev, nullptr, true);
+    const int rc = ctx_launch_sums(c);
+    return rc ? rc : ctx_launch_closure(c, resid_dev, nullptr, false);
 }
 
 void kgs::ctx_finish(kgs_ctx *c, double residual)
@@ -457,9 +486,7 @@ namespace {
 int run_iteration(kgs_ctx *c, double *residual, int *bad)
 {
     int rc;
-    if ((rc = ctx_launch_coef(c)) || (rc = ctx_launch_stages(c)) || (rc = ctx_launch_sums(c)) ||
-        (rc = ctx_launch_closure(c, c->resid, nullptr)))
-        return rc;
+    if ((rc = ctx_launch_coef(c)) || (rc = ctx_launch_stages(c)) || (rc = ctx_launch_close(c, c->resid))) return rc;
     KGS_CHECK(cudaMemcpyAsync(c->h_resid, c->resid, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     KGS_CHECK(cudaStreamSynchronize(c->stream));
     if (c->persist && *reinterpret_cast<const int *>(c->h_resid + 2) != 0) {
@@ -567,7 +594,7 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         (rc = upload(c, &c->d_vgbase, std::vector<int>(t.oct_vgbase, t.oct_vgbase + 8))) ||
         (rc = upload(c, &c->d_vg_oct, t.vg_oct)) || (rc = dalloc_t(c, &c->blk_mass, close_blocks(n))) ||
         (rc = dalloc_t(c, &c->blk_res, (size_t)c->n_red_blocks * 10)) ||
-        (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->scale, 2)) ||
+        (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->red_count, 1)) ||
         (rc = dalloc_t(c, &c->resid, 3)))
         return fail(rc);
     if (t.pack && ((rc = upload(c, &c->lines, t.lines32)) || (rc = upload(c, &c->xnodes, t.xnodes32)) || (rc = dalloc_t(c, &c->rho_w32, 6 * n))))
@@ -593,7 +620,9 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
                          cudaMemset(c->FZ2, 0, (size_t)t.ny * t.nx * t.Nvs * rsz) != cudaSuccess))
         return fail(KGS_ECUDA);
     if (cudaMallocHost(&c->h_resid, 3 * sizeof(double)) != cudaSuccess) return fail(KGS_ENOMEM);
-    if (cudaMemset(c->resid, 0, 3 * sizeof(double)) != cudaSuccess) return fail(KGS_ECUDA);
+    if (cudaMemset(c->resid, 0, 3 * sizeof(double)) != cudaSuccess ||
+        cudaMemset(c->red_count, 0, sizeof(unsigned)) != cudaSuccess)
+        return fail(KGS_ECUDA);
     c->ev.resize(2 * t.stage_n.size());
     for (auto &e : c->ev)
         if (cudaEventCreate(&e) != cudaSuccess) return fail(KGS_ECUDA);
@@ -668,7 +697,7 @@ int kgs_close_sums(kgs_ctx *c, const double *sums_dev, double *residual)
     // the closure takes the lagged velocity centre from the coefficients of
     // this iteration, which kgs_sweep_sums computed
     int rc;
-    if ((rc = ctx_launch_closure(c, c->resid, sums_dev))) return rc;
+    if ((rc = ctx_launch_closure(c, c->resid, sums_dev, false))) return rc;
     KGS_CHECK(cudaMemcpyAsync(c->h_resid, c->resid, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     KGS_CHECK(cudaStreamSynchronize(c->stream));
     const double r = c->h_resid[0];
