@@ -24,10 +24,12 @@
 // copy planes (cp.async, a slot ahead), and four warps read the accumulators
 // of the previous unit with tcgen05.ld (two sets take turns in tensor memory)
 // and apply bias + ReLU, bias only, or the ReLU mask of the backward pass.
-// What bounds it: the tensor core's reads of the shifted windows (their core
-// matrices straddle two 128-byte lines) at about 90 cycles per MMA instead of
-// 56.  With a CTA per unit, which loaded its first planes before and read its
-// accumulators after its MMAs, a unit took 65000 cycles for 378 MMAs.
+// What bounds it: 112 -> 112 channels on 64^3 voxels take 125 us (1.42
+// PFLOP/s), of which the MMAs are 76 us at their rate of 61 cycles; the rest
+// is the weights' stream (12%) and the copies and epilogue beside it.  With a
+// CTA per unit, which loaded its first planes before and read its
+// accumulators after its MMAs, and one thread forming every descriptor anew,
+// the layer took 222 us.
 //
 // The weight gradient (wgrad_tc_kernel) is the per-tap GEMM dW[t][co][ci] =
 // sum over voxels v of dy[v][co] in[v + off(t)][ci], with the output
@@ -139,19 +141,29 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// MMA and commit are issued by one elected lane of a converged warp.  The
+// whole warp runs the issuing loop so that descriptors and addresses stay in
+// uniform registers, where the instruction takes them: from a branch of one
+// thread they are moved there for every MMA, which then cost 128 cycles to
+// issue against the 61 that the tensor core takes (128 x 112 x 16).
 __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
         "setp.ne.u32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
 }
 
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16])
@@ -165,6 +177,27 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// Bounded wait of a whole warp.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+
+// Warp index as a value that the compiler knows to be uniform.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0); }
+
+// Which 16-byte pieces of a voxel row a group of threads copies: eight threads
+// take four channel octets of two neighbouring voxels, so that they read 64
+// contiguous bytes per voxel and, with ten voxels per octet in shared memory,
+// write to eight different 16-byte columns of the banks.
+__host__ __device__ constexpr int row_threads(int X, int C8) { return X / 2 * ((C8 + 3) / 4) * 8; }
+__device__ __forceinline__ void row_piece(int u, int X, int &x, int &c8)
+{
+    const int l = u % 8, g = u / 8;
+    x = g % (X / 2) * 2 + l / 4;
+    c8 = g / (X / 2) * 4 + l % 4;
 }
 
 // Weights W[t][co][ci] -> packed[t][ci/8][co][8]: each tap becomes one
@@ -203,7 +236,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
     const int n_pairs = (int)(u1 - u0);
     const size_t vol = (size_t)dm.D * dm.H * dm.W;
-    const int t = threadIdx.x, warp = t / 32, lane = t % 32;
+    const int t = threadIdx.x, warp = uniform_warp(), lane = t % 32;
     const uint32_t halo_a = smem_u32(sm), w_a = halo_a + HZ * plane_bytes;
     volatile int *fail = &s_fail;  // written by the pipeline threads
     // weight copy T (pair T / 27 of this CTA, tap T % 27) goes through ring slot T % NBUF
@@ -244,7 +277,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
     int issued = -1;  // last weight copy issued (thread 0)
 
     if (t == 0 && RES) {
@@ -264,15 +297,14 @@ __global__ void __launch_bounds__(THREADS, 1)
             bulk_copy(w_a + (uint32_t)(T % NBUF) * w_bytes, wpk + (size_t)(T % 27) * cout_p * dm.cin_p, w_bytes, full(T));
             issued = T;
         }
-    } else if (t == 32) {
+    } else if (warp == 1) {
         // MMA issuer: per tap and channel pair, one MMA of 128 x N x 16 for
-        // each output plane, both reading the same weights.  The thread's own
-        // instruction latency sets the pace of small layers, so descriptors
+        // each output plane, both reading the same weights.  Descriptors
         // advance by additions (their address field counts 16-byte units) and
         // ring slots by counters: with both formed anew for every MMA a step
         // of two MMAs took 300 cycles whatever its size.
         const uint32_t idesc = instr_desc(128, cout_p);
-        const uint64_t a_desc = smem_desc(0, HX * 16, (uint32_t)C8 * HX * 16), a_kc = 2 * HX;
+        const uint64_t a_desc = smem_desc(0, HX * 16, (uint32_t)C8 * HX * 16);
         const uint64_t b_desc = smem_desc(0, (uint32_t)cout_p * 16, 8 * 16), b_kc = 2 * (uint32_t)cout_p;
         const uint32_t halo16 = halo_a >> 4, plane16 = plane_bytes >> 4, row16 = (uint32_t)C8 * HX;
         const int KC = C8 / 2;
@@ -281,26 +313,26 @@ __global__ void __launch_bounds__(THREADS, 1)
         uint32_t phase = 0;
         bool ok = true;
         if (RES) {
-            ok = mbar_wait(smem_u32(&full_bar[0]), 0);
-            if (ok) s_last = 0;
+            ok = warp_wait(smem_u32(&full_bar[0]), 0);
+            if (ok) T = 1;
         }
         for (int j = 0; j < n_pairs && ok; j++) {
             if (j > 0) n0 += fresh(u0 + j) ? 4 : 2;
             const bool end = j + 1 == n_pairs || fresh(u0 + j + 1);  // the column ends here
             const uint32_t acc = tmem + (uint32_t)((j & 1) * OZ * TMEM_HALF);
             // the accumulators of pair j - 2 have been read
-            if (j >= 2) ok = mbar_wait(smem_u32(&acc_empty[j & 1]), (uint32_t)((j - 2) / 2 & 1));
-            ok = ok && mbar_wait(pfull(n0), puse(n0));
+            if (j >= 2) ok = warp_wait(smem_u32(&acc_empty[j & 1]), (uint32_t)((j - 2) / 2 & 1));
+            ok = ok && warp_wait(pfull(n0), puse(n0));
             uint32_t first = 0;  // the pair's first MMA overwrites its accumulator
             for (int kz = 0; kz < 3 && ok; kz++) {
-                ok = !*fail && mbar_wait(pfull(n0 + kz + 1), puse(n0 + kz + 1));
+                ok = warp_wait(pfull(n0 + kz + 1), puse(n0 + kz + 1));
                 tc_fence_after();
                 const uint64_t pa0 = a_desc + halo16 + (uint32_t)((n0 + kz) % HZ) * plane16;      // output z0
                 const uint64_t pa1 = a_desc + halo16 + (uint32_t)((n0 + kz + 1) % HZ) * plane16;  // output z0 + 1
                 for (int ky = 0; ky < 3 && ok; ky++)
                     for (int kx = 0; kx < 3; kx++) {
                         if (!RES) {
-                            if (!ok || *fail || !mbar_wait(smem_u32(&full_bar[slot]), phase)) {
+                            if (!ok || !warp_wait(smem_u32(&full_bar[slot]), phase)) {
                                 ok = false;
                                 break;
                             }
@@ -309,16 +341,16 @@ __global__ void __launch_bounds__(THREADS, 1)
                         uint64_t d0 = pa0 + (uint32_t)ky * row16 + kx, d1 = pa1 + (uint32_t)ky * row16 + kx;
                         uint64_t bd = b_desc + ((w_a + (uint32_t)(RES ? 9 * kz + 3 * ky + kx : slot) * w_bytes) >> 4);
                         for (int kc = 0; kc < KC; kc++) {
-                            tc_mma(acc, d0, bd, idesc, first);
-                            tc_mma(acc + TMEM_HALF, d1, bd, idesc, first);
-                            first = 1;
-                            d0 += a_kc;
-                            d1 += a_kc;
+                            tc_mma(acc, d0, bd, idesc, first | (uint32_t)kc);
+                            tc_mma(acc + TMEM_HALF, d1, bd, idesc, first | (uint32_t)kc);
+                            d0 += 2 * HX;
+                            d1 += 2 * HX;
                             bd += b_kc;
                         }
+                        first = 1;
                         if (!RES) {
                             tc_commit(smem_u32(&empty_bar[slot]));
-                            s_last = T++;
+                            T++;
                             if (++slot == NBUF) slot = 0, phase ^= 1;
                         }
                     }
@@ -333,16 +365,21 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             if (ok) tc_commit(smem_u32(&acc_full[j & 1]));
         }
-        if (!ok) *fail = 1;
         // all MMAs of the CTA are complete once the done barrier has fired
         tc_commit(smem_u32(&done_bar));
-        if (!mbar_wait(smem_u32(&done_bar), 0)) *fail = 1;
+        ok = warp_wait(smem_u32(&done_bar), 0) && ok;
+        if (lane == 0) {
+            s_last = T - 1;
+            if (!ok) *fail = 1;
+        }
     } else if (warp >= FIRST_LOADER) {
         // loaders: a thread keeps its (x, channel octet) and walks down the
         // rows of a plane; whole rows per pass
-        const int lt = t - FIRST_LOADER * 32, per = HX * C8, rows = LOADERS / per;
-        const int r0 = lt / per, c8 = lt % per / HX, px = lt % HX;  // x fastest: conflict-free stores
-        const bool idle = r0 >= rows;
+        const int lt = t - FIRST_LOADER * 32, per = row_threads(HX, C8), rows = LOADERS / per;
+        int px, c8;
+        row_piece(lt % per, HX, px, c8);
+        const int r0 = lt / per;
+        const bool idle = r0 >= rows || c8 >= C8;
         int n = 0;
         bool ok = true;
         auto load = [&](long long u, int p) {  // plane z0 - 1 + p of unit u as plane n
@@ -365,7 +402,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (long long u = u0; u < u1 && ok; u++) {
             for (int p = fresh(u) ? 0 : 2; p < 4; p++, n++) {
                 // plane n reuses the slot of plane n - HZ once no MMA reads it
-                if (n >= HZ && (*fail || !mbar_wait(pempty(n - HZ), puse(n - HZ)))) {
+                if (n >= HZ && (*fail || !warp_wait(pempty(n - HZ), puse(n - HZ)))) {
                     *fail = 1;  // the issuer's wait on this plane then gives up too
                     ok = false;
                     break;
@@ -394,7 +431,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // (output rows) while the MMAs of the next pair run
         const int quad = warp % 4, row = quad * 32 + lane;
         for (int j = 0; j < n_pairs; j++) {
-            if (*fail || !mbar_wait(smem_u32(&acc_full[j & 1]), (uint32_t)(j / 2 & 1))) {
+            if (*fail || !warp_wait(smem_u32(&acc_full[j & 1]), (uint32_t)(j / 2 & 1))) {
                 *fail = 1;
                 break;
             }
@@ -470,23 +507,24 @@ __global__ void __launch_bounds__(THREADS, 1)
 // 8 channels (16 bytes), so tiles move with 16-byte asynchronous copies and
 // need no transpose.  A CTA takes the three taps that share (kz, ky) -- three
 // accumulators in tensor memory -- for a chunk of 8 x 16-voxel tiles.  Per
-// tile it stages dy of the tile, [y][co/8][x][16 B], and rows y0 + ky - 1 ..
+// tile it stages dy of the tile, [y][co/8][x of 10][16 B], and rows y0 + ky - 1 ..
 // y0 + ky + 14, columns x0 - 1 .. x0 + 8 of input plane z + kz - 1,
 // [y][ci/8][x][16 B]; the windows of that block at x offsets 0, 1, 2 are the
 // B operands of the three taps.
 //
-// What bounds it: per tile the tensor core needs about 2000 cycles (24 MMAs of
-// 128 x 112 x 16, whose x-shifted windows read two 128-byte lines per core
-// matrix) and the copies bring 64 KB.  Eight warps only copy and one thread
-// only issues MMAs, through barriers per tile buffer, so neither waits for
-// the other beyond the three buffers.  A copying thread keeps its (x, channel
-// octet) from tile to tile and walks down the rows by adding one stride: with
-// the place of every 16-byte piece recomputed by divisions, and CTA barriers
-// between copies and MMAs, a tile took 4800 cycles even in the smallest layer
-// (8 x 32^3 training step: 2.69 ms of weight gradients).
+// What bounds it: the traffic from L2.  A tile brings 64 KB for 24 MMAs of 128
+// x 112 x 16 (1500 cycles of the tensor core), because tensor memory holds
+// three taps' accumulators and the nine (kz, ky) read the tiles again: 1.2 GB
+// for a 112 -> 112 layer on 8 x 32^3 voxels, 305 us or 3.9 TB/s.  Nine warps
+// only copy and one only issues MMAs, through barriers per tile buffer, so
+// neither waits for the other beyond the three buffers; a copying thread
+// keeps its (x, channel octet) from tile to tile and walks down the rows by
+// adding one stride.  With CTA barriers between copies and MMAs and the place
+// of every 16-byte piece recomputed by divisions the layer took 490 us, and a
+// 16 -> 48 one 297 us instead of 107.
 constexpr int WG_BUF = 3;           // tile buffers
 constexpr int WG_TMEM = 512;        // three accumulators of 128 columns
-constexpr int WG_COPY = 256;        // copying threads: warps 0 .. 7
+constexpr int WG_COPY = 288;        // copying threads: warps 0 .. 8
 constexpr int WG_THREADS = WG_COPY + 32;  // and the warp of the MMA thread
 
 // Voxel tiles of 128 per CTA: chunks as long as 32 tiles, shorter ones where
@@ -509,22 +547,17 @@ __host__ __device__ constexpr uint32_t instr_desc_mn(int M, int N)
 struct WgLayout {
     uint32_t a_bytes, h_bytes, buf_bytes, total;
 };
-// Shared memory of the weight-gradient CTA: WG_BUF x (dy tile, input block),
-// then a pad such that every MMA read stays inside the allocation even if
-// the two descriptor strides were applied the other way round.
+// Shared memory of the weight-gradient CTA: WG_BUF x (dy tile, input block).
+// The MMA reads 16 octets of dy where there are cout_p / 8; the excess lies in
+// the input block behind it and feeds accumulator rows that are not stored.
 __host__ __device__ inline WgLayout wg_layout(int cin_p, int cout_p)
 {
     const int c8o = cout_p / 8, c8i = cin_p / 8;
     WgLayout L;
-    L.a_bytes = (uint32_t)(TY * c8o * TX * 16);
+    L.a_bytes = (uint32_t)(TY * c8o * HX * 16);  // eight voxels in the room of HX (row_piece)
     L.h_bytes = (uint32_t)(TY * c8i * HX * 16);
     L.buf_bytes = L.a_bytes + L.h_bytes;
-    const int over_a = 13 * c8o * 128 + 256 - (int)L.h_bytes;  // past the buffer end, strides swapped
-    const int over_b = c8i * (c8i - 3) * HX * 16 + 2 * HX * 16;
-    int pad = 2048;
-    if (over_a > pad) pad = over_a;
-    if (over_b > pad) pad = over_b;
-    L.total = WG_BUF * L.buf_bytes + (uint32_t)pad + 128;
+    L.total = WG_BUF * L.buf_bytes + 128;
     return L;
 }
 
@@ -545,7 +578,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     const int n_tiles = tiles_x * tiles_y * dm.D;
     const int tile0 = chunk * tiles_per_cta, nt = min(n_tiles, tile0 + tiles_per_cta) - tile0;
     const size_t vol = (size_t)dm.D * dm.H * dm.W;
-    const int t = threadIdx.x, warp = t / 32, lane = t % 32;
+    const int t = threadIdx.x, warp = uniform_warp(), lane = t % 32;
     volatile int *fail = &s_fail;
 
     if (t == 0) {
@@ -566,29 +599,31 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
 
-    if (t < WG_COPY) {
+    if (warp < WG_COPY / 32) {
         // The copying threads split in two parts, one per tensor, in the ratio
         // of their pieces; a part covers whole voxel rows of its block at a
         // time, a thread one (x, octet) of them.
-        const int na = TX * C8o, nh = HX * C8i;  // 16-byte pieces per row
-        const int ra = WG_COPY / (na + nh);             // rows of the dy tile per pass (na + nh <= 252)
+        const int na = row_threads(TX, C8o), nh = row_threads(HX, C8i);
+        const int ra = WG_COPY / (na + nh);             // rows of the dy tile per pass (na + nh <= 288)
         const int rh = (WG_COPY - ra * na) / nh;        // rows of the input block per pass
         const bool is_a = t < ra * na;
         const int u = is_a ? t : t - ra * na;
         const int per = is_a ? na : nh, rows = is_a ? ra : rh, C8 = is_a ? C8o : C8i;
-        const bool idle = u >= rows * per;
-        const int X = is_a ? TX : HX, r0 = u / per, c8 = u % per / X, px = u % X;  // x fastest: conflict-free stores
-        const uint32_t s_off = (is_a ? 0u : L.a_bytes) + (uint32_t)((r0 * C8 + c8) * X + px) * 16;
-        const uint32_t s_step = (uint32_t)(rows * C8 * X) * 16;
+        int px, c8;
+        row_piece(u % per, is_a ? TX : HX, px, c8);
+        const int r0 = u / per;
+        const bool idle = r0 >= rows || c8 >= C8;
+        const uint32_t s_off = (is_a ? 0u : L.a_bytes) + (uint32_t)((r0 * C8 + c8) * HX + px) * 16;
+        const uint32_t s_step = (uint32_t)(rows * C8 * HX) * 16;
         const int cp = is_a ? cout_p : cin_p;
         const __nv_bfloat16 *tensor = (is_a ? dy : in) + (size_t)b * vol * cp + c8 * 8;
         const long long g_step = (long long)rows * dm.W * cp;
         for (int i = 0; i < nt; i++) {
             // tile i reuses the buffer of tile i - WG_BUF: its MMAs must have completed
             if (i >= WG_BUF &&
-                (*fail || !mbar_wait(smem_u32(&empty_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF - 1) & 1))) {
+                (*fail || !warp_wait(smem_u32(&empty_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF - 1) & 1))) {
                 *fail = 1;
                 break;
             }
@@ -615,19 +650,20 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         cp_async_wait<0>();
         fence_async_smem();
         if (nt > 0 && !*fail) mbar_arrive(smem_u32(&full_bar[(nt - 1) % WG_BUF]));
-    } else if (t == WG_COPY) {
+    } else {
         // descriptors advance by additions (16-byte units), as in conv_tc_kernel
         const uint32_t idesc = instr_desc_mn(128, cin_p);
-        const uint64_t a_desc = smem_desc(0, (uint32_t)(C8o * TX * 16), TX * 16), a_ks = 2 * C8o * TX;
+        const uint64_t a_desc = smem_desc(0, (uint32_t)(C8o * HX * 16), HX * 16), a_ks = 2 * C8o * HX;
         const uint64_t b_desc = smem_desc(0, (uint32_t)(C8i * HX * 16), HX * 16), b_ks = 2 * C8i * HX;
         uint32_t first = 0;
+        bool ok = true;
+        int slot = 0;
+        uint32_t phase = 0;
         for (int i = 0; i < nt; i++) {
-            if (*fail || !mbar_wait(smem_u32(&full_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF) & 1)) {
-                *fail = 1;
-                break;
-            }
+            ok = warp_wait(smem_u32(&full_bar[slot]), phase);
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t abuf = base + (uint32_t)(i % WG_BUF) * L.buf_bytes;
+            const uint32_t abuf = base + (uint32_t)slot * L.buf_bytes;
             uint64_t ad = a_desc + (abuf >> 4), bd = b_desc + ((abuf + L.a_bytes) >> 4);
             for (int ks = 0; ks < TY / 2; ks++) {  // K = 16 voxels: tile rows 2ks, 2ks + 1
                 tc_mma(tmem, ad, bd, idesc, first);
@@ -637,11 +673,13 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                 ad += a_ks;
                 bd += b_ks;
             }
-            tc_commit(smem_u32(&empty_bar[i % WG_BUF]));
+            tc_commit(smem_u32(&empty_bar[slot]));
+            if (++slot == WG_BUF) slot = 0, phase ^= 1;
         }
         // every MMA issued has completed once the done barrier fires
         tc_commit(smem_u32(&done_bar));
-        if (!mbar_wait(smem_u32(&done_bar), 0)) *fail = 1;
+        ok = warp_wait(smem_u32(&done_bar), 0) && ok;
+        if (lane == 0 && !ok) *fail = 1;
     }
     __syncthreads();  // the other threads wait here, not polling; s_fail is uniform after it
     tc_fence_after();
