@@ -17,21 +17,6 @@ double maxwellian(double rho, const double U[3], double T, const double xi[3])
 
 }  // namespace
 
-void pack_order(int v0, int count, int nxo, std::vector<int> &place)
-{
-    place.clear();
-    for (int half = 0; half < 2; half++) {
-        const int b = half * NT, n = std::min(NT, count - b);
-        if (n <= 0) break;
-        const int head = std::min(n, (nxo - (v0 + b) % nxo) % nxo), full = (n - head) / nxo, pairs = full / 2;
-        for (int q = 0; q < pairs; q++)
-            for (int ix = 0; ix < nxo; ix++)
-                for (int h = 0; h < 2; h++) place.push_back(b + head + (2 * q + h) * nxo + ix);
-        for (int v = 0; v < head; v++) place.push_back(b + v);
-        for (int v = head + 2 * pairs * nxo; v < n; v++) place.push_back(b + v);
-    }
-}
-
 bool dev_source_applies(const kgs_grid *grid, const kgs_bc *bc)
 {
     for (int s = 0; s < 6; s++)

@@ -9,6 +9,7 @@
 
 #include "../../include/kgs.h"
 #include "kgs_internal.h"
+#include "kgs_pack.h"
 
 namespace kgs {
 
@@ -112,14 +113,6 @@ struct HostTables {
 int validate_problem(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid *vg, const kgs_gas *gas,
                      const kgs_bc *bc, int precision, int wall_norm, int v_per_cta, int block_z, int vz_begin = 0,
                      int vz_end = 0, int order = 1, int dev_source = 0);
-
-// Natural places (0 .. count-1, ix fastest) of the slots of one packed velocity
-// group that starts at place v0 of its octant, lines of nxo nodes.  Each half
-// of the group (the velocities one thread of the moment phase sums) holds, in
-// this order: its pairs of whole lines with the two lines interleaved node by
-// node, the line its start cuts (head), an unpaired whole line, and the line
-// its end cuts (tail).
-void pack_order(int v0, int count, int nxo, std::vector<int> &place);
 
 // The deviation-form FP32 source applies: equal widths along each axis and
 // no free-stream side (the reference Maxwellian is the rest state).
