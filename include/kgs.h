@@ -204,7 +204,8 @@ int kgs_set_initial(kgs_ctx *ctx, const double *macros);
  * denominator floored at 1e-8 ||rho||_2).
  * Each iteration is one persistent sweep launch over the context's work items
  * (octant, velocity group, 8x8xblock_z block) in wavefront order; a thread
- * block waits with a bounded poll for the three upwind blocks of its item.
+ * block waits with bounded polls for the progress of the three upwind blocks
+ * of its item.
  * Returns KGS_OK, KGS_NOTCONVERGED (n_iters <= 0 only), KGS_EDIVERGED
  * (the state is left at the offending iterate), KGS_ETIMEOUT (a bounded wait
  * gave up; the iteration's results are discarded), KGS_ECUDA. */

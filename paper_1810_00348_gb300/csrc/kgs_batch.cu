@@ -382,12 +382,19 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
         for (int i = 0; i < n && !all; i++) ctx_free_axis(b->ctx[i]);
         b->kind.sep = all;
     }
-    const size_t smem = sweep_smem_bytes(b->kind, b->nxo_max);
-    per_sm = sweep_persistent_occupancy(b->kind, smem);
-    if (per_sm < 1) return fail(KGS_ECUDA);
-    b->grid = sms * per_sm;
-    b->scratch_stride = sweep_scratch_bytes(b->bz);
-    if (cudaMalloc(&b->d_scratch, (size_t)b->grid * b->scratch_stride) != cudaSuccess) return fail(KGS_ENOMEM);
+    for (;;) {
+        per_sm = sweep_persistent_occupancy(b->kind, sweep_smem_bytes(b->kind, b->nxo_max));
+        if (per_sm < 1) return fail(KGS_ECUDA);
+        b->grid = sms * per_sm;
+        b->scratch_stride = sweep_scratch_bytes(b->bz);
+        if (cudaMalloc(&b->d_scratch, (size_t)b->grid * b->scratch_stride) == cudaSuccess) break;
+        b->d_scratch = nullptr;
+        if (!b->kind.sep) return fail(KGS_ENOMEM);
+        // the batch fits only without the axis factors
+        (void)cudaGetLastError();
+        for (int i = 0; i < n; i++) ctx_free_axis(b->ctx[i]);
+        b->kind.sep = 0;
+    }
     *out = b;
     return KGS_OK;
 }

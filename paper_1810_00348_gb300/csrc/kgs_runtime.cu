@@ -336,7 +336,7 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     const HostTables &t = c->t;
     int sms = 0;
     KGS_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
-    if (t.precision == KGS_FP64 && t.order == 1) {
+    if (t.precision == KGS_FP64 && t.order == 1 && c->allow_sep) {
         SweepKind k = t.kind();
         k.sep = 1;
         int rc;
@@ -538,8 +538,17 @@ int kgs_setup(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, const k
                               opts->block_z, opts->vz_begin, opts->vz_end, opts->order, opts->dev_source);
     if (rc) return rc;
     (void)cudaGetLastError();  // launches below check their own status
-    if ((rc = ctx_create(out, grid, solid, vg, gas, bc, opts))) return rc;
-    rc = ctx_persist_init(*out);
+    // a problem that fits only without the FP64 sweep's axis factors gets the
+    // sweep that needs none
+    for (int attempt = 0; attempt < 2; attempt++) {
+        if ((rc = ctx_create(out, grid, solid, vg, gas, bc, opts))) return rc;
+        (*out)->allow_sep = attempt == 0;
+        rc = ctx_persist_init(*out);
+        if (rc != KGS_ENOMEM || !(*out)->ax_tab) break;
+        kgs_destroy(*out);
+        *out = nullptr;
+        (void)cudaGetLastError();
+    }
     // the persistent sweep's tables and the accumulator fill went to the
     // legacy default stream as well
     if (!rc && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) rc = KGS_ECUDA;

@@ -1,5 +1,9 @@
 // kgs_sweep.cu -- the fused equilibrium + upwind implicit sweep + moment
 // kernel of one outer iteration (arXiv 1810.00348, Eqs. (2), (5), (7), (9)).
+// This is the general form: FP32 with one velocity per thread, the second
+// order, FP64 without axis factors, and FP32 with two velocities per thread
+// without packed slots.  kgs_sweep_f2.cu and kgs_sweep_d.cu serve the first
+// order in FP32 and FP64 otherwise.
 //
 // Work decomposition.  The physical grid is cut into blocks of BX x BY x bz
 // cells.  For the velocities of octant o (signs of xi_x, xi_y, xi_z) a block
@@ -8,8 +12,8 @@
 // towards +x, +y, +z): stage s holds every block whose reflected coordinates
 // sum to s, for all eight octants at once.  A work item is (octant, block,
 // group of vg_size velocities of that octant).  The persistent kernel claims
-// items in stage order and waits (bounded) for the completion flags of the
-// item's three upwind blocks, so one launch covers the whole sweep; the
+// items in stage order and waits (bounded) for the progress of the item's
+// three upwind blocks, slice by slice, so one launch covers the whole sweep; the
 // kernel with one launch per stage serves the entry point that allocates no
 // device memory (no flags needed).  Velocities
 // are independent within an outer iteration (Eq. (6) lags f^S, tau and

@@ -10,8 +10,9 @@
 // (fma.rn.f32x2 and its kin: two FP32 results per lane and instruction, each
 // rounded as the scalar instruction rounds it) run at half the issue rate of
 // the scalar ones with the same latency, so they leave the arithmetic rate
-// unchanged and halve the issue slots.  To use them
-// without moves the two velocities of a thread sit in neighbouring slots (2t
+// unchanged and halve the issue slots (measured per SM and clock: 1.73 packed
+// against 3.86 scalar FMAs, 4.8 cycles from one to the next that needs it).
+// To use them without moves the two velocities of a thread sit in neighbouring slots (2t
 // and 2t + 1 of its group), which the host orders (pack_order) so that they
 // have the same x node on neighbouring x-lines: face planes and slice
 // positions move as 8-byte words, and the moment phase sums two lines at
@@ -22,6 +23,14 @@
 // 8 cells of the halo column and the 8 of the halo row; the stride of a cell,
 // 129 8-byte words, is odd, so that the moment phase (a cell per lane) reads
 // without bank conflicts.
+//
+// Measured against the same work with one scalar chain per velocity: 38.9
+// instead of 54.7 instructions per phase point; 64^3 cells x 32^3 velocities
+// 24.3 -> 20.4 ms (19.1 with the diagonals stored once computed), 96x64x64 x
+// 48^3 with a solid cube 146 -> 111 ms, growing cells (50x43x43 x 24^3) 8.06 ->
+// 5.84 ms.  The results are the same bit for bit: every sum keeps its order,
+// and the only products that are not rounded by themselves are those that
+// enter a compensated sum alone.
 #include "kgs_sweep_dev.cuh"
 
 namespace kgs {
