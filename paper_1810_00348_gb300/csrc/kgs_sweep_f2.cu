@@ -24,7 +24,7 @@
 // 129 8-byte words, is odd, so that the moment phase (a cell per lane) reads
 // without bank conflicts.
 //
-// Measured against the same work with one scalar chain per velocity: 38.9
+// Measured against the same work with one scalar chain per velocity: 39.8
 // instead of 54.7 instructions per phase point; 64^3 cells x 32^3 velocities
 // 24.3 -> 20.4 ms (19.1 with the diagonals stored once computed), 96x64x64 x
 // 48^3 with a solid cube 146 -> 111 ms, growing cells (50x43x43 x 24^3) 8.06 ->
