@@ -31,6 +31,7 @@
 // 5.84 ms.  The results are the same bit for bit: every sum keeps its order,
 // and the only products that are not rounded by themselves are those that
 // enter a compensated sum alone.
+#include "kgs_pack.h"
 #include "kgs_sweep_dev.cuh"
 
 namespace kgs {
@@ -213,13 +214,13 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
         const float4 *xs = reinterpret_cast<const float4 *>(a.xnodes) + (size_t)o * a.xn_stride;
         for (int ix = t; ix < nxo; ix += NT) xn[ix] = xs[ix];
     }
-    // the half of the group that this thread sums in the moment phase: see
-    // pack_order for the order of its slots
+    // the half of the group that this thread sums in the moment phase
+    static_assert(PACK_HALF == NT, "a thread sums one half of the group");
     const int mcl = t % SLICE, mvp = t / SLICE;  // NT = 2 * SLICE
     const int mb = mvp * NT, mn = min(NT, nvg - mb);
-    const int head = mn > 0 ? min(mn, (nxo - (v0 + mb) % nxo) % nxo) : 0;
-    const int full = mn > 0 ? (mn - head) / nxo : 0;
-    const int tail = mn > 0 ? mn - head - full * nxo : 0;
+    const PackHalf half(v0 + mb, mn, nxo);
+    const int head = half.head, full = half.full, tail = half.tail;
+    const int first = LINE > 0 ? nxo - head : half.first;  // node of the head's first velocity (16: no line is cut)
     const int mline = mn > 0 ? (v0 + mb) / nxo - line0 : 0;  // line of its first velocity
 
     // the persistent sweep reads the wall densities in FP32: converting them
@@ -536,9 +537,7 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
                 }
                 const float *hc = cxh + cl * cxs, *lc = cxl + cl * cxs;
                 const float2 *sp = slice + cl * CSP + mb / 2;
-                // the units of the half in line order: the line that its start
-                // cuts, the pairs of whole lines, an odd whole line, the line
-                // that its end cuts
+                // the units of the half in line order (PackHalf)
                 const int pairs = full / 2;
                 const int n_units = (head > 0) + pairs + (full & 1) + (tail > 0);
                 const float *seq = reinterpret_cast<const float *>(sp + pairs * nxo);  // the unpaired ones
@@ -558,7 +557,7 @@ __device__ __forceinline__ void sweep_item2(const SweepArgs &a, const int4 w, co
                         }
                     } else {
                         const int n = k < 0 ? head : (k == pairs && (full & 1)) ? nxo : tail;
-                        const int ix0 = k < 0 ? nxo - head : 0;
+                        const int ix0 = k < 0 ? first : 0;
                         for (int ix = ix0; ix < ix0 + n; ix++) {
                             float hi, lo;
                             if constexpr (LINE > 0) {
