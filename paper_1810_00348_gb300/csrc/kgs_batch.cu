@@ -253,7 +253,7 @@ bool batch_step(kgs_batch *b, bool retire, std::vector<int> &count, std::vector<
         const double r = b->h_resid[2 * i];
         bad |= b->h_resid[2 * i + 1] != 0.0;
         ctx_finish(b->ctx[i], r);
-        b->kernel_launches += b->ctx[i]->ax_tab ? 4 : 3;  // coefficients, axis factors (FP64), closure, residual
+        b->kernel_launches += b->ctx[i]->ax_tab ? 5 : 3;  // coefficients, axis factors and centres (FP64), closure, residual
         count[i]++;
         b->done[i]++;
         last[i] = r;

@@ -297,7 +297,8 @@ __global__ void __launch_bounds__(CLOSE_CELLS * NPART) part_sums_kernel(const Pa
     }
 }
 
-// The 13 sums about 0 -> the sums about U: c = xi - U expanded in each.
+// The 13 sums about some velocity -> the sums about that velocity + U: c - U
+// expanded in each.
 __device__ __forceinline__ void shift_sums(double (&s)[SUM_F0], const double U[3])
 {
     const double S0 = s[P_S0], S1[3] = {s[P_S1X], s[P_S1Y], s[P_S1Z]};
@@ -377,11 +378,15 @@ __device__ __forceinline__ void cell_sums(const AccSumArgs &a, size_t c, const d
         ref_slots(a.ref, U, ref);
 #pragma unroll
         for (int q = 0; q < SUM_F0; q++) s[q] += ref[q];
-    } else if (a.raw) {
+    } else if (a.centre) {
         double U[3];
         const double *cf = static_cast<const double *>(a.coef) + c * NCOEF;
-        for (int d = 0; d < 3; d++) U[d] = -0.5 * cf[C_M2UX + d];
-        shift_sums(s, U);
+        const int i = (int)(c % a.nx), j = (int)(c / a.nx % a.ny), k = (int)(c / ((size_t)a.nx * a.ny));
+        const double *cen = a.centre + slice_centre(i, j, k, a.nx, a.ny);
+        if (cen[3] == 0.0) {
+            for (int d = 0; d < 3; d++) U[d] = -0.5 * cf[C_M2UX + d] - cen[d];
+            shift_sums(s, U);
+        }
     }
 #pragma unroll
     for (int q = 0; q < SUM_F0; q++) S[q] = s[q];

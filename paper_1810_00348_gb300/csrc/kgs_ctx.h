@@ -29,6 +29,7 @@ struct kgs_ctx {
     bool allow_sep = true;                                // may use the separated FP64 sweep
     void *ax_tab = nullptr;                               // separated FP64 sweep: axis factors (null: not used)
     double *ax_nodes = nullptr;                           // HostTables::ax_nodes
+    double *centre = nullptr;                             // SweepArgs::centre
     float *lines = nullptr, *xnodes = nullptr;            // packed FP32 sweep: HostTables::lines32, xnodes32
     float *rho_w32 = nullptr;                             // packed FP32 sweep: rho_w in FP32
     void *FX2 = nullptr, *FY2 = nullptr, *FZ2 = nullptr;  // second face planes of the order-2 sweep

@@ -111,6 +111,9 @@ struct SweepArgs {
     const void *ax_tab;           // separated FP64 sweep: double4[ncell][ax_n] axis factors (kgs_sweep_d.cu)
     int ax_n, ax_nx, ax_ny;       // nodes of the three axes, of x and of y, in HostTables::ax_nodes order
     int ax_neg[3];                // negative nodes of each axis (they come first)
+    const double *centre;         // separated FP64 sweep: [nz][nby][nbx][4] the velocity about which the sums of
+                                  // the cells of one block's slice are taken and, if not 0 in the fourth place,
+                                  // that each cell's are about its own U^n instead (slice_centre)
     int nxo_max;                  // max over octants of oct_nx
     int any_solid;                // the problem has solid cells
     const uint8_t *blk_plain;     // [nbz][nby][nbx]: 1 = no solid cell and no solid neighbour in the block (or NULL)
@@ -234,6 +237,13 @@ int sweep_d_occupancy(const SweepKind &k, size_t smem);
 cudaError_t launch_sweep_d(const SweepKind &k, const BatchSweepArgs &b, int nxo_max, int grid, cudaStream_t s);
 cudaError_t launch_axis_tables(const void *coef, const double *nodes, unsigned long long ncell, int nvx, int nvy,
                                int na, void *tab, cudaStream_t s);
+cudaError_t launch_slice_centres(const void *coef, int nx, int ny, int nz, double *centre, cudaStream_t s);
+// Entry of SweepArgs::centre for cell (i, j, k) of an nx x ny x nz grid.
+__host__ __device__ inline size_t slice_centre(int i, int j, int k, int nx, int ny)
+{
+    const int nbx = (nx + BX - 1) / BX, nby = (ny + BY - 1) / BY;
+    return (((size_t)k * nby + j / BY) * nbx + i / BX) * 4;
+}
 
 // The packed FP32 kernels (k.pack), reached through the functions above.
 size_t sweep2_smem_bytes(const SweepKind &k, int nxo_max);
@@ -290,7 +300,8 @@ struct AccSumArgs {
     const void *acc;
     int nacc;
     int acc_slots;
-    int raw;                      // FP64: the accumulated sums are about 0, not about U^n
+    const double *centre;         // FP64: about what the accumulated sums are (SweepArgs::centre); NULL: about U^n
+    int nx, ny;
     unsigned long long ncell;
     const uint8_t *solid;         // [ncell] or NULL
     double *sums;                 // [NSUM][ncell]

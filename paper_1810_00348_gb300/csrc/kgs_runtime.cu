@@ -168,6 +168,7 @@ SweepArgs kgs::ctx_sweep_args(const kgs_ctx *c)
     a.ax_nx = t.ax_nx;
     a.ax_ny = t.ax_ny;
     for (int d = 0; d < 3; d++) a.ax_neg[d] = t.ax_neg[d];
+    a.centre = c->centre;
     a.any_solid = t.any_solid ? 1 : 0;
     a.blk_plain = c->blk_plain;
     a.coef = c->coef;
@@ -203,7 +204,8 @@ int kgs::ctx_launch_coef(kgs_ctx *c)
     if (c->ax_tab) {
         KGS_CHECK(launch_axis_tables(c->coef, c->ax_nodes, t.ncell, t.ax_nx, t.ax_ny, (int)t.ax_nodes.size(),
                                      c->ax_tab, c->stream));
-        c->kernel_launches += 1;
+        KGS_CHECK(launch_slice_centres(c->coef, t.nx, t.ny, t.nz, c->centre, c->stream));
+        c->kernel_launches += 2;
     }
     return KGS_OK;
 }
@@ -215,10 +217,13 @@ SweepKind kgs::ctx_kind(const kgs_ctx *c)
     return k;
 }
 
+static size_t centre_values(const HostTables &t) { return (size_t)t.nbx * t.nby * t.nz * 4; }
+
 int kgs::ctx_alloc_axis(kgs_ctx *c)
 {
     const HostTables &t = c->t;
     int rc = upload(c, &c->ax_nodes, t.ax_nodes);
+    if (!rc) rc = dalloc_t(c, &c->centre, centre_values(t));
     if (!rc) rc = dalloc(c, &c->ax_tab, t.ncell * t.ax_nodes.size() * 4 * sizeof(double));
     if (rc == KGS_ENOMEM) {
         // the sweep that needs no axis factors serves a problem whose factors do not fit
@@ -231,14 +236,16 @@ int kgs::ctx_alloc_axis(kgs_ctx *c)
 
 void kgs::ctx_free_axis(kgs_ctx *c)
 {
-    for (void *p : {static_cast<void *>(c->ax_nodes), c->ax_tab}) {
+    for (void *p : {static_cast<void *>(c->ax_nodes), static_cast<void *>(c->centre), c->ax_tab}) {
         if (!p) continue;
         c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
         cudaFree(p);
     }
     if (c->ax_tab) c->device_bytes -= c->t.ncell * c->t.ax_nodes.size() * 4 * sizeof(double);
     if (c->ax_nodes) c->device_bytes -= c->t.ax_nodes.size() * sizeof(double);
+    if (c->centre) c->device_bytes -= centre_values(c->t) * sizeof(double);
     c->ax_tab = nullptr;
+    c->centre = nullptr;
     c->ax_nodes = nullptr;
 }
 
@@ -388,7 +395,9 @@ static AccSumArgs acc_args(const kgs_ctx *c)
     aa.acc = c->acc;
     aa.nacc = t.nacc;
     aa.acc_slots = t.acc_slots;
-    aa.raw = c->ax_tab != nullptr;
+    aa.centre = c->centre;
+    aa.nx = t.nx;
+    aa.ny = t.ny;
     aa.ncell = t.ncell;
     aa.solid = c->solid;
     aa.sums = c->sums;

@@ -22,19 +22,26 @@
 //  * f = num / den from the hardware reciprocal r (relative error below
 //    2^-20): with e = 1 - den r, f = q + q (e + e^2), q = num r, is off by
 //    e^3: four operations instead of six.
-//  * The moment sums are raw (about 0, not about U^n), so that the weights of
-//    a node are table entries: four multiply-adds per velocity for
-//    P_a = sum w_x xi_x^a f along a line, 16 per line for the 13 sums.  The
-//    sums kernel shifts them to U^n.  The incoming wall flux of an octant
+//  * The moment sums of a slice are about one velocity C, the middle of the
+//    range of U^n over its fluid cells, so that the weights of a node are table
+//    entries: four multiply-adds per velocity for P_a = sum w_x (xi_x - C_x)^a f
+//    along a line, 16 per line for the 13 sums.  The sums kernel shifts them to
+//    U^n, which costs no digits while U^n is near C.  A slice over which U^n
+//    varies by more than CENTRE_RANGE of the thermal speed either way (a shock,
+//    the front of a body) is summed about each cell's own U^n: eight operations
+//    per velocity, 24 per line.  About 0 the shift subtracts terms of size
+//    rho |U|^3, which left the heat flux of a Mach 2 stream 17 times and of a
+//    Mach 5 stream 280 times further off.  The incoming wall flux of an octant
 //    along d is its first moment along d up to sign.
 //
 // Cells are visited row by row: with the pipe saturated by one chain there is
 // nothing to gain from independent cells.
 //
-// Measured: 32^3 cells x 32^3 velocities 87.2 -> 35.1 ms (30.7 ms are the 18
-// operations at the pipe's rate), 27x19x22 x 17x14x20 19.3 -> 3.9 ms (with the
-// overlap of neighbouring blocks), error against a 64-bit evaluation unchanged
-// (4e-15 of the fields).
+// Measured: 32^3 cells x 32^3 velocities 87.2 -> 35.6 ms (30.7 ms are the 18
+// operations at the pipe's rate), 27x19x22 x 17x14x20 19.3 -> 4.0 ms (with the
+// overlap of neighbouring blocks).  Error of the heat flux against extended
+// precision as with every sum about U^n: 8.7e-16 (8.6e-16) around a cube at
+// Mach 2, 4.3e-14 (4.2e-14) in a Mach 2 stream, 1.3e-13 (1.6e-13) at Mach 5.
 #include "kgs_sweep_dev.cuh"
 
 namespace kgs {
@@ -43,14 +50,21 @@ namespace {
 constexpr int VG = NT;           // velocities per group
 constexpr int CS = VG + 1;       // odd stride of a cell: conflict-free per-cell reads
 constexpr int HCOL = SLICE, HROW = SLICE + BY, NPOS = SLICE + BY + BX;
-constexpr int LW = 10;           // line weights: W, Wy, Wz, Wyy, Wzz, Wyz, Wr, Wry, Wrz (r = y^2 + z^2), -
+constexpr int XW = 6;            // of an x node: w x^a (x about the slice's centre, a < 4), xi_x, w_x
+constexpr int LW = 12;           // of a line: W, Wy, Wz, Wyy, Wzz, Wyz, Wr, Wry, Wrz (r = y^2 + z^2; y and z about
+                                 // the slice's centre), xi_y, xi_z, W = w_y w_z
+// Largest distance of U^n from the centre of its slice, in thermal speeds of
+// the coldest cell: at 1/8 the sums are as exact as about U^n itself (heat
+// flux off by 1.0 to 1.1 times as much over random fields), at 0.45 1.8 times.
+constexpr double CENTRE_RANGE = 0.125;
 static_assert(BX * CS >= NPART * SLICE, "reduction buffer in the halo row");
 
 struct LayoutD {
     static constexpr size_t off_cell = align16(sizeof(double) * NPOS * CS);  // [SLICE][4] 1/tau, 1/dx, 1/dy, 1/dz
     static constexpr size_t off_flag = off_cell + sizeof(double) * SLICE * 4;
-    static constexpr size_t off_x = off_flag + sizeof(int) * SLICE;           // [nxm][4] w_x xi_x^a
-    __host__ __device__ static size_t off_line(int nxm) { return off_x + sizeof(double) * 4 * nxm; }
+    static constexpr size_t off_cen = off_flag + sizeof(int) * SLICE;         // [2][4] centre of this and the next slice
+    static constexpr size_t off_x = off_cen + sizeof(double) * 8;             // [nxm][6] w_x (xi_x - C_x)^a, xi_x, w_x
+    __host__ __device__ static size_t off_line(int nxm) { return off_x + sizeof(double) * XW * nxm; }
     __host__ __device__ static size_t off_h(int nxm, int lines_max)           // [SLICE][lines_max][4]
     {
         return off_line(nxm) + align16(sizeof(double) * LW * lines_max);
@@ -90,6 +104,39 @@ __global__ void __launch_bounds__(256)
     tab[i] = out;
 }
 
+// SweepArgs::centre: the middle of the range of U^n over the fluid cells of
+// each block's slice (0 without any), and whether U^n is too far from it
+// (CENTRE_RANGE) somewhere.
+__global__ void __launch_bounds__(SLICE)
+    centre_kernel(const double *__restrict__ coef, int nx, int ny, double *__restrict__ centre)
+{
+    __shared__ double lo[4][2], hi[4][2];
+    const int nbx = (nx + BX - 1) / BX, nby = (ny + BY - 1) / BY;
+    const int bx = blockIdx.x % nbx, by = blockIdx.x / nbx % nby, k = blockIdx.x / (nbx * nby);
+    const int t = threadIdx.x, i = bx * BX + t % BX, j = by * BY + t / BX;
+    const double *r = coef + ((size_t)i + (size_t)nx * (j + (size_t)ny * k)) * NCOEF;
+    const bool fluid = i < nx && j < ny && !(flag_bits(r[C_FLAGS]) & F_SOLID);
+    for (int d = 0; d < 4; d++) {  // U^n along the axes, 1/(RT)
+        const double v = fluid ? (d < 3 ? -0.5 * r[C_M2UX + d] : r[C_RT1]) : 0.0;
+        double a = fluid ? v : INFINITY, b = fluid ? v : -INFINITY;
+        for (int off = 16; off > 0; off >>= 1) {
+            a = fmin(a, __shfl_xor_sync(0xffffffffu, a, off));
+            b = fmax(b, __shfl_xor_sync(0xffffffffu, b, off));
+        }
+        if (t % 32 == 0) lo[d][t / 32] = a, hi[d][t / 32] = b;
+    }
+    __syncthreads();
+    if (t > 0) return;
+    double far2 = 0.0, *out = centre + (size_t)blockIdx.x * 4;
+    for (int d = 0; d < 3; d++) {
+        const double a = fmin(lo[d][0], lo[d][1]), h = 0.5 * (fmax(hi[d][0], hi[d][1]) - a);
+        out[d] = h >= 0.0 ? a + h : 0.0;
+        far2 += h * h;
+    }
+    const double rt1 = fmax(hi[3][0], hi[3][1]);  // of the coldest cell, thermal speed^2 = 2 / rt1
+    out[3] = rt1 > 0.0 && !(far2 * rt1 <= 2.0 * CENTRE_RANGE * CENTRE_RANGE) ? 1.0 : 0.0;
+}
+
 __device__ __forceinline__ double4 ld_rec(const double4 *p)
 {
     const double2 *q = reinterpret_cast<const double2 *>(p);
@@ -104,6 +151,7 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
     double *slice = reinterpret_cast<double *>(smem);
     double *cell4 = reinterpret_cast<double *>(smem + LayoutD::off_cell);
     int *cflag = reinterpret_cast<int *>(smem + LayoutD::off_flag);
+    double *cen2 = reinterpret_cast<double *>(smem + LayoutD::off_cen);
     double *wxp = reinterpret_cast<double *>(smem + LayoutD::off_x);
     double *lw = reinterpret_cast<double *>(smem + LayoutD::off_line(a.nxo_max));
     double *H = reinterpret_cast<double *>(smem + LayoutD::off_h(a.nxo_max, lines_max));
@@ -165,30 +213,56 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
     }
     const double mgx = mt[(size_t)(a.side_inflow[sidex] ? MT_INFLOW : sidex) * Nv + gv];
     const double mgy = mt[(size_t)(a.side_inflow[sidey] ? MT_INFLOW : sidey) * Nv + gv];
-    // moment weights of the octant's x nodes and of the group's lines
+    // nodes of the moment phase
     for (int ix = t; ix < nxo; ix += NT) {
         const size_t g = (size_t)a.oct_vstart[o] + ix;  // the octant's first line
-        const double x = vel[g * 4], wx = static_cast<const double *>(a.velm)[g * 8];
-        wxp[ix * 4 + 0] = wx;
-        wxp[ix * 4 + 1] = wx * x;
-        wxp[ix * 4 + 2] = wx * x * x;
-        wxp[ix * 4 + 3] = wx * x * x * x;
+        wxp[ix * XW + 4] = vel[g * 4];
+        wxp[ix * XW + 5] = static_cast<const double *>(a.velm)[g * 8];
     }
     for (int l = t; l < nlines; l += NT) {
         const size_t g = (size_t)a.oct_vstart[o] + (size_t)(line0 + l) * nxo;
-        const double y = vel[g * 4 + 1], z = vel[g * 4 + 2], W = static_cast<const double *>(a.velm)[g * 8 + 1];
-        const double r = y * y + z * z;
-        double *e = lw + l * LW;
-        e[0] = W;
-        e[1] = W * y;
-        e[2] = W * z;
-        e[3] = W * y * y;
-        e[4] = W * z * z;
-        e[5] = W * y * z;
-        e[6] = W * r;
-        e[7] = W * y * r;
-        e[8] = W * z * r;
+        lw[l * LW + 9] = vel[g * 4 + 1];
+        lw[l * LW + 10] = vel[g * 4 + 2];
+        lw[l * LW + 11] = static_cast<const double *>(a.velm)[g * 8 + 1];
     }
+    auto load_centre = [&](int lk) {
+        if (t < 4) cen2[lk % 2 * 4 + t] = a.centre[slice_centre(GX(0), GY(0), GZ(lk), nx, ny) + t];
+    };
+    // their weights about a slice's centre: warp 0 the x nodes, the others a
+    // third of every line's, so that no warp runs a long chain before the sweep
+    auto build_weights = [&](const double *cen) {
+        const int part = t / 32, lane = t % 32;
+        if (part == 0) {
+            for (int ix = lane; ix < nxo; ix += 32) {
+                double *e = wxp + ix * XW;
+                const double x = e[4] - cen[0], wx = e[5], x2 = x * x;
+                e[0] = wx;
+                e[1] = wx * x;
+                e[2] = wx * x2;
+                e[3] = wx * x * x2;
+            }
+            return;
+        }
+        for (int l = lane; l < nlines; l += 32) {
+            double *e = lw + l * LW;
+            const double y = e[9] - cen[1], z = e[10] - cen[2], W = e[11];
+            if (part == 1) {
+                e[0] = W;
+                e[1] = W * y;
+                e[3] = W * y * y;
+                e[5] = W * y * z;
+            } else if (part == 2) {
+                e[2] = W * z;
+                e[4] = W * z * z;
+                e[6] = W * (y * y + z * z);
+            } else {
+                const double Wr = W * (y * y + z * z);
+                e[7] = Wr * y;
+                e[8] = Wr * z;
+            }
+        }
+    };
+    load_centre(0);
     // the half of the group that this thread sums in the moment phase
     const int mcl = t % SLICE, mvp = t / SLICE;  // NT = 2 * SLICE
     const int mb = mvp * (VG / 2), me = min(mb + VG / 2, nvg);
@@ -317,6 +391,10 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
         if (t == 0) pipe.wait(min(lk + 2, ez));
         __syncthreads();
         if (lk + 1 < ez) prefetch(lk + 1);
+        // the moment phase sums about one velocity of the slice or about U^n
+        const double *cen = cen2 + lk % 2 * 4;
+        const bool shared_centre = cen[3] == 0.0;
+        if (shared_centre) build_weights(cen);  // read after the next barrier
 
         // ---- sweep of the slice: Eq. (2) fused into Eq. (7), row by row ----
         // the G records of the next two cells are in flight
@@ -396,25 +474,29 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
         }
         __syncthreads();
         if (t == 0) pipe.announce(lk + 1, ez);
-        if (lk + 1 < ez) build_h(lk + 1);
+        if (lk + 1 < ez) {
+            build_h(lk + 1);
+            load_centre(lk + 1);
+        }
 
-        // ---- raw moments of the slice over the group's velocities ----
+        // ---- moments of the slice about its centre over the group's velocities ----
         const int li = mcl % BX, lj = mcl / BX;
         const int flags = cflag[mcl];
         const bool live = li < ex && lj < ey && !(flags & F_SOLID);
         double S[P_FX];
 #pragma unroll
         for (int q = 0; q < P_FX; q++) S[q] = 0.0;
-        if (live) {
+        const double *m2u = coef + CELL(GX(li), GY(lj), z) * NCOEF + C_M2UX;  // -2 U^n, read where live
+        if (live && shared_centre) {
             const double *sp = slice + mcl * CS;
             int v = mb, ix = (v0 + mb) % nxo, l = (v0 + mb) / nxo - line0;
             while (v < me) {
                 // the part of line l in this half
                 const int end = min(me, v + nxo - ix);
                 double P0 = 0.0, P1 = 0.0, P2 = 0.0, P3 = 0.0;
-                const double2 *wp = reinterpret_cast<const double2 *>(wxp) + 2 * ix;
+                const double2 *wp = reinterpret_cast<const double2 *>(wxp + XW * ix);
 #pragma unroll 4
-                for (; v < end; v++, wp += 2) {
+                for (; v < end; v++, wp += XW / 2) {
                     const double f = sp[v];
                     const double2 w01 = wp[0], w23 = wp[1];
                     P0 = fma(w01.x, f, P0);
@@ -441,9 +523,45 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
                 ix = 0;
                 l++;
             }
+        } else if (live) {
+            const double cx = -0.5 * m2u[0], cy = -0.5 * m2u[1], cz = -0.5 * m2u[2];
+            const double *sp = slice + mcl * CS;
+            int v = mb, ix = (v0 + mb) % nxo, l = (v0 + mb) / nxo - line0;
+            while (v < me) {
+                const int end = min(me, v + nxo - ix);
+                double P0 = 0.0, P1 = 0.0, P2 = 0.0, P3 = 0.0;
+                const double2 *xp = reinterpret_cast<const double2 *>(wxp + XW * ix + 4);
+#pragma unroll 4
+                for (; v < end; v++, xp += XW / 2) {
+                    const double2 n = *xp;
+                    const double x = n.x - cx, p0 = n.y * sp[v], p1 = p0 * x, p2 = p1 * x;
+                    P0 += p0;
+                    P1 += p1;
+                    P2 += p2;
+                    P3 = fma(p2, x, P3);
+                }
+                const double *e = lw + l * LW + 9;
+                const double y = e[0] - cy, z2 = e[1] - cz, W = e[2], r = fma(y, y, z2 * z2);
+                const double q0 = W * P0, q1 = W * P1, q2 = W * P2, y0 = y * q0, z0q = z2 * q0, e2 = fma(r, q0, q2);
+                S[P_S0] += q0;
+                S[P_S1X] += q1;
+                S[P_S1Y] += y0;
+                S[P_S1Z] += z0q;
+                S[P_S2XX] += q2;
+                S[P_S2YY] = fma(y, y0, S[P_S2YY]);
+                S[P_S2ZZ] = fma(z2, z0q, S[P_S2ZZ]);
+                S[P_S2XY] = fma(y, q1, S[P_S2XY]);
+                S[P_S2XZ] = fma(z2, q1, S[P_S2XZ]);
+                S[P_S2YZ] = fma(z2, y0, S[P_S2YZ]);
+                S[P_S3X] = fma(r, q1, fma(W, P3, S[P_S3X]));
+                S[P_S3Y] = fma(y, e2, S[P_S3Y]);
+                S[P_S3Z] = fma(z2, e2, S[P_S3Z]);
+                ix = 0;
+                l++;
+            }
         }
         // combine the two halves; the incoming flux towards the wall ahead is
-        // the octant's first moment along the axis up to sign
+        // the octant's first moment along the axis (about 0) up to sign
         if (mvp == 1) {
 #pragma unroll
             for (int q = 0; q < P_FX; q++) red[q * SLICE + mcl] = S[q];
@@ -455,9 +573,14 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
             double out[NPART];
 #pragma unroll
             for (int q = 0; q < P_FX; q++) out[q] = S[q];
-            out[P_FX] = live && (flags & (F_WALL_SIDE << headx)) ? (px ? S[P_S1X] : -S[P_S1X]) : 0.0;
-            out[P_FY] = live && (flags & (F_WALL_SIDE << heady)) ? (py ? S[P_S1Y] : -S[P_S1Y]) : 0.0;
-            out[P_FZ] = live && (flags & (F_WALL_SIDE << headz)) ? (pz ? S[P_S1Z] : -S[P_S1Z]) : 0.0;
+            auto flux = [&](int side, bool up, int d, double s1) {
+                if (!live || !(flags & (F_WALL_SIDE << side))) return 0.0;
+                const double f = fma(shared_centre ? cen[d] : -0.5 * m2u[d], S[P_S0], s1);
+                return up ? f : -f;
+            };
+            out[P_FX] = flux(headx, px, 0, S[P_S1X]);
+            out[P_FY] = flux(heady, py, 1, S[P_S1Y]);
+            out[P_FZ] = flux(headz, pz, 2, S[P_S1Z]);
             double2 *pp = reinterpret_cast<double2 *>(scratch + ((size_t)lk * SLICE + mcl) * NPART);
 #pragma unroll
             for (int q = 0; q < NPART; q += 2) pp[q / 2] = make_double2(out[q], out[q + 1]);
@@ -518,6 +641,13 @@ cudaError_t launch_axis_tables(const void *coef, const double *nodes, unsigned l
     const size_t n = (size_t)ncell * na;
     axis_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(static_cast<const double *>(coef), nodes, ncell, nvx, nvy,
                                                             na, static_cast<double4 *>(tab));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_slice_centres(const void *coef, int nx, int ny, int nz, double *centre, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((nx + BX - 1) / BX) * ((ny + BY - 1) / BY) * nz;
+    centre_kernel<<<nb, SLICE, 0, s>>>(static_cast<const double *>(coef), nx, ny, centre);
     return cudaGetLastError();
 }
 
