@@ -37,6 +37,7 @@ struct kgs_batch {
     int4 *d_items = nullptr;
     size_t items_cap = 0;
     int n_items = 0;
+    std::vector<char> items_active;     // the instances that the work list holds
     int *d_counter = nullptr, *d_flags = nullptr, *d_flag_off = nullptr, *d_error = nullptr;
     size_t n_flags = 0;
     int *d_pos = nullptr;               // place of each item in its accumulator chain
@@ -93,6 +94,7 @@ int build_items(kgs_batch *b)
     for (int s = 0; s < max_stage; s++)
         for (int i = 0; i < b->n; i++)
             if (b->active[i]) ctx_stage_items(b->ctx[i]->t, i, s, items);
+    b->items_active = b->active;
     b->n_items = (int)items.size();
     if (items.size() > b->items_cap) {
         if (b->d_items) cudaFree(b->d_items);
@@ -170,7 +172,7 @@ int rebuild(kgs_batch *b)
 {
     int rc;
     destroy_graphs(b);
-    if ((rc = build_items(b))) return rc;
+    if (b->items_active != b->active && (rc = build_items(b))) return rc;
     for (int which = 0; which < 2; which++) {
         if ((rc = upload_args(b, which))) return rc;
         cudaGraph_t g = nullptr;
@@ -365,36 +367,28 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
         cudaMemset(b->d_resid, 0, (2 * n + 1) * sizeof(double)) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess)
         return fail(KGS_ECUDA);
+    // the work list of all instances: a later one is no longer
+    if (int rc = build_items(b)) return fail(rc);
     // persistent grid: as many CTAs as fit on the device at once
-    int sms = 0, per_sm = 0;
+    int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess) return fail(KGS_ECUDA);
-    if (b->precision == KGS_FP64) {
-        // one kernel serves every instance: the separated sweep if all of
-        // them have their axis factors
-        SweepKind k = b->kind;
-        k.sep = 1;
-        bool all = sweep_persistent_occupancy(k, sweep_smem_bytes(k, b->nxo_max)) >= 1;
-        for (int i = 0; i < n && all; i++) {
-            const int rc = ctx_alloc_axis(b->ctx[i]);
-            if (rc) return fail(rc);
-            all = b->ctx[i]->ax_tab != nullptr;
-        }
-        for (int i = 0; i < n && !all; i++) ctx_free_axis(b->ctx[i]);
-        b->kind.sep = all;
+    const SweepPerSm per_sm = sweep_per_sm(b->kind, b->nxo_max);
+    const int most = std::max(per_sm.general, per_sm.sep);
+    if (most < 1) return fail(KGS_ECUDA);
+    b->scratch_stride = sweep_scratch_bytes(b->bz);
+    if (cudaMalloc(&b->d_scratch, (size_t)sms * most * b->scratch_stride) != cudaSuccess) return fail(KGS_ENOMEM);
+    // One kernel serves every instance: the separated FP64 sweep if all of
+    // them have their axis factors.  They come last, so that a batch that
+    // fits only without them still runs.
+    b->kind.sep = per_sm.sep > 0;
+    for (int i = 0; i < n && b->kind.sep; i++) {
+        const int rc = ctx_alloc_axis(b->ctx[i]);
+        if (rc) return fail(rc);
+        if (!b->ctx[i]->ax_tab) b->kind.sep = 0;
     }
-    for (;;) {
-        per_sm = sweep_persistent_occupancy(b->kind, sweep_smem_bytes(b->kind, b->nxo_max));
-        if (per_sm < 1) return fail(KGS_ECUDA);
-        b->grid = sms * per_sm;
-        b->scratch_stride = sweep_scratch_bytes(b->bz);
-        if (cudaMalloc(&b->d_scratch, (size_t)b->grid * b->scratch_stride) == cudaSuccess) break;
-        b->d_scratch = nullptr;
-        if (!b->kind.sep) return fail(KGS_ENOMEM);
-        // the batch fits only without the axis factors
-        (void)cudaGetLastError();
-        for (int i = 0; i < n; i++) ctx_free_axis(b->ctx[i]);
-        b->kind.sep = 0;
-    }
+    for (int i = 0; i < n && !b->kind.sep; i++) ctx_free_axis(b->ctx[i]);
+    b->grid = sms * (b->kind.sep ? per_sm.sep : per_sm.general);
+    if (b->grid < 1) return fail(KGS_ENOMEM);
     *out = b;
     return KGS_OK;
 }

@@ -26,7 +26,6 @@ struct kgs_ctx {
     double *mac = nullptr, *mac_new = nullptr, *rho_w = nullptr, *rho_w_new = nullptr;
     void *coef = nullptr, *vel = nullptr, *velm = nullptr, *mtab = nullptr, *FX = nullptr, *FY = nullptr,
          *FZ = nullptr;
-    bool allow_sep = true;                                // may use the separated FP64 sweep
     void *ax_tab = nullptr;                               // separated FP64 sweep: axis factors (null: not used)
     double *ax_nodes = nullptr;                           // HostTables::ax_nodes
     double *centre = nullptr;                             // SweepArgs::centre

@@ -227,6 +227,12 @@ cudaError_t launch_sweep_persistent(const SweepKind &k, const BatchSweepArgs &b,
 // Resident CTAs per SM of the persistent kernel (also sets its shared-memory limit).
 int sweep_persistent_occupancy(const SweepKind &k, size_t smem);
 size_t sweep_smem_bytes(const SweepKind &k, int nxo_max);
+// The two of them for the kernel that needs no axis factors and for the
+// separated one (0 where it does not apply or its tables do not fit).
+struct SweepPerSm {
+    int general, sep;
+};
+SweepPerSm sweep_per_sm(SweepKind k, int nxo_max);
 // Sweep launch (one wavefront stage, order 1, no deviation-form source).
 cudaError_t launch_sweep(const SweepKind &k, const SweepArgs &a, int n_items, int max_vg, cudaStream_t s);
 

@@ -343,18 +343,13 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     const HostTables &t = c->t;
     int sms = 0;
     KGS_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
-    if (t.precision == KGS_FP64 && t.order == 1 && c->allow_sep) {
-        SweepKind k = t.kind();
-        k.sep = 1;
-        int rc;
-        if (sweep_persistent_occupancy(k, sweep_smem_bytes(k, t.nxo_max)) >= 1 && (rc = ctx_alloc_axis(c))) return rc;
-    }
-    const SweepKind kind = ctx_kind(c);
-    const int per_sm = sweep_persistent_occupancy(kind, sweep_smem_bytes(kind, t.nxo_max));
+    // CTAs per SM without and with the axis factors of the separated FP64 sweep
+    const SweepPerSm per_sm = sweep_per_sm(t.kind(), t.nxo_max);
+    const int most = std::max(per_sm.general, per_sm.sep);
     // the second-order sweep and the deviation-form source exist only in the
     // persistent kernel
-    if (per_sm < 1 && (t.order == 2 || t.dev)) return KGS_EINVAL;
-    if (per_sm < 1) {
+    if (most < 1 && (t.order == 2 || t.dev)) return KGS_EINVAL;
+    if (most < 1) {
         // the launch per stage, with per-group partials
         return dalloc(c, &c->part, (size_t)t.n_vg * NPART * t.ncell * 8);
     }
@@ -364,13 +359,17 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     chain_positions(items, std::vector<const HostTables *>(1, &t), pos);
     int rc;
     c->p_n_flags = (size_t)t.n_vg * t.nbx * t.nby * t.nbz;
-    c->persist_grid = sms * per_sm;
     c->scratch_stride = sweep_scratch_bytes(t.bz);
     if ((rc = upload(c, &c->p_items, items)) || (rc = upload(c, &c->p_pos, pos)) ||
         (rc = dalloc_t(c, &c->p_counter, 1 + c->p_n_flags + ctx_n_tokens(t))) ||
         (rc = upload(c, &c->p_flag_off, std::vector<int>(1, 0))) || (rc = dalloc_t(c, &c->p_args, 2)) ||
-        (rc = dalloc(c, &c->p_scratch, (size_t)c->persist_grid * c->scratch_stride)) || (rc = ctx_alloc_acc(c)))
+        (rc = dalloc(c, &c->p_scratch, (size_t)sms * most * c->scratch_stride)) || (rc = ctx_alloc_acc(c)))
         return rc;
+    // the axis factors come last: everything else is there, so that a problem
+    // that fits only without them still runs
+    if (per_sm.sep > 0 && (rc = ctx_alloc_axis(c))) return rc;
+    c->persist_grid = sms * (c->ax_tab ? per_sm.sep : per_sm.general);
+    if (c->persist_grid < 1) return KGS_ENOMEM;
     c->p_flags = c->p_counter + 1;
     c->p_tok = c->p_flags + c->p_n_flags;
     // the sweep's arguments, once for each of the two state buffers that the
@@ -547,17 +546,8 @@ int kgs_setup(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, const k
                               opts->block_z, opts->vz_begin, opts->vz_end, opts->order, opts->dev_source);
     if (rc) return rc;
     (void)cudaGetLastError();  // launches below check their own status
-    // a problem that fits only without the FP64 sweep's axis factors gets the
-    // sweep that needs none
-    for (int attempt = 0; attempt < 2; attempt++) {
-        if ((rc = ctx_create(out, grid, solid, vg, gas, bc, opts))) return rc;
-        (*out)->allow_sep = attempt == 0;
-        rc = ctx_persist_init(*out);
-        if (rc != KGS_ENOMEM || !(*out)->ax_tab) break;
-        kgs_destroy(*out);
-        *out = nullptr;
-        (void)cudaGetLastError();
-    }
+    if ((rc = ctx_create(out, grid, solid, vg, gas, bc, opts))) return rc;
+    rc = ctx_persist_init(*out);
     // the persistent sweep's tables and the accumulator fill went to the
     // legacy default stream as well
     if (!rc && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) rc = KGS_ECUDA;

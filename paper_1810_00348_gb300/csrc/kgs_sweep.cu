@@ -1133,6 +1133,18 @@ size_t sweep_smem_bytes(const SweepKind &k, int nxo_max)
     return k.tv == 2 ? SmemLayout<float, 2>::total(nxo_max, false) : SmemLayout<float, 1>::total(nxo_max, line);
 }
 
+SweepPerSm sweep_per_sm(SweepKind k, int nxo_max)
+{
+    SweepPerSm n{};
+    k.sep = 0;
+    n.general = sweep_persistent_occupancy(k, sweep_smem_bytes(k, nxo_max));
+    if (k.precision == 0 && k.order == 1) {
+        k.sep = 1;
+        n.sep = sweep_persistent_occupancy(k, sweep_smem_bytes(k, nxo_max));
+    }
+    return n;
+}
+
 cudaError_t launch_sweep(const SweepKind &k, const SweepArgs &a, int n_items, int max_vg, cudaStream_t s)
 {
     if (n_items == 0 || max_vg == 0) return cudaSuccess;

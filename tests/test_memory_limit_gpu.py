@@ -1,0 +1,92 @@
+"""Problems that fit the device only without the tables that make a sweep
+faster: they are set up, tuned and run all the same.  The rest of the device
+is held by a tensor meanwhile, which touches no memory.
+"""
+import contextlib
+
+import numpy as np
+import pytest
+
+from paper_1810_00348_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kgs():
+    from paper_1810_00348_gb300 import kgs as k
+    k.load()
+    return k
+
+
+@contextlib.contextmanager
+def leave(nbytes):
+    """Leave about nbytes of device memory free."""
+    import torch
+
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    hog = torch.empty(free - int(nbytes), dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+
+
+MB = 1 << 20
+CELLS = [62, 64, 63]  # 256 MB of accumulators, 375 MB of axis factors with 16^3 velocities
+
+
+def sizes(kgs, p, **kw):
+    """Device bytes of a context with all its tables, and of the axis factors."""
+    c = kgs.kgs_setup(p, precision=kgs.KGS_FP64, **kw)
+    n = kgs.kgs_info(c)["device_bytes"]
+    kgs.kgs_destroy(c)
+    return n, p.ncell * (len(p.xi_x) + len(p.xi_y) + len(p.xi_z)) * 32
+
+
+def test_fp64_without_room_for_axis_factors(kgs):
+    p = inputs.cavity(CELLS, 16, Kn=0.5)
+    full, factors = sizes(kgs, p)
+    assert factors > 300 * MB
+    ref = kgs.kgs_setup(p, precision=kgs.KGS_FP64)
+    assert kgs.kgs_iterate(ref, 1)[0] == kgs.KGS_OK
+    want = kgs.kgs_moments(ref).copy()
+    kgs.kgs_destroy(ref)
+    with leave(full - 100 * MB):  # the factors fit, or what they leave no room for
+        c = kgs.kgs_setup(p, precision=kgs.KGS_FP64)
+        assert kgs.kgs_info(c)["device_bytes"] < full - 200 * MB
+        assert kgs.kgs_iterate(c, 1)[0] == kgs.KGS_OK
+        got = kgs.kgs_moments(c)
+        kgs.kgs_destroy(c)
+    assert np.max(np.abs(got - want)) <= 1e-12
+
+
+def test_autotune_and_batch_without_room_for_axis_factors(kgs):
+    p = inputs.cavity(CELLS, 16, Kn=0.4)
+    full, _ = sizes(kgs, p)
+    with leave(full - 100 * MB):
+        vpc, bz = kgs.kgs_autotune(p, precision=kgs.KGS_FP64)
+    assert vpc == 128 and bz in (8, 16, 32)
+    q = inputs.cavity(CELLS, 16, Kn=0.3)  # not tuned yet: the batch tunes it
+    with leave(full - 100 * MB):
+        b = kgs.kgs_batch_setup([q], precision=kgs.KGS_FP64)
+        rc, done, _ = kgs.kgs_batch_iterate(b, 1)
+        assert rc == kgs.KGS_OK and done == [1]
+        kgs.kgs_batch_destroy(b)
+
+
+def test_batch_takes_its_device_memory_at_set_up(kgs):
+    """The work list is there before the factors, not looked for at the first iteration."""
+    import torch
+
+    p = inputs.cavity([8, 8, 256], 24, Kn=0.5)
+    b = kgs.kgs_batch_setup([p] * 8, precision=kgs.KGS_FP64, v_per_cta=128, block_z=1)
+    before = torch.cuda.mem_get_info()[0]
+    assert kgs.kgs_batch_iterate(b, 1)[0] == kgs.KGS_OK
+    # 8 instances x 256 blocks x 112 groups, 20 bytes each: 4.6 MB, in two allocations of 2 MB pages
+    taken = before - torch.cuda.mem_get_info()[0]
+    kgs.kgs_batch_destroy(b)
+    assert taken < 4 * MB, taken
