@@ -41,7 +41,6 @@ struct kgs_batch {
     int *d_counter = nullptr, *d_flags = nullptr, *d_flag_off = nullptr, *d_error = nullptr;
     size_t n_flags = 0;
     int *d_pos = nullptr;               // place of each item in its accumulator chain
-    size_t pos_cap = 0;
     int *d_tok = nullptr;               // chain tokens of all instances
     size_t n_tok = 0;
     std::vector<size_t> tok_off;        // first token of each instance
@@ -96,22 +95,10 @@ int build_items(kgs_batch *b)
             if (b->active[i]) ctx_stage_items(b->ctx[i]->t, i, s, items);
     b->items_active = b->active;
     b->n_items = (int)items.size();
-    if (items.size() > b->items_cap) {
-        if (b->d_items) cudaFree(b->d_items);
-        b->d_items = nullptr;
-        KGS_CHECK(cudaMalloc(&b->d_items, items.size() * sizeof(int4)));
-        b->items_cap = items.size();
-    }
     std::vector<const HostTables *> tabs(b->n);
     for (int i = 0; i < b->n; i++) tabs[i] = &b->ctx[i]->t;
     std::vector<int> pos;
     chain_positions(items, tabs, pos);
-    if (pos.size() > b->pos_cap) {
-        if (b->d_pos) cudaFree(b->d_pos);
-        b->d_pos = nullptr;
-        KGS_CHECK(cudaMalloc(&b->d_pos, pos.size() * sizeof(int)));
-        b->pos_cap = pos.size();
-    }
     if (!items.empty()) {
         KGS_CHECK(cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
         KGS_CHECK(cudaMemcpy(b->d_pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice));
@@ -336,7 +323,7 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
         o.v_per_cta = vpc;
         o.block_z = bz;
         int rc = ctx_create(&b->ctx[i], &p.grid, p.solid, &p.vgrid, &p.gas, &p.bc, &o);
-        if (rc || (rc = ctx_alloc_acc(b->ctx[i]))) return fail(rc);
+        if (rc) return fail(rc);
         const HostTables &t = b->ctx[i]->t;
         b->tok_off.push_back(b->n_tok);
         b->n_tok += ctx_n_tokens(t);
@@ -367,8 +354,6 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
         cudaMemset(b->d_resid, 0, (2 * n + 1) * sizeof(double)) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess)
         return fail(KGS_ECUDA);
-    // the work list of all instances: a later one is no longer
-    if (int rc = build_items(b)) return fail(rc);
     // persistent grid: as many CTAs as fit on the device at once
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess) return fail(KGS_ECUDA);
@@ -377,9 +362,16 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
     if (most < 1) return fail(KGS_ECUDA);
     b->scratch_stride = sweep_scratch_bytes(b->bz);
     if (cudaMalloc(&b->d_scratch, (size_t)sms * most * b->scratch_stride) != cudaSuccess) return fail(KGS_ENOMEM);
-    // One kernel serves every instance: the separated FP64 sweep if all of
-    // them have their axis factors.  They come last, so that a batch that
-    // fits only without them still runs.
+    // the room of the work list: that of all instances is the longest
+    for (const kgs_ctx *c : b->ctx) b->items_cap += (size_t)c->t.n_vg * c->t.nbx * c->t.nby * c->t.nbz;
+    if (cudaMalloc(&b->d_items, b->items_cap * sizeof(int4)) != cudaSuccess ||
+        cudaMalloc(&b->d_pos, b->items_cap * sizeof(int)) != cudaSuccess)
+        return fail(KGS_ENOMEM);
+    // What the batch can do without or with less of comes last, so that one
+    // that fits only without it still runs: the accumulators and, where one
+    // kernel can serve every instance, the axis factors of the separated FP64
+    // sweep for all of them.
+    if (int rc = ctx_alloc_acc(b->ctx.data(), n)) return fail(rc);
     b->kind.sep = per_sm.sep > 0;
     for (int i = 0; i < n && b->kind.sep; i++) {
         const int rc = ctx_alloc_axis(b->ctx[i]);
@@ -473,20 +465,25 @@ int kgs_batch_solve(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
             }
         }
     }
-    // FP64 phase from each mixed state (macros, wall densities, mass target)
+    // FP64 phase from each mixed state (macros, wall densities, mass target);
+    // the mixed batch gives its memory back first
+    std::vector<std::vector<unsigned char>> state(n);
+    for (int i = 0; i < n; i++) {
+        size_t len = 0;
+        if ((rc = kgs_save(m->ctx[i], nullptr, &len))) return finish(rc);
+        state[i].resize(len);
+        if ((rc = kgs_save(m->ctx[i], state[i].data(), &len))) return finish(rc);
+    }
+    kgs_batch_destroy(m);
+    m = nullptr;
     kgs_opts od = *opts;
     od.precision = KGS_FP64;
     od.dev_source = 0;
     od.v_per_cta = 128;
     od.block_z = opts->block_z > 0 ? opts->block_z : 32;
     if ((rc = kgs_batch_setup(&d, n, probs, &od))) return finish(rc);
-    std::vector<unsigned char> state;
     for (int i = 0; i < n; i++) {
-        size_t len = 0;
-        if ((rc = kgs_save(m->ctx[i], nullptr, &len))) return finish(rc);
-        state.resize(len);
-        if ((rc = kgs_save(m->ctx[i], state.data(), &len)) || (rc = kgs_load(d->ctx[i], state.data(), len)))
-            return finish(rc);
+        if ((rc = kgs_load(d->ctx[i], state[i].data(), state[i].size()))) return finish(rc);
         // every instance with budget left runs at least one FP64 iteration
         // (it confirms the tolerance), at most max(1, budget - mixed iterations)
         d->active[i] = nm[i] < budget;

@@ -30,7 +30,7 @@ struct kgs_ctx {
     double *ax_nodes = nullptr;                           // HostTables::ax_nodes
     double *centre = nullptr;                             // SweepArgs::centre
     float *lines = nullptr, *xnodes = nullptr;            // packed FP32 sweep: HostTables::lines32, xnodes32
-    float *rho_w32 = nullptr;                             // packed FP32 sweep: rho_w in FP32
+    float *rho_w32 = nullptr;                             // packed FP32 sweep: rho_w in FP32 (in the room of sums)
     void *FX2 = nullptr, *FY2 = nullptr, *FZ2 = nullptr;  // second face planes of the order-2 sweep
     void *part = nullptr;   // staged sweep only: per-(group, cell) partials
     void *acc = nullptr;    // persistent sweep: ordered accumulators [nacc][ncell][acc_slots]
@@ -96,8 +96,9 @@ SweepKind ctx_kind(const kgs_ctx *c);
 // context keeps the sweep that needs none (ax_tab stays null).
 int ctx_alloc_axis(kgs_ctx *c);
 void ctx_free_axis(kgs_ctx *c);
-// Ordered accumulators of a context whose sweep runs persistent.
-int ctx_alloc_acc(kgs_ctx *c);
+// Ordered accumulators of n contexts whose sweep runs persistent:
+// HostTables::nacc each or, without the memory for that, nacc_least.
+int ctx_alloc_acc(kgs_ctx *const *c, int n);
 // Chain tokens per (accumulator, block) of one instance.
 inline size_t ctx_n_tokens(const HostTables &t) { return (size_t)t.nacc * t.nbx * t.nby * t.nbz; }
 // Place of every item of a stage-ordered work list in its accumulator chain

@@ -53,6 +53,16 @@ int dalloc(kgs_ctx *c, void **p, size_t bytes)
     return KGS_OK;
 }
 
+// Free an allocation of dalloc again (nothing for null).
+void dfree(kgs_ctx *c, void **p, size_t bytes)
+{
+    if (!*p) return;
+    c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), *p));
+    cudaFree(*p);
+    c->device_bytes -= bytes;
+    *p = nullptr;
+}
+
 template <typename T>
 int dalloc_t(kgs_ctx *c, T **p, size_t n)
 {
@@ -236,17 +246,9 @@ int kgs::ctx_alloc_axis(kgs_ctx *c)
 
 void kgs::ctx_free_axis(kgs_ctx *c)
 {
-    for (void *p : {static_cast<void *>(c->ax_nodes), static_cast<void *>(c->centre), c->ax_tab}) {
-        if (!p) continue;
-        c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
-        cudaFree(p);
-    }
-    if (c->ax_tab) c->device_bytes -= c->t.ncell * c->t.ax_nodes.size() * 4 * sizeof(double);
-    if (c->ax_nodes) c->device_bytes -= c->t.ax_nodes.size() * sizeof(double);
-    if (c->centre) c->device_bytes -= centre_values(c->t) * sizeof(double);
-    c->ax_tab = nullptr;
-    c->centre = nullptr;
-    c->ax_nodes = nullptr;
+    dfree(c, &c->ax_tab, c->t.ncell * c->t.ax_nodes.size() * 4 * sizeof(double));
+    dfree(c, reinterpret_cast<void **>(&c->ax_nodes), c->t.ax_nodes.size() * sizeof(double));
+    dfree(c, reinterpret_cast<void **>(&c->centre), centre_values(c->t) * sizeof(double));
 }
 
 int kgs::ctx_launch_stages(kgs_ctx *c)
@@ -324,17 +326,29 @@ void kgs::chain_positions(const std::vector<int4> &items, const std::vector<cons
     }
 }
 
-int kgs::ctx_alloc_acc(kgs_ctx *c)
+int kgs::ctx_alloc_acc(kgs_ctx *const *ctx, int n)
 {
-    const HostTables &t = c->t;
-    const size_t bytes = (size_t)t.nacc * t.ncell * t.acc_slots * 8;
-    int rc = dalloc(c, &c->acc, bytes);
-    if (rc) return rc;
-    // every slot read by the sums is stored by the first item of its chain in
-    // every iteration; all-ones bytes (NaN in both precisions) make any slot
-    // that is not show up in the results at once
-    KGS_CHECK(cudaMemset(c->acc, 0xff, bytes));
-    c->use_acc = 1;
+    for (int least = 0; least < 2; least++) {
+        int rc = KGS_OK;
+        for (int i = 0; i < n && !rc; i++) {
+            kgs_ctx *c = ctx[i];
+            HostTables &t = c->t;
+            if (least) t.nacc = t.nacc_least;
+            const size_t bytes = (size_t)t.nacc * t.ncell * t.acc_slots * 8;
+            if ((rc = dalloc(c, &c->acc, bytes))) break;
+            // every slot read by the sums is stored by the first item of its chain in
+            // every iteration; all-ones bytes (NaN in both precisions) make any slot
+            // that is not show up in the results at once
+            KGS_CHECK(cudaMemset(c->acc, 0xff, bytes));
+            c->use_acc = 1;
+        }
+        if (rc != KGS_ENOMEM || least) return rc;
+        (void)cudaGetLastError();
+        for (int i = 0; i < n; i++) {
+            const HostTables &t = ctx[i]->t;
+            dfree(ctx[i], reinterpret_cast<void **>(&ctx[i]->acc), (size_t)t.nacc * t.ncell * t.acc_slots * 8);
+        }
+    }
     return KGS_OK;
 }
 
@@ -355,18 +369,21 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     }
     std::vector<int4> items;
     for (int s = 0; s < (int)t.stage_n.size(); s++) ctx_stage_items(t, 0, s, items);
-    std::vector<int> pos;
-    chain_positions(items, std::vector<const HostTables *>(1, &t), pos);
     int rc;
     c->p_n_flags = (size_t)t.n_vg * t.nbx * t.nby * t.nbz;
     c->scratch_stride = sweep_scratch_bytes(t.bz);
-    if ((rc = upload(c, &c->p_items, items)) || (rc = upload(c, &c->p_pos, pos)) ||
+    if ((rc = upload(c, &c->p_items, items)) || (rc = dalloc_t(c, &c->p_pos, items.size())) ||
         (rc = dalloc_t(c, &c->p_counter, 1 + c->p_n_flags + ctx_n_tokens(t))) ||
         (rc = upload(c, &c->p_flag_off, std::vector<int>(1, 0))) || (rc = dalloc_t(c, &c->p_args, 2)) ||
-        (rc = dalloc(c, &c->p_scratch, (size_t)sms * most * c->scratch_stride)) || (rc = ctx_alloc_acc(c)))
+        (rc = dalloc(c, &c->p_scratch, (size_t)sms * most * c->scratch_stride)))
         return rc;
-    // the axis factors come last: everything else is there, so that a problem
-    // that fits only without them still runs
+    // what a sweep can do without or with less of comes last, so that a
+    // problem that fits only without it still runs: the accumulators, whose
+    // number the chain places depend on, and the axis factors
+    if ((rc = ctx_alloc_acc(&c, 1))) return rc;
+    std::vector<int> pos;
+    chain_positions(items, std::vector<const HostTables *>(1, &t), pos);
+    KGS_CHECK(cudaMemcpy(c->p_pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice));
     if (per_sm.sep > 0 && (rc = ctx_alloc_axis(c))) return rc;
     c->persist_grid = sms * (c->ax_tab ? per_sm.sep : per_sm.general);
     if (c->persist_grid < 1) return KGS_ENOMEM;
@@ -605,8 +622,12 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->red_count, 1)) ||
         (rc = dalloc_t(c, &c->resid, 3)))
         return fail(rc);
-    if (t.pack && ((rc = upload(c, &c->lines, t.lines32)) || (rc = upload(c, &c->xnodes, t.xnodes32)) || (rc = dalloc_t(c, &c->rho_w32, 6 * n))))
-        return fail(rc);
+    if (t.pack) {
+        if ((rc = upload(c, &c->lines, t.lines32)) || (rc = upload(c, &c->xnodes, t.xnodes32))) return fail(rc);
+        // written before the sweep and read by it; the sums are written after it
+        static_assert(NSUM * sizeof(double) >= 6 * sizeof(float), "the FP32 wall densities share the room of the sums");
+        c->rho_w32 = reinterpret_cast<float *>(c->sums);
+    }
     if (t.precision == KGS_FP64) {
         if ((rc = upload(c, reinterpret_cast<double **>(&c->velm), t.velm64))) return fail(rc);
     } else {

@@ -81,6 +81,8 @@ extern "C" int kgs_solve(const kgs_problem *p, const double *initial, double tol
     if ((rc = kgs_save(m, nullptr, &len))) return finish(rc);
     state.resize(len);
     if ((rc = kgs_save(m, state.data(), &len))) return finish(rc);
+    kgs_destroy(m);  // its memory may be needed for the FP64 context
+    m = nullptr;
     kgs_opts od = opts_for(p, KGS_FP64, tol, std::max(1, max_iters - n_mixed), stream);  // >= 1: confirms tol
     if ((rc = kgs_setup(&d, &p->grid, p->solid, &p->vgrid, &p->gas, &p->bc, &od))) return finish(rc);
     if ((rc = kgs_load(d, state.data(), len))) return finish(rc);

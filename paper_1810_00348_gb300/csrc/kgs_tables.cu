@@ -251,7 +251,13 @@ void build_tables(HostTables &t, const kgs_grid *grid, const uint8_t *solid, con
     // receives a group of every block.  Counting over all octants keeps the
     // chains of small velocity grids short: with one or two groups per octant
     // all eight octants would otherwise add one after the other.
+    // Where the memory for them is not there, the groups of one octant share
+    // them instead of all groups (128^3 cells x 4^3 velocities: 1 in 0.25 GB
+    // instead of 8 in 2.1 GB).
     t.nacc = std::max(1, std::min(NACC_MAX, t.n_vg));
+    t.nacc_least = t.nacc;
+    for (int o = 0; o < 8; o++)
+        if (t.oct_vcount[o] > 0) t.nacc_least = std::min(t.nacc_least, t.groups(o));
 
     // ---- wall tables: kinds 0..5 domain sides, 6 solid surfaces ----
     double wallU[7][3], wallT[7];

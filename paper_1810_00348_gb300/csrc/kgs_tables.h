@@ -42,6 +42,7 @@ struct HostTables {
     int xn_stride = 1;
     int n_vg = 0, max_vg = 0, nxo_max = 1;
     int nacc = 1;                            // ordered accumulators of the persistent sweep
+    int nacc_least = 1;                      // as many as the memory is needed for in any case
     int acc_slots = ACC_COMPACT;             // ACC_SPLIT if a cell has walls on both sides along an axis
     std::vector<int> vg_oct;                 // octant of each velocity group
     std::vector<double> vel64;               // [Nvs][4] xi_x, xi_y, xi_z, w

@@ -90,3 +90,44 @@ def test_batch_takes_its_device_memory_at_set_up(kgs):
     taken = before - torch.cuda.mem_get_info()[0]
     kgs.kgs_batch_destroy(b)
     assert taken < 4 * MB, taken
+
+
+def few_velocities():
+    # one velocity group per octant: all eight octants share one accumulator of 128 bytes per cell, or use eight
+    return inputs.cavity([96, 100, 92], 4, Kn=0.5)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_context_and_batch_with_room_for_one_accumulator(kgs, precision):
+    p = few_velocities()
+    c = kgs.kgs_setup(p, precision=precision)
+    full = kgs.kgs_info(c)["device_bytes"]
+    assert kgs.kgs_iterate(c, 2)[0] == kgs.KGS_OK
+    want = kgs.kgs_moments(c).copy()
+    kgs.kgs_destroy(c)
+    extra = 7 * 128 * p.ncell + (12 * 32 * p.ncell if precision == kgs.KGS_FP64 else 0)
+    with leave(full - extra + 200 * MB):
+        c = kgs.kgs_setup(p, precision=precision)
+        assert kgs.kgs_iterate(c, 2)[0] == kgs.KGS_OK
+        got = kgs.kgs_moments(c).copy()
+        kgs.kgs_destroy(c)
+        b = kgs.kgs_batch_setup([p], precision=precision, v_per_cta=0 if precision else 128, block_z=32)
+        assert kgs.kgs_batch_iterate(b, 2)[0] == kgs.KGS_OK
+        batch = kgs.kgs_batch_moments(b, 0).copy()
+        kgs.kgs_batch_destroy(b)
+    tol = 1e-12 if precision == kgs.KGS_FP64 else 1e-5
+    assert np.max(np.abs(got - want)) <= tol and np.max(np.abs(batch - want)) <= tol
+
+
+def test_solvers_hold_one_phase_at_a_time(kgs):
+    p = few_velocities()
+    c = kgs.kgs_setup(p, precision=kgs.KGS_FP64)
+    full = kgs.kgs_info(c)["device_bytes"]
+    kgs.kgs_destroy(c)
+    # room for the FP64 phase with one accumulator and no axis factors
+    with leave(full - (7 * 128 + 12 * 32) * p.ncell + 250 * MB):
+        rc, m, nm, nd, r = kgs.kgs_solve(p, tol=0.9, max_iters=50)
+        assert rc == kgs.KGS_OK and nd >= 1 and r < 0.9
+        rc, b, nm, nd, res = kgs.kgs_batch_solve([p], tol=0.9, max_iters=50, v_per_cta=256, block_z=32)
+        assert rc == kgs.KGS_OK and nd[0] >= 1 and res[0] < 0.9
+        kgs.kgs_batch_destroy(b)
