@@ -179,6 +179,18 @@ typedef struct {
     double last_residual;
 } kgs_info_t;
 
+/* Device memory.  A context holds about 450 (KGS_MIXED) or 530 (KGS_FP64) bytes
+ * per cell, 128 bytes per cell and accumulator (152 where a cell has walls on
+ * both sides along an axis; one accumulator per velocity group of an octant,
+ * at most 8), face planes of 4 or 8 bytes x velocities x (nx ny + ny nz + nx nz)
+ * and scratch of up to 2.5 MB x block_z.  It takes more where that makes the
+ * sweep faster, up to a third of what is free on the device at the time:
+ * accumulators up to 8 on small velocity grids, and, for KGS_FP64 at first
+ * order, axis factors of 32 (nvx + nvy + nvz) bytes per cell (64^3 cells x 32^3
+ * velocities: 0.8 GB), without which a sweep takes about 2.5 times as long.
+ * device_bytes of kgs_info tells what a context holds.  The results of the two
+ * FP64 sweeps agree to rounding, not bit for bit. */
+
 /* Build a context: copy the grids, mask and parameters to the device,
  * precompute per-velocity tables and start from the uniform state (the free
  * stream if any side is an inflow, else rho = 1, U = 0, T = 1, q = 0), with

@@ -372,15 +372,10 @@ int kgs_batch_setup(kgs_batch **out, int n, const kgs_problem *probs, const kgs_
     // kernel can serve every instance, the axis factors of the separated FP64
     // sweep for all of them.
     if (int rc = ctx_alloc_acc(b->ctx.data(), n)) return fail(rc);
-    b->kind.sep = per_sm.sep > 0;
-    for (int i = 0; i < n && b->kind.sep; i++) {
-        const int rc = ctx_alloc_axis(b->ctx[i]);
-        if (rc) return fail(rc);
-        if (!b->ctx[i]->ax_tab) b->kind.sep = 0;
-    }
-    for (int i = 0; i < n && !b->kind.sep; i++) ctx_free_axis(b->ctx[i]);
+    if (per_sm.sep > 0)
+        if (int rc = ctx_alloc_axis(b->ctx.data(), n, per_sm.general < 1)) return fail(rc);
+    b->kind.sep = b->ctx[0]->ax_tab != nullptr;
     b->grid = sms * (b->kind.sep ? per_sm.sep : per_sm.general);
-    if (b->grid < 1) return fail(KGS_ENOMEM);
     *out = b;
     return KGS_OK;
 }

@@ -92,12 +92,12 @@ void ctx_stage_items(const HostTables &t, int inst, int stage, std::vector<int4>
 int ctx_persist_init(kgs_ctx *c);
 // Kernel of a standalone context's sweep.
 SweepKind ctx_kind(const kgs_ctx *c);
-// Axis factors of the separated FP64 sweep; without the memory for them the
-// context keeps the sweep that needs none (ax_tab stays null).
-int ctx_alloc_axis(kgs_ctx *c);
-void ctx_free_axis(kgs_ctx *c);
+// Axis factors of the separated FP64 sweep, for all n contexts or for none
+// (ax_tab stays null): without the room for them (or they are required:
+// KGS_ENOMEM) the sweep that needs none serves them.
+int ctx_alloc_axis(kgs_ctx *const *c, int n, bool required);
 // Ordered accumulators of n contexts whose sweep runs persistent:
-// HostTables::nacc each or, without the memory for that, nacc_least.
+// HostTables::nacc each or, without the room for that, nacc_least.
 int ctx_alloc_acc(kgs_ctx *const *c, int n);
 // Chain tokens per (accumulator, block) of one instance.
 inline size_t ctx_n_tokens(const HostTables &t) { return (size_t)t.nacc * t.nbx * t.nby * t.nbz; }

@@ -229,26 +229,44 @@ SweepKind kgs::ctx_kind(const kgs_ctx *c)
 
 static size_t centre_values(const HostTables &t) { return (size_t)t.nbx * t.nby * t.nz * 4; }
 
-int kgs::ctx_alloc_axis(kgs_ctx *c)
+// Memory that only makes a sweep faster is taken up to a third of what is free
+// after the `needed` bytes that are still to come: the rest stays for other
+// contexts and for the caller.
+static bool room_for(size_t extra, size_t needed)
 {
-    const HostTables &t = c->t;
-    int rc = upload(c, &c->ax_nodes, t.ax_nodes);
-    if (!rc) rc = dalloc_t(c, &c->centre, centre_values(t));
-    if (!rc) rc = dalloc(c, &c->ax_tab, t.ncell * t.ax_nodes.size() * 4 * sizeof(double));
-    if (rc == KGS_ENOMEM) {
-        // the sweep that needs no axis factors serves a problem whose factors do not fit
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
         (void)cudaGetLastError();
-        ctx_free_axis(c);
-        rc = KGS_OK;
+        return false;
     }
-    return rc;
+    return needed <= free_bytes && extra <= (free_bytes - needed) / 3;
 }
 
-void kgs::ctx_free_axis(kgs_ctx *c)
+static size_t axis_bytes(const HostTables &t) { return t.ncell * t.ax_nodes.size() * 4 * sizeof(double); }
+
+static void ctx_free_axis(kgs_ctx *c)
 {
-    dfree(c, &c->ax_tab, c->t.ncell * c->t.ax_nodes.size() * 4 * sizeof(double));
+    dfree(c, &c->ax_tab, axis_bytes(c->t));
     dfree(c, reinterpret_cast<void **>(&c->ax_nodes), c->t.ax_nodes.size() * sizeof(double));
     dfree(c, reinterpret_cast<void **>(&c->centre), centre_values(c->t) * sizeof(double));
+}
+
+int kgs::ctx_alloc_axis(kgs_ctx *const *ctx, int n, bool required)
+{
+    size_t bytes = 0;
+    for (int i = 0; i < n; i++) bytes += axis_bytes(ctx[i]->t);
+    if (!required && !room_for(bytes, 0)) return KGS_OK;
+    int rc = KGS_OK;
+    for (int i = 0; i < n && !rc; i++) {
+        kgs_ctx *c = ctx[i];
+        rc = upload(c, &c->ax_nodes, c->t.ax_nodes);
+        if (!rc) rc = dalloc_t(c, &c->centre, centre_values(c->t));
+        if (!rc) rc = dalloc(c, &c->ax_tab, axis_bytes(c->t));
+    }
+    if (!rc) return rc;
+    (void)cudaGetLastError();
+    for (int i = 0; i < n; i++) ctx_free_axis(ctx[i]);
+    return rc == KGS_ENOMEM && !required ? KGS_OK : rc;
 }
 
 int kgs::ctx_launch_stages(kgs_ctx *c)
@@ -328,7 +346,14 @@ void kgs::chain_positions(const std::vector<int4> &items, const std::vector<cons
 
 int kgs::ctx_alloc_acc(kgs_ctx *const *ctx, int n)
 {
-    for (int least = 0; least < 2; least++) {
+    size_t needed = 0, extra = 0;
+    for (int i = 0; i < n; i++) {
+        const HostTables &t = ctx[i]->t;
+        const size_t one = t.ncell * t.acc_slots * 8;
+        needed += t.nacc_least * one;
+        extra += (t.nacc - t.nacc_least) * one;
+    }
+    for (int least = extra > 0 && !room_for(extra, needed); least < 2; least++) {
         int rc = KGS_OK;
         for (int i = 0; i < n && !rc; i++) {
             kgs_ctx *c = ctx[i];
@@ -384,9 +409,8 @@ int kgs::ctx_persist_init(kgs_ctx *c)
     std::vector<int> pos;
     chain_positions(items, std::vector<const HostTables *>(1, &t), pos);
     KGS_CHECK(cudaMemcpy(c->p_pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice));
-    if (per_sm.sep > 0 && (rc = ctx_alloc_axis(c))) return rc;
+    if (per_sm.sep > 0 && (rc = ctx_alloc_axis(&c, 1, per_sm.general < 1))) return rc;
     c->persist_grid = sms * (c->ax_tab ? per_sm.sep : per_sm.general);
-    if (c->persist_grid < 1) return KGS_ENOMEM;
     c->p_flags = c->p_counter + 1;
     c->p_tok = c->p_flags + c->p_n_flags;
     // the sweep's arguments, once for each of the two state buffers that the

@@ -131,3 +131,27 @@ def test_solvers_hold_one_phase_at_a_time(kgs):
         rc, b, nm, nd, res = kgs.kgs_batch_solve([p], tol=0.9, max_iters=50, v_per_cta=256, block_z=32)
         assert rc == kgs.KGS_OK and nd[0] >= 1 and res[0] < 0.9
         kgs.kgs_batch_destroy(b)
+
+
+def test_tables_for_speed_take_a_third_of_free_memory_at_most(kgs):
+    p = inputs.cavity(CELLS, 16, Kn=0.5)
+    full, factors = sizes(kgs, p)
+    held = {}
+    for more in (0.5, 1.5, 2.5, 4.0):  # left free beside the context, in factors
+        with leave(full + more * factors):
+            c = kgs.kgs_setup(p, precision=kgs.KGS_FP64)
+            held[more] = kgs.kgs_info(c)["device_bytes"]
+            kgs.kgs_destroy(c)
+            b = kgs.kgs_batch_setup([p], precision=kgs.KGS_FP64, v_per_cta=128, block_z=32)
+            assert kgs.kgs_batch_info(b, 0)["device_bytes"] >= factors or more < 2.0
+            kgs.kgs_batch_destroy(b)
+    assert held[2.5] == held[4.0] == full
+    assert held[0.5] == held[1.5] <= full - factors
+    q = few_velocities()
+    c = kgs.kgs_setup(q, precision=kgs.KGS_MIXED)
+    full = kgs.kgs_info(c)["device_bytes"]
+    kgs.kgs_destroy(c)
+    with leave(full + 1.5 * 7 * 128 * q.ncell):
+        c = kgs.kgs_setup(q, precision=kgs.KGS_MIXED)
+        assert kgs.kgs_info(c)["device_bytes"] == full - 7 * 128 * q.ncell
+        kgs.kgs_destroy(c)
