@@ -417,9 +417,11 @@ __device__ __forceinline__ void persistent_loop(const BatchSweepArgs &b, Item it
             }
             pipe.go = ok;
             if (ok) pipe.wait(1);
+            s_go = pipe.go;
         }
         __syncthreads();
-        if (!pipe.go) break;
+        // not pipe.go: thread 0 may be in the item already and clear it there
+        if (!s_go) break;
         void *scratch = static_cast<unsigned char *>(b.scratch) + (size_t)blockIdx.x * b.scratch_stride;
         item_sweep(sa, make_int4(o, bxr, byr, bzr), vg, scratch, pipe);
         __syncthreads();
