@@ -185,6 +185,14 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity)
     return __all_sync(0xffffffffu, mbar_wait(bar, parity));
 }
 
+// The same for warps that also give up once another has (*fail, written while
+// they run).  The flag goes into the vote: lanes that read different values
+// must not part before a vote of all of them.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const volatile int *fail)
+{
+    return __all_sync(0xffffffffu, *fail == 0 && mbar_wait(bar, parity));
+}
+
 // Warp index as a value that the compiler knows to be uniform.
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0); }
 
@@ -402,7 +410,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (long long u = u0; u < u1 && ok; u++) {
             for (int p = fresh(u) ? 0 : 2; p < 4; p++, n++) {
                 // plane n reuses the slot of plane n - HZ once no MMA reads it
-                if (n >= HZ && (*fail || !warp_wait(pempty(n - HZ), puse(n - HZ)))) {
+                if (n >= HZ && !warp_wait(pempty(n - HZ), puse(n - HZ), fail)) {
                     *fail = 1;  // the issuer's wait on this plane then gives up too
                     ok = false;
                     break;
@@ -431,7 +439,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // (output rows) while the MMAs of the next pair run
         const int quad = warp % 4, row = quad * 32 + lane;
         for (int j = 0; j < n_pairs; j++) {
-            if (*fail || !warp_wait(smem_u32(&acc_full[j & 1]), (uint32_t)(j / 2 & 1))) {
+            if (!warp_wait(smem_u32(&acc_full[j & 1]), (uint32_t)(j / 2 & 1), fail)) {
                 *fail = 1;
                 break;
             }
@@ -447,6 +455,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const size_t vo = (size_t)b * vol + ((size_t)z * dm.H + vy) * dm.W + vx;
                 for (int c0 = 0; c0 < cout_p; c0 += 16) {
                     float v[16];
+                    __syncwarp();  // lanes outside the volume skip the stores
                     tc_ld16(acc + (uint32_t)(oz * TMEM_HALF + c0), v);  // all lanes
                     if (!inside) continue;
                     if (MODE == 1) {
@@ -622,8 +631,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         const long long g_step = (long long)rows * dm.W * cp;
         for (int i = 0; i < nt; i++) {
             // tile i reuses the buffer of tile i - WG_BUF: its MMAs must have completed
-            if (i >= WG_BUF &&
-                (*fail || !warp_wait(smem_u32(&empty_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF - 1) & 1))) {
+            if (i >= WG_BUF && !warp_wait(smem_u32(&empty_bar[i % WG_BUF]), (uint32_t)(i / WG_BUF - 1) & 1, fail)) {
                 *fail = 1;
                 break;
             }
@@ -692,6 +700,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         for (int q = warp / 4; q < 3 * nb; q += 2) {
             const int kx = q / nb, c0 = q % nb * 16;
             float v[16];
+            __syncwarp();  // lanes without a channel skip the stores
             tc_ld16(tmem + ((uint32_t)((warp % 4) * 32) << 16) + (uint32_t)(kx * 128 + c0), v);
             if (co >= cout_p) continue;
             float *dst = part + ((((size_t)b * n_chunks + chunk) * 27 + (kz * 3 + ky) * 3 + kx) * cout_p + co) * cin_p + c0;
