@@ -492,6 +492,56 @@ __device__ __forceinline__ void close_solid(const ClosureArgs &a, size_t c)
     for (int s = 0; s < 6; s++) a.rho_w_new[s * a.ncell + c] = 0.0;
 }
 
+// Whether this block is the last one of its launch to come here; what the
+// others wrote before is then visible to every thread of it (through L2).
+__device__ __forceinline__ bool last_block(unsigned *count)
+{
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(count, 1u) == gridDim.x - 1;
+        if (last) *count = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return last != 0;
+}
+
+// Total of the closure blocks' masses, by all threads of a block into every one
+// of them: RED_THREADS strided sums, then a tree, whatever the block's size.
+__device__ __forceinline__ double total_mass(const double *blk_mass, int n)
+{
+    __shared__ double sh[RED_THREADS];
+    const int nt = blockDim.x;
+    for (int v = threadIdx.x; v < RED_THREADS; v += nt) {
+        double m = 0.0;
+#pragma unroll 8
+        for (int b = v; b < n; b += RED_THREADS) m += __ldcg(&blk_mass[b]);
+        sh[v] = m;
+    }
+    for (int k = RED_THREADS / 2; k > 0; k >>= 1) {
+        __syncthreads();
+        for (int v = threadIdx.x; v < k; v += nt) sh[v] += sh[v + k];
+    }
+    __syncthreads();
+    return sh[0];
+}
+
+// The total mass for the Section 3.4 rescale, which the residual kernel applies.
+// Up to MASS_DIRECT closure blocks every block of that kernel adds their masses
+// itself (8 loads per thread); beyond, where that work grows with the square
+// of the cells (256^3 cells with 32 per closure block: 70 ms), the last block
+// of the closure leaves the total, which adds 4 us to a small problem's
+// iteration (16^3 cells: 361 instead of 357 us).
+constexpr int MASS_DIRECT = 2048;
+__device__ __forceinline__ void leave_total_mass(const ClosureArgs &a)
+{
+    if (!a.rescale || gridDim.x <= MASS_DIRECT || !last_block(&a.state->closed)) return;
+    const double m = total_mass(a.blk_mass, gridDim.x);
+    if (threadIdx.x == 0) a.state->mass = m;
+}
+
 // Closure from sums in memory, one thread per cell (CLOSE_CELLS cells per
 // block); the block's cell masses are summed in a fixed order for the Section
 // 3.4 rescale.
@@ -511,6 +561,7 @@ __global__ void __launch_bounds__(CLOSE_CELLS) closure_kernel(const ClosureArgs 
     static_assert(CLOSE_CELLS == 32, "one warp per block's cells");
     for (int off = 16; off > 0; off >>= 1) mass += __shfl_down_sync(0xffffffffu, mass, off);
     if (threadIdx.x == 0) a.blk_mass[blockIdx.x] = mass;
+    leave_total_mass(a);
 }
 
 // Closure straight from the accumulators: the sums of a cell stay in the
@@ -540,32 +591,20 @@ __global__ void __launch_bounds__(ACC_CELLS) acc_close_kernel(const AccSumArgs a
     if (threadIdx.x % 32 == 0) wm[threadIdx.x / 32] = mass;
     __syncthreads();
     if (threadIdx.x == 0) k.blk_mass[blockIdx.x] = (wm[0] + wm[1]) + (wm[2] + wm[3]);
+    leave_total_mass(k);
 }
 
-// Total mass and the Section 3.4 rescale factor, the rescale, the divergence
-// check and the Section 4.1 residual in one launch.  Every block sums the
-// masses of all blocks of the closure itself (the same fixed order in each:
-// strided per-thread sums, then a tree); the last block to finish adds the
-// blocks' residual sums, again in a fixed order, and resets the counter.
+// The Section 3.4 rescale, the divergence check and the Section 4.1 residual in
+// one launch; the last block to finish adds the blocks' residual sums in a
+// fixed order.
 __global__ void __launch_bounds__(RED_THREADS) residual_kernel(const ResidualArgs a)
 {
     __shared__ double sh[10][RED_THREADS];
-    __shared__ int any_bad, last;
+    __shared__ int any_bad;
     const size_t ncell = a.ncell;
     const int t = threadIdx.x;
     double s = 1.0;
-    if (a.rescale) {
-        double M = 0.0;
-        for (int b = t; b < a.n_mass; b += RED_THREADS) M += a.blk_mass[b];
-        sh[0][t] = M;
-        __syncthreads();
-        for (int k = RED_THREADS / 2; k > 0; k >>= 1) {
-            if (t < k) sh[0][t] += sh[0][t + k];
-            __syncthreads();
-        }
-        s = a.M0 / sh[0][0];
-        __syncthreads();
-    }
+    if (a.rescale) s = a.M0 / (a.n_mass <= MASS_DIRECT ? total_mass(a.blk_mass, a.n_mass) : a.state->mass);
     if (t == 0) any_bad = 0;
     const size_t c = (size_t)blockIdx.x * RED_THREADS + t;
     double v[10];
@@ -617,14 +656,7 @@ __global__ void __launch_bounds__(RED_THREADS) residual_kernel(const ResidualArg
     if (t == 0) {
         a.blk_bad[blockIdx.x] = any_bad;
     }
-    __syncthreads();
-    if (t == 0) {
-        __threadfence();
-        last = atomicAdd(a.count, 1u) == gridDim.x - 1;
-        __threadfence();
-    }
-    __syncthreads();
-    if (!last) return;
+    if (!last_block(&a.state->checked)) return;
     for (int q = 0; q < 10; q++) v[q] = 0.0;
     bad = 0;
     for (int b = t; b < (int)gridDim.x; b += RED_THREADS) {
@@ -647,7 +679,6 @@ __global__ void __launch_bounds__(RED_THREADS) residual_kernel(const ResidualArg
     }
     a.out[0] = res;
     a.out[1] = any_bad ? 1.0 : 0.0;
-    *a.count = 0;
 }
 
 // rho_w^0 from the flux of f^{S,0} through each wall face (Eq. (9) with the

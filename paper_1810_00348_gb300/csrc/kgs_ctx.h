@@ -45,7 +45,7 @@ struct kgs_ctx {
     int *d_vstart = nullptr, *d_vcount = nullptr, *d_vgbase = nullptr, *d_vg_oct = nullptr;
     double *blk_mass = nullptr, *blk_res = nullptr, *resid = nullptr;
     int *blk_bad = nullptr;
-    unsigned *red_count = nullptr;   // blocks of the residual kernel that have finished (zero between launches)
+    kgs::CloseState *close_state = nullptr;
     double *h_resid = nullptr;  // pinned: residual, divergence flag, wait-error word
     // persistent sweep of a standalone context: one launch per iteration over
     // the work items in stage order; a CTA waits (bounded) for the three

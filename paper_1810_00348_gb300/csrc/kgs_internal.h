@@ -272,6 +272,12 @@ struct PartSumArgs {
     RefMoments ref;               // moments of the reference Maxwellian, added to every cell
 };
 
+// What the closure and the residual kernel of an iteration pass on; all zero
+// before the first iteration.
+struct CloseState {
+    unsigned closed, checked;     // blocks of either kernel that have finished (zero between launches)
+    double mass;                  // total mass, of a closure of many blocks
+};
 struct ClosureArgs {
     int nx, ny, nz;
     unsigned long long ncell;
@@ -286,6 +292,8 @@ struct ClosureArgs {
     const double *dx, *dy, *dz;
     const uint8_t *solid;         // [ncell] or NULL
     double *blk_mass;             // [close_blocks(ncell)]
+    int rescale;                  // the mass is wanted
+    CloseState *state;
 };
 
 // dev_src (FP32 only): the C_RDX / C_RDY slots carry the exponent terms of
@@ -327,13 +335,13 @@ struct ResidualArgs {
     const double *mac;            // step n
     const uint8_t *solid;         // [ncell] or NULL
     unsigned long long ncell;
-    const double *blk_mass;       // [n_mass] of the closure
-    int n_mass;
     double M0;
     int rescale;                  // 1: scale the total mass to M0
     double *blk_res;              // [blocks of 256 cells][10]
     int *blk_bad;                 // [blocks of 256 cells]
-    unsigned *count;              // zero before the first launch; left zero
+    const double *blk_mass;       // [n_mass] of the closure, if rescale
+    int n_mass;
+    CloseState *state;
     double *out;                  // residual, divergence flag
 };
 cudaError_t launch_residual(const ResidualArgs &a, cudaStream_t s);

@@ -124,7 +124,7 @@ int noalloc_iterate(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid 
                  o_xnodes = cv.take(t.pack ? t.xnodes32.size() * sizeof(float) : 0);
     const size_t o_solid = cv.take(t.any_solid ? n : 0);
     const size_t o_bmass = cv.take(close_blocks(n) * sizeof(double)), o_bres = cv.take((size_t)n_red * 10 * sizeof(double)),
-                 o_bbad = cv.take(n_red * sizeof(int)), o_count = cv.take(2 * sizeof(double)),
+                 o_bbad = cv.take(n_red * sizeof(int)), o_state = cv.take(sizeof(CloseState)),
                  o_resid = cv.take(2 * sizeof(double));
     if (cv.used > (size_t)KGS_NOALLOC_SCRATCH_BYTES) return TOO_LARGE;  // for the fixed array
 
@@ -251,6 +251,8 @@ int noalloc_iterate(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid 
     ca.dz = reinterpret_cast<const double *>(b + o_dz);
     ca.solid = d_solid;
     ca.blk_mass = reinterpret_cast<double *>(b + o_bmass);
+    ca.state = reinterpret_cast<CloseState *>(b + o_state);
+    ca.rescale = M0 > 0.0 ? 1 : 0;
     double *d_resid = reinterpret_cast<double *>(b + o_resid);
     ResidualArgs ra;
     ra.mac_new = macros_out;
@@ -258,16 +260,17 @@ int noalloc_iterate(const kgs_grid *grid, const uint8_t *solid, const kgs_vgrid 
     ra.mac = macros_in;
     ra.solid = d_solid;
     ra.ncell = n;
-    ra.blk_mass = ca.blk_mass;
-    ra.n_mass = (int)close_blocks(n);
     ra.M0 = M0;
     ra.rescale = M0 > 0.0 ? 1 : 0;
     ra.blk_res = reinterpret_cast<double *>(b + o_bres);
     ra.blk_bad = reinterpret_cast<int *>(b + o_bbad);
-    ra.count = reinterpret_cast<unsigned *>(b + o_count);
+    ra.blk_mass = ca.blk_mass;
+    ra.n_mass = (int)close_blocks(n);
+    ra.state = ca.state;
     ra.out = d_resid;
-    if (launch_part_sums(pa, st) != cudaSuccess || launch_closure(ca, st) != cudaSuccess ||
-        cudaMemsetAsync(ra.count, 0, sizeof(unsigned), st) != cudaSuccess || launch_residual(ra, st) != cudaSuccess)
+    if (cudaMemsetAsync(ca.state, 0, sizeof(CloseState), st) != cudaSuccess ||
+        launch_part_sums(pa, st) != cudaSuccess || launch_closure(ca, st) != cudaSuccess ||
+        launch_residual(ra, st) != cudaSuccess)
         return KGS_ECUDA;
     double h[2] = {0.0, 0.0};
     // pageable destination: returns once the values are on the host

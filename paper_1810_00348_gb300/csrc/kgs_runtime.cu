@@ -492,6 +492,8 @@ int kgs::ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums, b
     ca.dz = c->ddz;
     ca.solid = c->solid;
     ca.blk_mass = c->blk_mass;
+    ca.state = c->close_state;
+    ca.rescale = c->mass_rescale;
     if (from_acc)
         KGS_CHECK(launch_acc_close(acc_args(c), ca, st));
     else
@@ -502,13 +504,13 @@ int kgs::ctx_launch_closure(kgs_ctx *c, double *resid_dev, const double *sums, b
     ra.mac = c->mac;
     ra.solid = c->solid;
     ra.ncell = t.ncell;
-    ra.blk_mass = c->blk_mass;
-    ra.n_mass = from_acc ? (int)acc_close_blocks(t.ncell) : (int)close_blocks(t.ncell);
     ra.M0 = c->M0;
     ra.rescale = c->mass_rescale;
     ra.blk_res = c->blk_res;
     ra.blk_bad = c->blk_bad;
-    ra.count = c->red_count;
+    ra.blk_mass = c->blk_mass;
+    ra.n_mass = from_acc ? (int)acc_close_blocks(t.ncell) : (int)close_blocks(t.ncell);
+    ra.state = c->close_state;
     ra.out = resid_dev;
     KGS_CHECK(launch_residual(ra, st));
     c->kernel_launches += 2;
@@ -643,7 +645,7 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         (rc = upload(c, &c->d_vgbase, std::vector<int>(t.oct_vgbase, t.oct_vgbase + 8))) ||
         (rc = upload(c, &c->d_vg_oct, t.vg_oct)) || (rc = dalloc_t(c, &c->blk_mass, close_blocks(n))) ||
         (rc = dalloc_t(c, &c->blk_res, (size_t)c->n_red_blocks * 10)) ||
-        (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->red_count, 1)) ||
+        (rc = dalloc_t(c, &c->blk_bad, c->n_red_blocks)) || (rc = dalloc_t(c, &c->close_state, 1)) ||
         (rc = dalloc_t(c, &c->resid, 3)))
         return fail(rc);
     if (t.pack) {
@@ -674,7 +676,7 @@ int kgs::ctx_create(kgs_ctx **out, const kgs_grid *grid, const uint8_t *solid, c
         return fail(KGS_ECUDA);
     if (cudaMallocHost(&c->h_resid, 3 * sizeof(double)) != cudaSuccess) return fail(KGS_ENOMEM);
     if (cudaMemset(c->resid, 0, 3 * sizeof(double)) != cudaSuccess ||
-        cudaMemset(c->red_count, 0, sizeof(unsigned)) != cudaSuccess)
+        cudaMemset(c->close_state, 0, sizeof(CloseState)) != cudaSuccess)
         return fail(KGS_ECUDA);
     c->ev.resize(2 * t.stage_n.size());
     for (auto &e : c->ev)
