@@ -56,7 +56,7 @@ constexpr int LW = 12;           // of a line: W, Wy, Wz, Wyy, Wzz, Wyz, Wr, Wry
 // Largest distance of U^n from the centre of its slice, in thermal speeds of
 // the coldest cell: at 1/8 the sums are as exact as about U^n itself (heat
 // flux off by 1.0 to 1.1 times as much over random fields), at 0.45 1.8 times.
-constexpr double CENTRE_RANGE = 0.125;
+constexpr float CENTRE_RANGE = 0.125f;
 static_assert(BX * CS >= NPART * SLICE, "reduction buffer in the halo row");
 
 struct LayoutD {
@@ -106,35 +106,37 @@ __global__ void __launch_bounds__(256)
 
 // SweepArgs::centre: the middle of the range of U^n over the fluid cells of
 // each block's slice (0 without any), and whether U^n is too far from it
-// (CENTRE_RANGE) somewhere.
+// (CENTRE_RANGE) somewhere.  In FP32: any velocity near U^n will do, and the
+// FP64 pipe takes 3 us for the comparisons.
 __global__ void __launch_bounds__(SLICE)
     centre_kernel(const double *__restrict__ coef, int nx, int ny, double *__restrict__ centre)
 {
-    __shared__ double lo[4][2], hi[4][2];
+    __shared__ float lo[4][2], hi[4][2];
     const int nbx = (nx + BX - 1) / BX, nby = (ny + BY - 1) / BY;
     const int bx = blockIdx.x % nbx, by = blockIdx.x / nbx % nby, k = blockIdx.x / (nbx * nby);
     const int t = threadIdx.x, i = bx * BX + t % BX, j = by * BY + t / BX;
     const double *r = coef + ((size_t)i + (size_t)nx * (j + (size_t)ny * k)) * NCOEF;
     const bool fluid = i < nx && j < ny && !(flag_bits(r[C_FLAGS]) & F_SOLID);
     for (int d = 0; d < 4; d++) {  // U^n along the axes, 1/(RT)
-        const double v = fluid ? (d < 3 ? -0.5 * r[C_M2UX + d] : r[C_RT1]) : 0.0;
-        double a = fluid ? v : INFINITY, b = fluid ? v : -INFINITY;
+        const float v = fluid ? (d < 3 ? -0.5f * (float)r[C_M2UX + d] : (float)r[C_RT1]) : 0.f;
+        float a = fluid ? v : INFINITY, b = fluid ? v : -INFINITY;
         for (int off = 16; off > 0; off >>= 1) {
-            a = fmin(a, __shfl_xor_sync(0xffffffffu, a, off));
-            b = fmax(b, __shfl_xor_sync(0xffffffffu, b, off));
+            a = fminf(a, __shfl_xor_sync(0xffffffffu, a, off));
+            b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, off));
         }
         if (t % 32 == 0) lo[d][t / 32] = a, hi[d][t / 32] = b;
     }
     __syncthreads();
     if (t > 0) return;
-    double far2 = 0.0, *out = centre + (size_t)blockIdx.x * 4;
+    float far2 = 0.f;
+    double *out = centre + (size_t)blockIdx.x * 4;
     for (int d = 0; d < 3; d++) {
-        const double a = fmin(lo[d][0], lo[d][1]), h = 0.5 * (fmax(hi[d][0], hi[d][1]) - a);
-        out[d] = h >= 0.0 ? a + h : 0.0;
+        const float a = fminf(lo[d][0], lo[d][1]), h = 0.5f * (fmaxf(hi[d][0], hi[d][1]) - a);
+        out[d] = h >= 0.f ? a + h : 0.f;
         far2 += h * h;
     }
-    const double rt1 = fmax(hi[3][0], hi[3][1]);  // of the coldest cell, thermal speed^2 = 2 / rt1
-    out[3] = rt1 > 0.0 && !(far2 * rt1 <= 2.0 * CENTRE_RANGE * CENTRE_RANGE) ? 1.0 : 0.0;
+    const float rt1 = fmaxf(hi[3][0], hi[3][1]);  // of the coldest cell, thermal speed^2 = 2 / rt1
+    out[3] = rt1 > 0.f && !(far2 * rt1 <= 2.f * CENTRE_RANGE * CENTRE_RANGE) ? 1.0 : 0.0;
 }
 
 __device__ __forceinline__ double4 ld_rec(const double4 *p)
