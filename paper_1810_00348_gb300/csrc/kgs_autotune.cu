@@ -19,6 +19,12 @@ namespace {
 std::mutex g_tune_mutex;
 std::map<std::string, std::pair<int, int>> g_tune_cache;
 
+// Part of the key of every choice in a file: raised whenever the sweep kernels
+// or the rules that pick one change, so that a choice timed on other kernels
+// (a mixed problem sent to the general sweep by "128 velocities") is timed
+// anew.  1, without this mark: one kernel for every shape.
+constexpr int KERNEL_REVISION = 2;
+
 std::string shape_key(const kgs_problem *p, int precision)
 {
     bool any_solid = false;
@@ -27,8 +33,8 @@ std::string shape_key(const kgs_problem *p, int precision)
         for (long long i = 0; i < n && !any_solid; i++) any_solid = p->solid[i] != 0;
     }
     char buf[160];
-    std::snprintf(buf, sizeof buf, "p%d_c%dx%dx%d_v%dx%dx%d_s%d", precision, p->grid.nx, p->grid.ny, p->grid.nz,
-                  p->vgrid.nvx, p->vgrid.nvy, p->vgrid.nvz, any_solid ? 1 : 0);
+    std::snprintf(buf, sizeof buf, "r%d_p%d_c%dx%dx%d_v%dx%dx%d_s%d", KERNEL_REVISION, precision, p->grid.nx,
+                  p->grid.ny, p->grid.nz, p->vgrid.nvx, p->vgrid.nvy, p->vgrid.nvz, any_solid ? 1 : 0);
     return buf;
 }
 
