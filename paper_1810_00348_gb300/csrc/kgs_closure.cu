@@ -741,12 +741,6 @@ __global__ void __launch_bounds__(128) wall_flux_init_kernel(const double *mac, 
     if (lane == 0) rho_w[idx] = F * wall_norm[kind * 6 + s];
 }
 
-__global__ void fill_kernel(double *p, size_t n, double v)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
 inline unsigned nblk(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -816,12 +810,6 @@ cudaError_t launch_wall_flux_init(const double *mac, const int8_t *wall_kind, co
 {
     wall_flux_init_kernel<<<nblk(6 * ncell, 4), 128, 0, s>>>(mac, wall_kind, wall_norm, axis64, nvx, nvy, nvz, ncell, R,
                                                               Pr, rho_w);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fill(double *p, unsigned long long n, double v, cudaStream_t s)
-{
-    fill_kernel<<<nblk(n, 256), 256, 0, s>>>(p, n, v);
     return cudaGetLastError();
 }
 

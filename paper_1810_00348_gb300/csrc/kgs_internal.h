@@ -349,6 +349,5 @@ cudaError_t launch_wall_flux_init(const double *mac, const int8_t *wall_kind, co
                                   const double *axis64, int nvx, int nvy, int nvz, unsigned long long ncell, double R,
                                   double Pr,
                                   double *rho_w, cudaStream_t s);
-cudaError_t launch_fill(double *p, unsigned long long n, double v, cudaStream_t s);
 
 }  // namespace kgs

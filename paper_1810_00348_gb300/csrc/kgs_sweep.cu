@@ -1,9 +1,9 @@
 // kgs_sweep.cu -- the fused equilibrium + upwind implicit sweep + moment
 // kernel of one outer iteration (arXiv 1810.00348, Eqs. (2), (5), (7), (9)).
 // This is the general form: FP32 with one velocity per thread, the second
-// order, FP64 without axis factors, and FP32 with two velocities per thread
-// without packed slots.  kgs_sweep_f2.cu and kgs_sweep_d.cu serve the first
-// order in FP32 and FP64 otherwise.
+// order, FP64 without axis factors, and, with one launch per stage only, FP32
+// with two velocities per thread without packed slots.  kgs_sweep_f2.cu and
+// kgs_sweep_d.cu serve the first order in FP32 and FP64 otherwise.
 //
 // Work decomposition.  The physical grid is cut into blocks of BX x BY x bz
 // cells.  For the velocities of octant o (signs of xi_x, xi_y, xi_z) a block
@@ -1055,10 +1055,9 @@ int occupancy_t(size_t smem)
     return n;
 }
 
-// Instantiation chosen at run time.  The first-order FP64 sweep comes here
-// only without the memory for its axis factors (k.sep = 0), two velocities per
-// thread only without packed slots (HostTables::pack = 0): both with the
-// general moment loop alone.
+// Instantiation chosen at run time: one velocity per thread.  The first-order
+// FP64 sweep comes here only without the memory for its axis factors
+// (k.sep = 0), with the general moment loop alone.
 template <template <typename, int, int, bool, int, bool> class F, typename... Args>
 auto dispatch(const SweepKind &k, Args &&...args)
 {
@@ -1069,16 +1068,12 @@ auto dispatch(const SweepKind &k, Args &&...args)
         return k.line16 ? F<float, 1, 16, true, 2, true>::run(args...) : F<float, 1, 0, true, 2, true>::run(args...);
     }
     if (k.dev) {  // uniform grids
-        if (k.tv == 2) return F<float, 2, 0, true, 1, true>::run(args...);
         return k.line16 ? F<float, 1, 16, true, 1, true>::run(args...) : F<float, 1, 0, true, 1, true>::run(args...);
     }
     if (k.precision == 0) {
         return k.uniform ? F<double, 1, 0, true, 1, false>::run(args...)
                          : F<double, 1, 0, false, 1, false>::run(args...);
     }
-    if (k.tv == 2)
-        return k.uniform ? F<float, 2, 0, true, 1, false>::run(args...)
-                         : F<float, 2, 0, false, 1, false>::run(args...);
     if (k.line16)
         return k.uniform ? F<float, 1, 16, true, 1, false>::run(args...)
                          : F<float, 1, 16, false, 1, false>::run(args...);
@@ -1100,6 +1095,7 @@ struct Occupancy {
 
 bool exists(const SweepKind &k)
 {
+    if (k.tv == 2 && !k.pack) return false;  // two velocities per thread: with packed slots
     if (k.order == 2) return k.tv == 1 && k.uniform;
     return !k.dev || (k.precision != 0 && k.uniform);
 }
@@ -1130,7 +1126,7 @@ size_t sweep_smem_bytes(const SweepKind &k, int nxo_max)
         return k.precision == 0 ? SmemLayout<double, 1, 2>::total(nxo_max, line)
                                 : SmemLayout<float, 1, 2>::total(nxo_max, line);
     if (k.precision == 0) return SmemLayout<double, 1>::total(nxo_max, false);
-    return k.tv == 2 ? SmemLayout<float, 2>::total(nxo_max, false) : SmemLayout<float, 1>::total(nxo_max, line);
+    return SmemLayout<float, 1>::total(nxo_max, line);
 }
 
 SweepPerSm sweep_per_sm(SweepKind k, int nxo_max)
