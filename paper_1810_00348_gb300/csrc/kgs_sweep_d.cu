@@ -50,9 +50,11 @@ namespace {
 constexpr int VG = NT;           // velocities per group
 constexpr int CS = VG + 1;       // odd stride of a cell: conflict-free per-cell reads
 constexpr int HCOL = SLICE, HROW = SLICE + BY, NPOS = SLICE + BY + BX;
-constexpr int XW = 6;            // of an x node: w x^a (x about the slice's centre, a < 4), xi_x, w_x
-constexpr int LW = 12;           // of a line: W, Wy, Wz, Wyy, Wzz, Wyz, Wr, Wry, Wrz (r = y^2 + z^2; y and z about
-                                 // the slice's centre), xi_y, xi_z, W = w_y w_z
+// Weights of a line: W = w_y w_z, Wy, Wz, Wyy, Wzz, Wyz, Wr, Wry, Wrz (r = y^2 + z^2;
+// y and z about the slice's centre), xi_y.  These tables are as small as they
+// can be: with 10 nodes per line (20 along x) two blocks fit an SM with 64
+// bytes to spare, and one block alone takes 1.4 times as long.
+constexpr int LW = 10;
 // Largest distance of U^n from the centre of its slice, in thermal speeds of
 // the coldest cell: at 1/8 the sums are as exact as about U^n itself (heat
 // flux off by 1.0 to 1.1 times as much over random fields), at 0.45 1.8 times.
@@ -63,8 +65,9 @@ struct LayoutD {
     static constexpr size_t off_cell = align16(sizeof(double) * NPOS * CS);  // [SLICE][4] 1/tau, 1/dx, 1/dy, 1/dz
     static constexpr size_t off_flag = off_cell + sizeof(double) * SLICE * 4;
     static constexpr size_t off_cen = off_flag + sizeof(int) * SLICE;         // [2][4] centre of this and the next slice
-    static constexpr size_t off_x = off_cen + sizeof(double) * 8;             // [nxm][6] w_x (xi_x - C_x)^a, xi_x, w_x
-    __host__ __device__ static size_t off_line(int nxm) { return off_x + sizeof(double) * XW * nxm; }
+    static constexpr size_t off_x = off_cen + sizeof(double) * 8;             // [nxm][4] w_x (xi_x - C_x)^a
+    __host__ __device__ static size_t off_xi(int nxm) { return off_x + sizeof(double) * 4 * nxm; }  // [nxm] xi_x
+    __host__ __device__ static size_t off_line(int nxm) { return off_xi(nxm) + align16(sizeof(double) * nxm); }
     __host__ __device__ static size_t off_h(int nxm, int lines_max)           // [SLICE][lines_max][4]
     {
         return off_line(nxm) + align16(sizeof(double) * LW * lines_max);
@@ -155,6 +158,7 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
     int *cflag = reinterpret_cast<int *>(smem + LayoutD::off_flag);
     double *cen2 = reinterpret_cast<double *>(smem + LayoutD::off_cen);
     double *wxp = reinterpret_cast<double *>(smem + LayoutD::off_x);
+    double *xi_x = reinterpret_cast<double *>(smem + LayoutD::off_xi(a.nxo_max));
     double *lw = reinterpret_cast<double *>(smem + LayoutD::off_line(a.nxo_max));
     double *H = reinterpret_cast<double *>(smem + LayoutD::off_h(a.nxo_max, lines_max));
     double *red = slice + HROW * CS;  // [NPART][SLICE]: the halo row is not read during the moment phase
@@ -218,14 +222,14 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
     // nodes of the moment phase
     for (int ix = t; ix < nxo; ix += NT) {
         const size_t g = (size_t)a.oct_vstart[o] + ix;  // the octant's first line
-        wxp[ix * XW + 4] = vel[g * 4];
-        wxp[ix * XW + 5] = static_cast<const double *>(a.velm)[g * 8];
+        xi_x[ix] = vel[g * 4];
+        wxp[ix * 4] = static_cast<const double *>(a.velm)[g * 8];
     }
+    const double *line_xi = vel + ((size_t)a.oct_vstart[o] + (size_t)line0 * nxo) * 4;  // first node of the first line
     for (int l = t; l < nlines; l += NT) {
         const size_t g = (size_t)a.oct_vstart[o] + (size_t)(line0 + l) * nxo;
         lw[l * LW + 9] = vel[g * 4 + 1];
-        lw[l * LW + 10] = vel[g * 4 + 2];
-        lw[l * LW + 11] = static_cast<const double *>(a.velm)[g * 8 + 1];
+        lw[l * LW] = static_cast<const double *>(a.velm)[g * 8 + 1];
     }
     auto load_centre = [&](int lk) {
         if (t < 4) cen2[lk % 2 * 4 + t] = a.centre[slice_centre(GX(0), GY(0), GZ(lk), nx, ny) + t];
@@ -236,9 +240,8 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
         const int part = t / 32, lane = t % 32;
         if (part == 0) {
             for (int ix = lane; ix < nxo; ix += 32) {
-                double *e = wxp + ix * XW;
-                const double x = e[4] - cen[0], wx = e[5], x2 = x * x;
-                e[0] = wx;
+                double *e = wxp + ix * 4;
+                const double x = xi_x[ix] - cen[0], wx = e[0], x2 = x * x;
                 e[1] = wx * x;
                 e[2] = wx * x2;
                 e[3] = wx * x * x2;
@@ -247,9 +250,8 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
         }
         for (int l = lane; l < nlines; l += 32) {
             double *e = lw + l * LW;
-            const double y = e[9] - cen[1], z = e[10] - cen[2], W = e[11];
+            const double y = e[9] - cen[1], z = line_xi[(size_t)l * nxo * 4 + 2] - cen[2], W = e[0];
             if (part == 1) {
-                e[0] = W;
                 e[1] = W * y;
                 e[3] = W * y * y;
                 e[5] = W * y * z;
@@ -496,9 +498,9 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
                 // the part of line l in this half
                 const int end = min(me, v + nxo - ix);
                 double P0 = 0.0, P1 = 0.0, P2 = 0.0, P3 = 0.0;
-                const double2 *wp = reinterpret_cast<const double2 *>(wxp + XW * ix);
+                const double2 *wp = reinterpret_cast<const double2 *>(wxp) + 2 * ix;
 #pragma unroll 4
-                for (; v < end; v++, wp += XW / 2) {
+                for (; v < end; v++, wp += 2) {
                     const double f = sp[v];
                     const double2 w01 = wp[0], w23 = wp[1];
                     P0 = fma(w01.x, f, P0);
@@ -532,18 +534,16 @@ __device__ __forceinline__ void sweep_item_d(const SweepArgs &a, const int4 w, c
             while (v < me) {
                 const int end = min(me, v + nxo - ix);
                 double P0 = 0.0, P1 = 0.0, P2 = 0.0, P3 = 0.0;
-                const double2 *xp = reinterpret_cast<const double2 *>(wxp + XW * ix + 4);
 #pragma unroll 4
-                for (; v < end; v++, xp += XW / 2) {
-                    const double2 n = *xp;
-                    const double x = n.x - cx, p0 = n.y * sp[v], p1 = p0 * x, p2 = p1 * x;
+                for (; v < end; v++, ix++) {
+                    const double x = xi_x[ix] - cx, p0 = wxp[ix * 4] * sp[v], p1 = p0 * x, p2 = p1 * x;
                     P0 += p0;
                     P1 += p1;
                     P2 += p2;
                     P3 = fma(p2, x, P3);
                 }
-                const double *e = lw + l * LW + 9;
-                const double y = e[0] - cy, z2 = e[1] - cz, W = e[2], r = fma(y, y, z2 * z2);
+                const double y = lw[l * LW + 9] - cy, z2 = line_xi[(size_t)l * nxo * 4 + 2] - cz, W = lw[l * LW];
+                const double r = fma(y, y, z2 * z2);
                 const double q0 = W * P0, q1 = W * P1, q2 = W * P2, y0 = y * q0, z0q = z2 * q0, e2 = fma(r, q0, q2);
                 S[P_S0] += q0;
                 S[P_S1X] += q1;
