@@ -43,10 +43,15 @@ FLOPS_PER_PP = 68
 # h_d = f_1 + (f_1 - f_2)/3 (a subtraction and an FMA each) and the scaled
 # coefficients 3 a_d / 2.
 FLOPS_PER_PP_ORDER2 = FLOPS_PER_PP + 9 + 3
-# dram__bytes_read.sum + dram__bytes_write.sum of one sweep launch (ncu, 32^3
-# cells x 32^3 velocities, 256 velocities per CTA, blocks 8x8x32): 2.897e9 B
-# over 1.074e9 phase points
-TRAFFIC_BYTES_PER_PP = 2.897e9 / 1.074e9
+# FP64 operations per phase-point update that the first-order FP64 sweep
+# executes (ncu, 32^3 cells x 32^3 velocities: 17.9 instructions, 14.1 of them
+# fused).  Its separated form needs fewer than the method's count above, which
+# would give a fraction of the peak above 1.
+FLOPS_PER_PP_FP64 = 32
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the packed
+# sweep (ncu, 32^3 cells x 32^3 velocities, 256 velocities per CTA, blocks
+# 8x8x32): 2.88e9 B over 1.074e9 phase points
+TRAFFIC_BYTES_PER_PP = 2.88e9 / 1.074e9
 TRAFFIC_SHAPE = (256, 32)
 SM_COUNT = 152
 FP32_LANES_PER_SM = 128
@@ -274,7 +279,8 @@ def run_ours(args, world, rank, local):
         traffic = TRAFFIC_BYTES_PER_PP * pp
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak, "traffic": traffic,
-                "kernel": "sweep_persistent_kernel<float>", "flops_per_phase_point": FLOPS_PER_PP,
+                "kernel": "sweep2_persistent_kernel" if info["v_per_cta"] == 256 else "sweep_persistent_kernel<float>",
+                "flops_per_phase_point": FLOPS_PER_PP,
                 "peak_basis": "FP32 FMA lanes: %d SMs x %d lanes x 2 x %.0f MHz (derived)" % (
                     SM_COUNT, FP32_LANES_PER_SM, sm_mhz),
                 "sweep_ms_per_step": sweep_ms_iter, "sweep_share_of_step": sweep_ms_iter / ms_step}
@@ -305,11 +311,12 @@ def run_ours(args, world, rank, local):
         kgs.kgs_iterate(c64, 1)
         k64 = max(1, min(args.steps, 3))
         ms64, sw64, _, _ = timed(c64, k64)
-        a64 = FLOPS_PER_PP * pp / (sw64 / k64 / 1e3) / 1e12
+        a64 = FLOPS_PER_PP_FP64 * pp / (sw64 / k64 / 1e3) / 1e12
         fp64 = {"value": pp * k64 * world / (ms64 / 1e3), "unit": "phase-point updates/s", "steps": k64,
                 "ms_per_step": ms64 / k64,
                 "roofline": {"bound": "alu", "achieved": a64, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                             "frac": a64 / FP64_PEAK_TFLOPS, "peak_basis": "nominal dense FP64 1.25 TFLOP/s"}}
+                             "frac": a64 / FP64_PEAK_TFLOPS, "flops_per_phase_point": FLOPS_PER_PP_FP64,
+                             "kernel": "sweep_d_kernel", "peak_basis": "nominal dense FP64 1.25 TFLOP/s"}}
         del c64
         if rank == 0 and args.cells == N_CELL and args.vels == N_VEL:
             # mixed against FP64 at the full size after two iterations from the

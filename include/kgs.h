@@ -180,7 +180,7 @@ typedef struct {
 } kgs_info_t;
 
 /* Device memory.  A context holds about 450 (KGS_MIXED) or 530 (KGS_FP64) bytes
- * per cell, 128 bytes per cell and accumulator (152 where a cell has walls on
+ * per cell, 128 bytes per cell and accumulator (160 where a cell has walls on
  * both sides along an axis; one accumulator per velocity group of an octant,
  * at most 8), face planes of 4 or 8 bytes x velocities x (nx ny + ny nz + nx nz)
  * and scratch of up to 2.5 MB x block_z.  It takes more where that makes the

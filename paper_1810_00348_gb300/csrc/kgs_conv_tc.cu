@@ -521,10 +521,12 @@ __global__ void __launch_bounds__(THREADS, 1)
 // [y][ci/8][x][16 B]; the windows of that block at x offsets 0, 1, 2 are the
 // B operands of the three taps.
 //
-// What bounds it: the traffic from L2.  A tile brings 64 KB for 24 MMAs of 128
-// x 112 x 16 (1500 cycles of the tensor core), because tensor memory holds
-// three taps' accumulators and the nine (kz, ky) read the tiles again: 1.2 GB
-// for a 112 -> 112 layer on 8 x 32^3 voxels, 305 us or 3.9 TB/s.  Nine warps
+// What bounds it: the copies.  A tile brings 64 KB for 24 MMAs of 128 x 112 x
+// 16 (1500 cycles of the tensor core), because tensor memory holds three taps'
+// accumulators and the nine (kz, ky) read the tiles again: 0.8 GB through L2
+// for a 112 -> 112 layer on 4 x 32^3 voxels in 117 us, 52% of the L2's rate
+// with the tensor core 40% busy (288 CTAs are 1.9 waves of 152 SMs); 305 us on
+// 8 x 32^3.  Nine warps
 // only copy and one only issues MMAs, through barriers per tile buffer, so
 // neither waits for the other beyond the three buffers; a copying thread
 // keeps its (x, channel octet) from tile to tile and walks down the rows by

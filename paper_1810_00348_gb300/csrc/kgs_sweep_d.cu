@@ -37,11 +37,11 @@
 // Cells are visited row by row: with the pipe saturated by one chain there is
 // nothing to gain from independent cells.
 //
-// Measured: 32^3 cells x 32^3 velocities 87.2 -> 35.6 ms (30.7 ms are the 18
+// Measured: 32^3 cells x 32^3 velocities 87.2 -> 35.7 ms (30.7 ms are the 18
 // operations at the pipe's rate), 27x19x22 x 17x14x20 19.3 -> 4.0 ms (with the
 // overlap of neighbouring blocks).  Error of the heat flux against extended
-// precision as with every sum about U^n: 8.7e-16 (8.6e-16) around a cube at
-// Mach 2, 4.3e-14 (4.2e-14) in a Mach 2 stream, 1.3e-13 (1.6e-13) at Mach 5.
+// precision as with every sum about U^n: 8.4e-16 (8.6e-16) around a cube at
+// Mach 2, 4.1e-14 (4.2e-14) in a Mach 2 stream, 1.3e-13 (1.6e-13) at Mach 5.
 #include "kgs_sweep_dev.cuh"
 
 namespace kgs {

@@ -4,7 +4,7 @@
 // a thread block works through its item.
 //
 // What bounds it.  A block holds one slice of 256 velocities in shared memory
-// (about 100 KB), so two blocks of four warps share an SM and the kernel is
+// (83 KB, 87.5 KB with its tables), so two blocks of four warps share an SM and the kernel is
 // bound by the issue slots of two warps per scheduler and by the latency of
 // their dependent chains, not by a pipe or by memory.  The packed forms
 // (fma.rn.f32x2 and its kin: two FP32 results per lane and instruction, each
