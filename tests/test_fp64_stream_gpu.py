@@ -21,6 +21,8 @@ import pytest
 from oracle import Oracle
 from paper_1810_00348_gb300 import inputs
 from tests import brute
+from tests.parity import assert_fields_close, assert_rho_w_close
+from tests.test_sweep_forms_gpu import FORMS, problem
 
 pytestmark = pytest.mark.gpu
 
@@ -100,3 +102,22 @@ def test_heat_flux_of_a_stream(kgs, mach, amp, body):
     # T = 2/3 of the second moments per mass: the same chain
     errT = np.max(np.abs(got[4] - ref[1]))
     assert errT <= 2.0 * 60.0 * EPS * np.max(ref[1])
+
+
+# the sums about one velocity per slice (fields that vary little) and about
+# each cell's own (fields that vary much), over the axes, grids and masks that
+# the tables depend on; the tolerance is that of the FP64 parity tests
+@pytest.mark.parametrize("form", range(len(FORMS)))
+@pytest.mark.parametrize("amp", [0.01, 0.2])
+def test_both_sums_over_forms(kgs, form, amp):
+    p = problem(**FORMS[form])
+    mac = inputs.random_macros(p, 30 + form, amp)
+    o = Oracle(p, mac)
+    c = kgs.kgs_setup(p, precision=kgs.KGS_FP64, block_z=4)
+    kgs.kgs_set_initial(c, mac)
+    o.iterate(1)
+    assert kgs.kgs_iterate(c, 1)[0] == kgs.KGS_OK
+    assert_fields_close(kgs.kgs_moments(c), o.macros(), 1e-10, solid=p.solid, what=str(FORMS[form]))
+    # a wall that no velocity crosses has no wall density (0 / 0 in the oracle)
+    rw = o.rho_w()
+    assert_rho_w_close(np.where(np.isnan(rw), 0.0, kgs.kgs_rho_w(c)), np.nan_to_num(rw, nan=0.0), 1e-10)
